@@ -194,9 +194,9 @@ typedef struct {
   long long pieces;     /* final tetrahedra evaluated (profile mode)                     */
   long long fp64_evals; /* weight evaluations taken by the FP64 branch (mixed, profile)  */
   long long kernels;    /* kernel launches made by the plan's calls (always counted)     */
-  long long queue_overflow; /* static weights (profile): final tetrahedra that found their
-                               batch's queue of long-series pieces full and were evaluated
-                               in place by the carving warp instead                      */
+  long long queue_overflow; /* static weights (profile): final tetrahedra of the carving warp's
+                               queue of long-series pieces that were evaluated before their
+                               work unit's end because the queue was full                */
   long long box_pieces;     /* dynamic weights (profile): final tetrahedra whose principal-
                                value terms were gathered into a box of D (far frequencies
                                by the box's moments) instead of evaluated per frequency    */
@@ -319,7 +319,7 @@ int chi0_interpolate_kq(chi0_plan_t *plan, const double *qfrac, double *e_kq, vo
 typedef struct {
   int static_variant;       /* block shape of the static weight kernel: FP32 0 = 256
                                threads x 2 blocks per SM (128 registers), 1 = 128 x 3,
-                               2 = 256 x 1; FP64 always 0                           */
+                               2 = 256 x 1; FP64 always 0 (64 threads)              */
   int static_threads;       /* its threads per block                                */
   int static_ctas_per_sm;   /* persistent CTAs per SM of the static weight kernel  */
   int dynamic_ctas_per_sm;  /* ... of the dynamic weight kernel                     */

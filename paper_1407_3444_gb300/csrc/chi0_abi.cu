@@ -47,10 +47,12 @@ struct chi0_plan {
   cudaEvent_t ev_readers = nullptr;           // a second one in the current set, which no call
   int npend = 0;                              // reads again); ev_staged: their copies done
   unsigned long long *counters_d = nullptr;
-  short *occ_d = nullptr, *emp_d = nullptr, *occq_d = nullptr, *empq_d = nullptr;
+  short *bounds_d = nullptr, *boundsq_d = nullptr;  // band bounds per corner (4 arrays): k; k+q
+  int group = 1;                              // q points a static launch may cover: slots of W2_d,
+                                              // dos_d, boundsq_d, Eq32_d and pairs_fx_d
   float *E32_d = nullptr, *Eq32_d = nullptr;  // energies - eF in FP32 (mixed precision): hi, then lo
   void *C32_d = nullptr;                      // complex64 copy of complex128 eigenvectors (mixed)
-  int *next_d = nullptr;                      // [2] batch counter, FP64 list size
+  int *next_d = nullptr;                      // unit counter of the static weights
   int *err_d = nullptr;                       // error word of the bounded device waits
   cudaStream_t cap_s = nullptr;               // graph mode: private stream the graph runs on,
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;  // ordered after / before the plan's stream
@@ -72,10 +74,6 @@ struct chi0_plan {
   double *ikq_E_d = nullptr;                  // chi0_interpolate_kq with host outputs
   void *ikq_C_d = nullptr;
   size_t ikq_E_cap = 0, ikq_C_cap = 0;
-  void *tq_d = nullptr;                       // queued final tetrahedra per batch
-  int *tq_n_d = nullptr;
-  int *tq_off_d = nullptr;                    // compacted queue: offsets and values
-  double *tq_val_d = nullptr;
   int static_grid = 0, dynamic_grid = 0;  // persistent CTAs of the weight kernels
   int static_variant = 0;                  // block shape of the static weight kernel
   int tc_gcap = 0;                         // corners per tensor-core round (0: most that fit)
@@ -170,19 +168,13 @@ static void release(chi0_plan_t *p) {
     if (p->ev_staged[i]) cudaEventDestroy(p->ev_staged[i]);
   if (p->ev_readers) cudaEventDestroy(p->ev_readers);
   cudaFree(p->counters_d);
-  cudaFree(p->occ_d);
-  cudaFree(p->emp_d);
-  cudaFree(p->empq_d);
-  cudaFree(p->occq_d);
+  cudaFree(p->bounds_d);
+  cudaFree(p->boundsq_d);
   cudaFree(p->E32_d);
   cudaFree(p->C32_d);
   cudaFree(p->Eq32_d);
   cudaFree(p->next_d);
   cudaFree(p->err_d);
-  cudaFree(p->tq_d);
-  cudaFree(p->tq_n_d);
-  cudaFree(p->tq_off_d);
-  cudaFree(p->tq_val_d);
   cudaFree(p->box_tab_d);
   cudaFree(p->box_part_d);
   cudaFree(p->box_tot_d);
@@ -202,6 +194,20 @@ extern "C" void chi0_destroy(chi0_plan_t *p) {
   else cudaDeviceSynchronize();
   release(p);
   delete p;
+}
+
+// band bounds per corner: four arrays of nc from base on
+static BandBounds bounds_at(short *base, long long nc) { return BandBounds{base, base + nc, base + 2 * nc, base + 3 * nc}; }
+
+// bounds and FP32 energies of the plan's own eigen-data
+static cudaError_t plan_bands(chi0_plan_t *p) {
+  const Grid &g = p->g;
+  BandArgs a{};
+  a.E[0] = p->E_d;
+  a.out = bounds_at(p->bounds_d, g.nc);
+  a.E32 = p->E32_d;
+  a.E32lo = p->E32_d ? p->E32_d + (size_t)g.nc * g.nb : nullptr;
+  return launch_bands(a, 1, g.nc, g.nb, g.ef, p->stream);
 }
 
 static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t *tt, chi0_band_window_t win,
@@ -295,38 +301,35 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
                 g.norb);
   CK(p, cudaMalloc(&p->err_d, sizeof(int)));
   CK(p, cudaMemsetAsync(p->err_d, 0, sizeof(int), p->stream));
-  if (!op.cma) {
-    const size_t es = op.precision == CHI0_PREC_FP64 ? sizeof(double) : sizeof(float);
-    CK(p, cudaMalloc(&p->W2_d, es * (size_t)g.nc * w * w));
+  if (g.nc >= (1LL << 31)) return fail(p, CHI0_EINVAL, "more than 2^31 corners");
+  const size_t es = op.precision == CHI0_PREC_FP64 ? sizeof(double) : sizeof(float);
+  const size_t w2b = op.cma ? 0 : es * (size_t)g.nc * w * w, ncb = (size_t)g.nc * g.nb;
+  {
+    // Small meshes: a static call takes several q points per launch (one is too little work for
+    // the chip), each with its own slot of scratch, as many as fit in 64 MB.  At 48^3 x 9 bands
+    // one q holds 44 MB and fills the chip by itself.
+    const size_t perq = w2b + 4 * sizeof(short) * (size_t)g.nc +
+                        (op.precision == CHI0_PREC_MIXED ? 2 * sizeof(float) * ncb : 0);
+    const size_t fit = perq ? ((size_t)64 << 20) / perq : 1;
+    p->group = fit < 1 ? 1 : (fit > (size_t)kMaxGroup ? kMaxGroup : (int)fit);
   }
+  const size_t G = (size_t)p->group;
+  if (!op.cma) CK(p, cudaMalloc(&p->W2_d, G * w2b));
   const size_t np = (size_t)static_batches(g.ntet) * dynamic_max_nw();
-  size_t ns = 2 * (size_t)static_batches(g.ntet);
-  if (ns < (size_t)static_blocks()) ns = (size_t)static_blocks();
+  const size_t ns = G * (size_t)static_max_units(g.ntet);
   p->part_cap = np > ns ? np : ns;
   CK(p, cudaMalloc(&p->partR, sizeof(double) * p->part_cap));
-  CK(p, cudaMalloc(&p->partI, sizeof(double) * p->part_cap));
-  CK(p, cudaMalloc(&p->dos_d, sizeof(double) * static_blocks()));
+  CK(p, cudaMalloc(&p->partI, sizeof(double) * np));
+  CK(p, cudaMalloc(&p->dos_d, sizeof(double) * G * static_blocks()));
   CK(p, cudaMalloc(&p->counters_d, sizeof(unsigned long long) * 4));
-  if (g.nc >= (1LL << 31)) return fail(p, CHI0_EINVAL, "more than 2^31 corners");
-  CK(p, cudaMalloc(&p->occ_d, sizeof(short) * g.nc));
-  CK(p, cudaMalloc(&p->emp_d, sizeof(short) * g.nc));
-  CK(p, cudaMalloc(&p->empq_d, sizeof(short) * g.nc));
-  CK(p, cudaMalloc(&p->occq_d, sizeof(short) * g.nc));
-  CK(p, cudaMalloc(&p->next_d, 2 * sizeof(int)));
-  {
-    const long long nbatch = static_batches(g.ntet);
-    const int fp64 = op.precision == CHI0_PREC_FP64;
-    CK(p, cudaMalloc(&p->tq_d, static_piece_bytes(fp64) * (size_t)nbatch * static_tab_cap()));
-    CK(p, cudaMalloc(&p->tq_n_d, sizeof(int) * (size_t)nbatch));
-    CK(p, cudaMalloc(&p->tq_off_d, sizeof(int) * (size_t)(nbatch + 1)));
-    CK(p, cudaMalloc(&p->tq_val_d, sizeof(double) * (size_t)nbatch * static_tab_cap()));
-  }
+  CK(p, cudaMalloc(&p->bounds_d, 4 * sizeof(short) * g.nc));
+  CK(p, cudaMalloc(&p->boundsq_d, G * 4 * sizeof(short) * g.nc));
+  CK(p, cudaMalloc(&p->next_d, sizeof(int)));
   if (op.precision == CHI0_PREC_MIXED) {
-    CK(p, cudaMalloc(&p->E32_d, 2 * sizeof(float) * (size_t)g.nc * g.nb));
-    CK(p, cudaMalloc(&p->Eq32_d, 2 * sizeof(float) * (size_t)g.nc * g.nb));
+    CK(p, cudaMalloc(&p->E32_d, 2 * sizeof(float) * ncb));
+    CK(p, cudaMalloc(&p->Eq32_d, G * 2 * sizeof(float) * ncb));
   }
-  CK(p, launch_bands(p->E_d, g.nc, g.nb, g.ef, p->occ_d, p->emp_d, p->E32_d, p->stream,
-                     p->E32_d ? p->E32_d + (size_t)g.nc * g.nb : nullptr));
+  CK(p, plan_bands(p));
   if (op.precision == CHI0_PREC_MIXED && !op.cma && p->dtype == CHI0_C128) {
     const long long ne = g.nc * (long long)g.norb * g.nb;
     CK(p, cudaMalloc(&p->C32_d, 8 * (size_t)ne));
@@ -494,6 +497,139 @@ int prepare_q(chi0_plan_t *p, const chi0_q_t &qd, Q &q, int *slot_used) {
 
 }  // namespace
 
+// |M|^2 of n prepared q points into W2 slots 0 .. n - 1
+static int enqueue_overlap(chi0_plan_t *p, const Q *q, int n, Timer &tm, bool tc) {
+  const chi0_opts_t &op = p->opts;
+  const int fp64 = op.precision == CHI0_PREC_FP64;
+  if (op.cma) return CHI0_OK;
+  const int wp = p->win.hi - p->win.lo;
+  const size_t slot = (fp64 ? sizeof(double) : sizeof(float)) * (size_t)p->g.nc * wp * wp;
+  tm.start(CHI0_K_OVERLAP);
+  if (tc) {
+    for (int i = 0; i < n; ++i)
+      CK(p, launch_overlap_tc(p->g, p->C32_d ? p->C32_d : p->C_d, p->dtype, q[i], (float *)((char *)p->W2_d + i * slot),
+                              tc_mode(op.overlap), op.wait_budget, op.test_stall, p->tc_gcap, p->err_d, p->stream));
+    p->stats.kernels += n;
+  } else {
+    OverlapArgs a{};
+    a.g = p->g;
+    a.nq = n;
+    for (int i = 0; i < n; ++i) {
+      a.q[i] = q[i];
+      a.W2[i] = (char *)p->W2_d + i * slot;
+    }
+    CK(p, launch_overlap(a, p->C_d, p->dtype, fp64, p->stream, p->C32_d));
+    p->stats.kernels += 1;
+  }
+  tm.stop();
+  return CHI0_OK;
+}
+
+// bounds and FP32 energies of n q points with explicit k+q energies into slots 0 .. n - 1
+static int enqueue_bands(chi0_plan_t *p, const Q *q, int n, Timer &tm) {
+  const Grid &g = p->g;
+  const size_t ncb = (size_t)g.nc * g.nb;
+  const bool mixed = p->opts.precision == CHI0_PREC_MIXED;
+  BandArgs a{};
+  for (int i = 0; i < n; ++i) a.E[i] = q[i].Eq;
+  a.out = bounds_at(p->boundsq_d, g.nc);
+  a.stride_c = 4 * (size_t)g.nc;
+  a.E32 = mixed ? p->Eq32_d : nullptr;
+  a.E32lo = mixed ? p->Eq32_d + ncb : nullptr;
+  a.stride_e = 2 * ncb;
+  tm.start(CHI0_K_BANDS);
+  CK(p, launch_bands(a, n, g.nc, g.nb, g.ef, p->stream));
+  p->stats.kernels += 1;
+  tm.stop();
+  return CHI0_OK;
+}
+
+static int enqueue_dos(chi0_plan_t *p, const Q &q, int slot, unsigned long long *pfx, Timer &tm) {
+  tm.start(CHI0_K_DOS);
+  CK(p, launch_dos(p->g, p->tet, p->E_d, q.lo, q.hi, p->dos_d + (size_t)slot * static_blocks(), static_blocks(), p->stream, pfx));
+  p->stats.kernels += 1;
+  tm.stop();
+  return CHI0_OK;
+}
+
+// Launches of a static call, a group of q points at a time: overlaps, DOS at Gamma, band bounds
+// of explicit k+q energies, weights, reduction.  A group is a run of q points that are all
+// shifts or all explicit; explicit data from the host go one q at a time (two staging buffers,
+// each copy beside the kernels of the q before).
+static int enqueue_static(chi0_plan_t *p, const chi0_q_t *qs, int nq, double *out, Timer &tm, bool tc, double *outP) {
+  const chi0_opts_t &op = p->opts;
+  const int fp64 = op.precision == CHI0_PREC_FP64;
+  const double scale = op.sign == CHI0_SIGN_PAPER ? -2.0 : 2.0;
+  cudaStream_t s = p->stream;
+  const Grid &g = p->g;
+  const int wp = p->win.hi - p->win.lo;
+  const size_t ncb = (size_t)g.nc * g.nb;
+  size_t poff = 0;  // band-pair output: offset of this q's w x w block
+  for (int i0 = 0; i0 < nq;) {
+    const bool ex = qs[i0].e_kq != nullptr;
+    const int most = ex && !op.inputs_on_device ? 1 : p->group;
+    Q q[kMaxGroup];
+    int n = 0, slot = -1;
+    for (; n < most && i0 + n < nq && (qs[i0 + n].e_kq != nullptr) == ex; ++n) {
+      const int rc = prepare_q(p, qs[i0 + n], q[n], &slot);
+      if (rc) return rc;
+    }
+    if (outP) CK(p, cudaMemsetAsync(p->pairs_fx_d, 0, sizeof(unsigned long long) * n * wp * wp, s));
+    int rc = enqueue_overlap(p, q, n, tm, tc);
+    if (!rc && ex) rc = enqueue_bands(p, q, n, tm);
+    if (rc) return rc;
+    StaticArgs a{};
+    a.g = g;
+    a.tet = p->tet;
+    a.Ek = fp64 ? (const void *)p->E_d : (const void *)p->E32_d;
+    const BandBounds kb = bounds_at(p->bounds_d, g.nc);
+    a.occ = kb.occ;
+    a.occf = kb.occf;
+    a.cma = op.cma;
+    a.tau = (float)op.tau;
+    a.next = p->next_d;
+    a.counters = op.profile ? p->counters_d : nullptr;
+    a.nq = n;
+    double *part = p->partR;
+    for (int i = 0; i < n; ++i) {
+      StaticQ &d = a.q[i];
+      d.q = q[i];
+      const int w = q[i].hi - q[i].lo;
+      const BandBounds qb = ex ? bounds_at(p->boundsq_d + (size_t)i * 4 * g.nc, g.nc) : kb;
+      d.emp = qb.emp;
+      d.empf = qb.empf;
+      d.Ekq = !ex ? a.Ek : (fp64 ? (const void *)q[i].Eq : (const void *)(p->Eq32_d + (size_t)i * 2 * ncb));
+      d.W2 = op.cma ? nullptr : (char *)p->W2_d + (fp64 ? sizeof(double) : sizeof(float)) * (size_t)i * g.nc * wp * wp;
+      d.partial = part;
+      part += static_units(g.ntet, w);
+      d.pairs = outP ? p->pairs_fx_d + (size_t)i * wp * wp : nullptr;
+      d.dos = nullptr;
+      if (q[i].gamma) {
+        if ((rc = enqueue_dos(p, q[i], i, d.pairs, tm))) return rc;
+        d.dos = p->dos_d + (size_t)i * static_blocks();
+      }
+    }
+    tm.start(CHI0_K_STATIC);
+    CK(p, launch_static(a, fp64, p->static_grid, s, p->static_variant));
+    p->stats.kernels += 1;
+    tm.stop();
+    tm.start(CHI0_K_REDUCE);
+    CK(p, launch_static_reduce(a, scale, static_blocks(), out + i0, s));
+    p->stats.kernels += 1;
+    if (outP)
+      for (int i = 0; i < n; ++i) {
+        const int w = q[i].hi - q[i].lo;
+        CK(p, launch_pairs_out(a.q[i].pairs, w * w, scale, outP + poff, s));
+        p->stats.kernels += 1;
+        poff += (size_t)w * w;
+      }
+    tm.stop();
+    if (slot >= 0) CK(p, cudaEventRecord(p->ev_free[slot], s));  // its staging buffer is free again
+    i0 += n;
+  }
+  return CHI0_OK;
+}
+
 // Every launch and device-side copy of one call, in stream order (the part a CUDA graph
 // captures): counters, then per q the overlap, DOS, band bounds, weights and reductions.
 static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double *om_d, int nw, bool dyn,
@@ -503,70 +639,26 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
   const int fp64 = op.precision == CHI0_PREC_FP64;
   const double scale = op.sign == CHI0_SIGN_PAPER ? -2.0 : 2.0;
   cudaStream_t s = p->stream;
-  CK(p, cudaMemsetAsync(p->counters_d, 0, sizeof(unsigned long long) * 4, s));
-  size_t poff = 0;  // band-pair output: offset of this q's w x w block
+  if (op.profile) CK(p, cudaMemsetAsync(p->counters_d, 0, sizeof(unsigned long long) * 4, s));
+  if (!dyn) return enqueue_static(p, qs, nq, outR, tm, tc, outP);
   for (int iq = 0; iq < nq; ++iq) {
     Q q;
     int slot = -1;
     int rc = prepare_q(p, qs[iq], q, &slot);
     if (rc) return rc;
-    const int wq = q.hi - q.lo;
-    unsigned long long *pfx = outP ? p->pairs_fx_d : nullptr;
-    if (pfx) CK(p, cudaMemsetAsync(pfx, 0, sizeof(unsigned long long) * wq * wq, s));
-    if (!op.cma) {
-      tm.start(CHI0_K_OVERLAP);
-      if (tc)
-        CK(p, launch_overlap_tc(p->g, p->C32_d ? p->C32_d : p->C_d, p->dtype, q, (float *)p->W2_d,
-                                tc_mode(op.overlap), op.wait_budget, op.test_stall, p->tc_gcap,
-                                p->err_d, s));
-      else
-        CK(p, launch_overlap(p->g, p->E_d, p->C_d, p->dtype, q, p->W2_d, fp64, s, p->C32_d));
-      p->stats.kernels += 1;
-      tm.stop();
-    }
+    if ((rc = enqueue_overlap(p, &q, 1, tm, tc))) return rc;
     const int ndos = static_blocks();
-    if (q.gamma) {
-      tm.start(CHI0_K_DOS);
-      CK(p, launch_dos(p->g, p->tet, p->E_d, q.lo, q.hi, p->dos_d, ndos, s, pfx));
-      p->stats.kernels += 1;
-      tm.stop();
-    }
+    if (q.gamma && (rc = enqueue_dos(p, q, 0, nullptr, tm))) return rc;
+    if (q.Eq && (rc = enqueue_bands(p, &q, 1, tm))) return rc;
     const int nb = (int)static_batches(p->g.ntet);
-    const short *empq = p->emp_d;
-    const void *Ek = fp64 ? (const void *)p->E_d : (const void *)p->E32_d;
-    const void *Ekq = Ek;
     const size_t ncb = (size_t)p->g.nc * p->g.nb;
-    const float *Eklo = fp64 ? nullptr : p->E32_d + ncb, *Ekqlo = Eklo;
-    if (q.Eq) {
-      tm.start(CHI0_K_BANDS);
-      CK(p, launch_bands(q.Eq, p->g.nc, p->g.nb, p->g.ef, p->occq_d, p->empq_d, fp64 ? nullptr : p->Eq32_d, s,
-                         fp64 ? nullptr : p->Eq32_d + ncb));
-      p->stats.kernels += 1;
-      tm.stop();
-      empq = p->empq_d;
-      Ekq = fp64 ? (const void *)q.Eq : (const void *)p->Eq32_d;
-      if (!fp64) Ekqlo = p->Eq32_d + ncb;
-    }
-    if (!dyn) {
-      // (the compacted queue indexes its pieces in 32 bits)
-      const bool compact = (long long)nb * static_tab_cap() < (1LL << 31);
-      StaticBufs sb{p->tq_d, p->tq_n_d, p->partR, p->next_d, static_tab_cap(), pfx,
-                    compact ? p->tq_off_d : nullptr, compact ? p->tq_val_d : nullptr};
-      tm.start(CHI0_K_STATIC);
-      CK(p, launch_static(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, p->occ_d, empq, sb,
-                          p->static_grid, p->counters_d, s, p->static_variant));
-      p->stats.kernels += compact ? 4 : 2;
-      tm.stop();
-      tm.start(CHI0_K_REDUCE);
-      CK(p, launch_reduce(p->partR, 2 * nb, 1, scale, q.gamma ? p->dos_d : nullptr, ndos, nullptr, outR + iq, s));
-      p->stats.kernels += 1;
-      if (pfx) {
-        CK(p, launch_pairs_out(pfx, wq * wq, scale, outP + poff, s));
-        p->stats.kernels += 1;
-        poff += (size_t)wq * wq;
-      }
-      tm.stop();
-    } else if (kk_du > 0.0) {
+    const short *occ = bounds_at(p->bounds_d, p->g.nc).occ;
+    const short *empq = bounds_at(q.Eq ? p->boundsq_d : p->bounds_d, p->g.nc).emp;
+    const void *Ek = fp64 ? (const void *)p->E_d : (const void *)p->E32_d;
+    const void *Ekq = !q.Eq ? Ek : (fp64 ? (const void *)q.Eq : (const void *)p->Eq32_d);
+    const float *Eklo = fp64 ? nullptr : p->E32_d + ncb, *Ekqlo = fp64 || !q.Eq ? Eklo : p->Eq32_d + ncb;
+    unsigned long long *counters = op.profile ? p->counters_d : nullptr;
+    if (kk_du > 0.0) {
       // Kramers-Kronig route: Im alone on the uniform grid (passes of at most maxw nodes), then
       // Re from Im over the whole grid
       const int maxw = dynamic_max_nw();
@@ -576,8 +668,8 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
                    p->ctr_d};
         int rows = nb;
         tm.start(CHI0_K_DYNAMIC);
-        CK(p, launch_dynamic_im(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, p->occ_d, empq,
-                                om_d + w0, nwc, db, p->dynamic_grid, p->counters_d, s, Eklo, Ekqlo, &rows));
+        CK(p, launch_dynamic_im(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, occ, empq,
+                                om_d + w0, nwc, db, p->dynamic_grid, counters, s, Eklo, Ekqlo, &rows));
         p->stats.kernels += fp64 ? 1 : 2;
         tm.stop();
         tm.start(CHI0_K_REDUCE);
@@ -598,8 +690,8 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
                    p->ctr_d};
         int rows = nb;
         tm.start(CHI0_K_DYNAMIC);
-        CK(p, launch_dynamic(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, p->occ_d, empq,
-                             om_d + w0, nwc, db, p->dynamic_grid, p->counters_d, s, Eklo, Ekqlo, &rows));
+        CK(p, launch_dynamic(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, occ, empq,
+                             om_d + w0, nwc, db, p->dynamic_grid, counters, s, Eklo, Ekqlo, &rows));
         p->stats.kernels += fp64 ? 4 : 5;  // box table, weights, box sums, box evaluation (+ row sums)
         tm.stop();
         tm.start(CHI0_K_REDUCE);
@@ -646,8 +738,7 @@ static void drop_graph(chi0_plan_t *p) {
 // band bounds and FP32 copies of the plan's current eigen-data (the mixed form's inputs)
 static int derive_inputs(chi0_plan_t *p) {
   const Grid &g = p->g;
-  CK(p, launch_bands(p->E_d, g.nc, g.nb, g.ef, p->occ_d, p->emp_d, p->E32_d, p->stream,
-                     p->E32_d ? p->E32_d + (size_t)g.nc * g.nb : nullptr));
+  CK(p, plan_bands(p));
   p->stats.kernels += 1;
   if (p->C32_d) {
     CK(p, launch_c128_to_c64(p->C_d, p->C32_d, g.nc * (long long)g.norb * g.nb, p->stream));
@@ -724,7 +815,7 @@ static int run(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double *omega, 
   size_t npairs = 0;
   if (pairs) {
     const int wp = p->win.hi - p->win.lo;
-    int rc = ensure(p, (void **)&p->pairs_fx_d, &p->pairs_fx_cap, sizeof(unsigned long long) * wp * wp);
+    int rc = ensure(p, (void **)&p->pairs_fx_d, &p->pairs_fx_cap, sizeof(unsigned long long) * p->group * wp * wp);
     if (rc) return rc;
     for (int iq = 0; iq < nq; ++iq) {
       const int lo = qs[iq].win.lo < 0 ? p->win.lo : qs[iq].win.lo, hi = qs[iq].win.lo < 0 ? p->win.hi : qs[iq].win.hi;

@@ -1,6 +1,6 @@
 // chi0_grid.cuh -- device helpers shared by the weight kernels: tetrahedron corners of the
 // k mesh (Sec. II: the integration domain split into tetrahedra) at k and at k+q, small
-// quotients without a division sequence, and warp sums.
+// quotients without a division sequence, band-pair sums and warp sums.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -64,6 +64,29 @@ __device__ __forceinline__ void tet_corners(const Grid &g, const Tet &tet, const
     cq[3] = cid(g, i0 + 1 + s[0], i1 + 1 + s[1], i2 + 1 + s[2]);
   }
   vol = tet.vol_builtin;
+}
+
+// double -> float rounded to nearest even by integer operations (keeps the conversion of
+// complex128 inputs off the FP64 pipe); magnitudes below 2^-126 flush to zero
+__device__ __forceinline__ float d2f_int(double x) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+  const unsigned hi = (unsigned)(u >> 32);
+  const unsigned sign = hi & 0x80000000u;
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;
+  if (e <= 0) return __uint_as_float(sign);
+  if (e >= 255) return __uint_as_float(sign | 0x7f800000u | (((u << 12) != 0ull && e > 1000) ? 0x400000u : 0u));
+  const unsigned long long mant = u & 0xFFFFFFFFFFFFFull;
+  unsigned m = (unsigned)(mant >> 29);
+  const unsigned rem = (unsigned)(mant & 0x1FFFFFFFull);
+  m += (rem > 0x10000000u) | ((rem == 0x10000000u) & (m & 1u));
+  return __uint_as_float(sign | (((unsigned)e << 23) + m));  // a mantissa carry rounds into the exponent
+}
+
+// band-pair output: 64-bit fixed point in units of 2^-50 (|pair totals| < 2^13; one rounding
+// of 2^-51 per term)
+constexpr double kPairScale = 1125899906842624.0;  // 2^50
+__device__ __forceinline__ void pair_add(unsigned long long *pairs, int idx, double v) {
+  atomicAdd(&pairs[idx], (unsigned long long)__double2ll_rn(v * kPairScale));
 }
 
 __device__ __forceinline__ double warp_sum(double v) {

@@ -57,43 +57,71 @@ struct Q {
 
 enum { DT_C64 = 1, DT_C128 = 2 };
 
-// |M_mn|^2 at every k corner for one q: W2[c][m-lo][n-lo] (fp64: double, else float)
-cudaError_t launch_overlap(const Grid &g, const double *E, const void *C, int dtype, const Q &q,
-                           void *W2, int fp64, cudaStream_t s, const void *C32);
+// q points that one launch may cover: their descriptors travel as a kernel argument (4 KB)
+constexpr int kMaxGroup = 32;
+
+// |M_mn|^2 at every k corner for a group of q: W2[iq][c][m-lo][n-lo] (fp64: double, else float);
+// the q points are all explicit or all on-grid shifts
+struct OverlapArgs {
+  Grid g;
+  int nq;
+  Q q[kMaxGroup];
+  void *W2[kMaxGroup];
+};
+cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int fp64, cudaStream_t s, const void *C32);
 // complex128 -> complex64 copy (the k-side eigenvectors of a mixed-precision plan)
 cudaError_t launch_c128_to_c64(const void *in, void *out, long long n, cudaStream_t s);
 
-// band bounds per corner: occ[c] (1 + highest occupied band), emp[c] (lowest empty band);
+// band bounds per corner: occ[c] (1 + highest occupied band), emp[c] (lowest empty band), occf[c]
+// (bands below it are all occupied), empf[c] (bands from it on are all empty)
+struct BandBounds {
+  short *occ, *emp, *occf, *empf;
+};
+// Bounds of nq sets of energies E[iq] (set iq's outputs iq * stride_c / stride_e further on);
 // E32 (optional) receives (float)(E - ef); E32lo (optional) the remainder
 // (float)((E - ef) - E32), so that E32 + E32lo carries E - ef to ~2^-48 relative
-cudaError_t launch_bands(const double *E, long long nc, int nb, double ef, short *occ, short *emp, float *E32,
-                         cudaStream_t s, float *E32lo = nullptr);
-
-// Work buffers of the static kernels (device memory owned by the plan).
-struct StaticBufs {
-  void *tq;        // queued final tetrahedra: [nbatch][static_tab_cap()] pieces
-  int *tq_n;       // [nbatch] queued per batch
-  double *partial; // [2 * nbatch]: series part, queued part
-  int *next;       // batch counter
-  int tcap;        // queue entries per batch (at most static_tab_cap())
-  unsigned long long *pairs = nullptr;  // band-pair output: [w][w] fixed-point totals (or none)
-  int *off = nullptr;      // compacted queue: [nbatch + 1] offsets and [nbatch * tcap] values
-  double *vals = nullptr;  // (both null: one warp per batch walks its queue)
+struct BandArgs {
+  const double *E[kMaxGroup];
+  BandBounds out;
+  float *E32, *E32lo;
+  size_t stride_c, stride_e;
 };
+cudaError_t launch_bands(const BandArgs &a, int nq, long long nc, int nb, double ef, cudaStream_t s);
 
-// static weights for one q: partial[2 * nbatch] (sum them for chi0); Ek/Ekq are the absolute
-// FP64 energies (fp64) or the FP32 energies relative to eF (mixed); occ from the k
-// energies, empq from the k+q energies
-cudaError_t launch_static(const Grid &g, const Tet &tet, const void *Ek, const void *Ekq, const Q &q,
-                          const void *W2, int cma, int fp64, float tau, const short *occ, const short *empq,
-                          const StaticBufs &sb, int nblocks, unsigned long long *counters, cudaStream_t s, int variant = 0);
+// one q of a static launch: k+q energies (FP64 absolute, or FP32 relative to eF) and their band
+// bounds, |M|^2, one FP64 partial per unit, the band-pair totals (or none), the Gamma DOS
+// partials (or none); u0, tlog: set by launch_static
+struct StaticQ {
+  Q q;
+  const void *Ekq, *W2;
+  const short *emp, *empf;
+  double *partial;
+  unsigned long long *pairs;
+  const double *dos;
+  int u0, tlog;
+};
+struct StaticArgs {
+  Grid g;
+  Tet tet;
+  const void *Ek;            // k energies: FP64 absolute, or FP32 relative to eF
+  const short *occ, *occf;   // their band bounds
+  int cma;
+  float tau;
+  int *next;                 // unit counter
+  unsigned long long *counters;  // profile: pieces, FP64 evaluations, queue overflows (or none)
+  int nq, units;
+  StaticQ q[kMaxGroup];
+};
+// static weights of a group of q points, then chi = scale * (sum of partials (+ Gamma DOS))
+cudaError_t launch_static(StaticArgs &a, int fp64, int nblocks, cudaStream_t s, int variant = 0);
+cudaError_t launch_static_reduce(const StaticArgs &a, double scale, int ndos, double *out, cudaStream_t s);
 int static_persistent_blocks(int fp64);
-long long static_batches(long long ntet);
-int static_tab_cap();
+long long static_batches(long long ntet);  // runs of 32 tetrahedra (the dynamic weights' batches)
+long long static_units(long long ntet, int w);   // partials of one q with a window of w bands
+long long static_max_units(long long ntet);      // ... of any window
 
 // message of the last failed call made without a plan (chi0_last_error(NULL))
 void set_global_error(const char *msg);
-size_t static_piece_bytes(int fp64);
 
 // Work buffers of the dynamic weights: one partial per (batch of 32 tetrahedra, frequency) for
 // the pieces evaluated directly, and the far-field box moments (per warp, then summed)

@@ -71,6 +71,19 @@ __device__ __forceinline__ float rcp(float x) {
   return __frcp_rn(x);
 #endif
 }
+// FP64 reciprocal of the static weights: the hardware seed and two Newton-Raphson steps (four
+// multiply-adds on the FP64 pipe, about 1 ulp; IEEE division takes more than twice that).
+__device__ __forceinline__ double rcp_nr(double x) {
+#ifdef __CUDA_ARCH__
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  r = fma(r, fma(-x, r, 1.0), r);
+  return fma(r, fma(-x, r, 1.0), r);
+#else
+  return 1.0 / x;
+#endif
+}
+__device__ __forceinline__ float rcp_nr(float x) { return rcp(x); }
 __device__ __forceinline__ double quot(double a, double b) { return a / b; }
 __device__ __forceinline__ float quot(float a, float b) { return __fdividef(a, b); }
 
@@ -253,6 +266,223 @@ template <typename T> __device__ T series_sum(const T x[4], const T f[4]) {
     big = tabs(term) > big ? tabs(term) : big;
     if (k >= 2 && tabs(term) + tabs(prev) <= Num<T>::tol * (tabs(sum) > big ? tabs(sum) : big)) break;
     prev = term;
+  }
+  return sum * ci;
+}
+
+// ------------------------------------------------------------------------------------
+// The same integral by a polynomial of fixed length about the MEAN of the knots (FP64 static
+// weights).  With c = mean(x), e = (x - c)/c and |e_j| <= R < 1, 1/(1 + t) is replaced on
+// [-R, R] by the degree K - 1 polynomial p(t) = sum_k p_k t^k, and
+//   sum_j f_j (1/V) int_S lambda_j / X = (1/c) sum_k a_k s_k,   a_k = p_k 6 k!/(k+4)!,
+//   s_k = sum_j f_j h_k(e_1..e_4, e_j) = [z^k] N(z)/Q(z)^2,
+//   Q(z) = prod_i (1 - e_i z) = 1 + E2 z^2 - E3 z^3 + E4 z^4   (E1 = sum e = 0 about the mean),
+//   N(z) = sum_j f_j Q(z)/(1 - e_j z) = N0 + N1 z + N2 z^2 + N3 z^3.
+// Dividing by Q is a three-term recurrence, so the sum is taken backward (Clenshaw's scheme,
+// applied once per factor Q): y_k = a_k - E2 y_{k+2} + E3 y_{k+3} - E4 y_{k+4}, the same from
+// y to z, and sum_k a_k s_k = N0 z_0 + N1 z_1 + N2 z_2 + N3 z_3 (Q/(1 - e_j z) = 1 + e_j z +
+// (E2 + e_j^2) z^2 + (E2 e_j - E3 + e_j^3) z^3).  Six multiply-adds per term
+// and no convergence test, against about twenty operations of the forward series_sum above;
+// the knots need not be sorted; E1 = 0 is what drops a fourth multiply-add per factor.
+// p is the Chebyshev series of 1/(1 + t) on [-R, R] cut after K terms (q = R/(1 + sqrt(1-R^2)),
+// error at most 2 q^K / ((1 - q) sqrt(1 - R^2))), which reaches R ~ 2 tol^(1/K) where the
+// Taylor series ends at tol^(1/K): 16 terms where Taylor takes 22 (R = 0.16).
+// One tier per K = 4, 8, 12, ...: its largest R, and its a_k in a table.
+constexpr double kMeanTolD = 1.0e-17;  // truncation (below one rounding)
+constexpr int kMeanTiersD = 14;
+constexpr double kMeanRD[kMeanTiersD] = {0.00009, 0.01373, 0.07195, 0.16362, 0.26542, 0.36291, 0.44985,
+                                         0.52463, 0.58785, 0.64092, 0.68541, 0.72278, 0.75431, 0.78103};
+constexpr double mean_sqrt(double x) {  // Newton's iteration (compile time, 0 < x <= 1)
+  double r = 1.0;
+  for (int i = 0; i < 60; ++i) r = 0.5 * (r + x / r);
+  return r;
+}
+constexpr double mean_err(double R, int K) {  // the Chebyshev truncation bound above
+  const double s = mean_sqrt(1.0 - R * R), q = R / (1.0 + s);
+  double t = 2.0 / ((1.0 - q) * s);
+  for (int i = 0; i < K; ++i) t *= q;
+  return t;
+}
+constexpr int mean_off(int tier) { return 2 * tier * (tier + 1); }  // a tier's first coefficient
+// threshold on the high word of max|e| (FP32: its bits): bits <= thr implies max|e| <= R
+constexpr int mean_bits(double x, bool dbl) {
+  int e = 0;
+  while (x < 1.0) {
+    x *= 2.0;
+    --e;
+  }
+  return dbl ? (((1023 + e) << 20) | (int)((x - 1.0) * 1048576.0)) - 1
+             : (((127 + e) << 23) | (int)((x - 1.0) * 8388608.0));
+}
+template <typename T, int NT> struct MeanTab {
+  T a[2 * NT * (NT + 1)];
+  int thr[NT];
+  constexpr MeanTab(const double (&R)[NT], double tol) : a(), thr() {
+    for (int i = 0; i < NT; ++i) {
+      const int K = 4 * (i + 1);
+      thr[i] = mean_bits(R[i], sizeof(T) == 8);
+      if (mean_err(R[i], K) > tol) thr[i] = -1 / (K - K);  // (compile error: R too large for K)
+      const double s = mean_sqrt(1.0 - R[i] * R[i]), q = R[i] / (1.0 + s);
+      // sum_n c_n T_n(t/R), c_0 = 1/s, c_n = 2 (-q)^n / s, collected in powers of u = t/R
+      double p[4 * NT] = {}, t0[4 * NT] = {}, t1[4 * NT] = {};
+      t0[0] = 1.0;
+      t1[1] = 1.0;
+      double c = 1.0 / s;
+      p[0] = c;
+      c *= -2.0 * q;
+      for (int n = 1; n < K; ++n) {
+        for (int k = 0; k <= n; ++k) p[k] += c * t1[k];
+        c *= -q;
+        double t2[4 * NT] = {};
+        for (int k = 0; k <= n && k + 1 < 4 * NT; ++k) t2[k + 1] = 2.0 * t1[k];
+        for (int k = 0; k <= n; ++k) {
+          t2[k] -= t0[k];
+          t0[k] = t1[k];
+        }
+        for (int k = 0; k < 4 * NT; ++k) t1[k] = t2[k];
+      }
+      double rk = 1.0;
+      for (int k = 0; k < K; ++k) {
+        // p_k differs from Taylor's (-1)^k by the truncation; a difference of a few roundings is
+        // this computation's own and is dropped (it would be a bias common to all pieces)
+        const double one = (k & 1) ? -1.0 : 1.0, dp = p[k] / rk - one;
+        const double pk = dp < 1e-15 && dp > -1e-15 ? one : p[k] / rk;
+        a[mean_off(i) + k] = (T)(pk * 6.0 / ((k + 1.0) * (k + 2.0) * (k + 3.0) * (k + 4.0)));
+        rk *= R[i];
+      }
+    }
+  }
+};
+__constant__ constexpr MeanTab<double, kMeanTiersD> kMeanD{kMeanRD, kMeanTolD};
+template <typename T> struct Mean;
+template <> struct Mean<float> {
+  static __device__ __forceinline__ int bits(float x) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(x) & 0x7fffffff;
+#else
+    int i;
+    memcpy(&i, &x, 4);
+    return i & 0x7fffffff;
+#endif
+  }
+};
+template <> struct Mean<double> {
+  static constexpr int tiers = kMeanTiersD;
+  static __device__ __forceinline__ int thr(int i) { return kMeanD.thr[i]; }
+  static __device__ __forceinline__ double a(int i) { return kMeanD.a[i]; }
+  static __device__ __forceinline__ int bits(double x) {
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x) & 0x7fffffff;
+#else
+    long long i;
+    memcpy(&i, &x, 8);
+    return (int)(i >> 32) & 0x7fffffff;
+#endif
+  }
+};
+// offsets e = d ci - 1 (one rounding each; 1/d = ci/(1 + e) holds for ci as it is), ci = 1/mean,
+// and the bits of max|e| (a NaN, from knots that are all 0, lies above every threshold)
+template <typename T> __device__ __forceinline__ int mean_offsets(const T d[4], T e[4], T &ci) {
+  ci = rcp_nr(((d[0] + d[1]) + (d[2] + d[3])) * T(0.25));
+  int r = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    e[i] = fma(d[i], ci, T(-1));
+    const int b = Mean<T>::bits(e[i]);
+    r = b > r ? b : r;
+  }
+  return r;
+}
+// the smallest of the first N tiers that holds max|e| of these bits (N: none)
+template <typename T, int N> __device__ __forceinline__ int mean_tier(int bits) {
+  int t = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) t += bits > Mean<T>::thr(i) ? 1 : 0;
+  return t;
+}
+template <typename T> __device__ __forceinline__ T mean_series(const T e[4], const T f[4], T ci, int tier) {
+  const T s = e[0] + e[1], e3 = -(s + e[2]);  // (sum of e = 0)
+  const T P = e[0] * e[1], Q = e[2] * e3;
+  const T E2 = (P + Q) - s * s, E3 = s * (Q - P), nE4 = -(P * Q), nE2 = -E2;
+  const int base = 2 * tier * (tier + 1);  // the tier's first coefficient
+  int t = 4 * tier;
+  // the last four terms (nothing above them), then four at a time
+  T Y3 = Mean<T>::a(base + t + 3), Y2 = Mean<T>::a(base + t + 2);
+  T Y1 = nE2 * Y3 + Mean<T>::a(base + t + 1), Y0 = nE2 * Y2 + (E3 * Y3 + Mean<T>::a(base + t));
+  T Z3 = Y3, Z2 = Y2, Z1 = nE2 * Z3 + Y1, Z0 = nE2 * Z2 + (E3 * Z3 + Y0);
+#pragma unroll 1
+  for (t -= 4; t >= 0; t -= 4) {
+    const T n3 = nE2 * Y1 + (E3 * Y2 + (nE4 * Y3 + Mean<T>::a(base + t + 3)));
+    const T n2 = nE2 * Y0 + (E3 * Y1 + (nE4 * Y2 + Mean<T>::a(base + t + 2)));
+    const T n1 = nE2 * n3 + (E3 * Y0 + (nE4 * Y1 + Mean<T>::a(base + t + 1)));
+    const T n0 = nE2 * n2 + (E3 * n3 + (nE4 * Y0 + Mean<T>::a(base + t)));
+    const T z3 = nE2 * Z1 + (E3 * Z2 + (nE4 * Z3 + n3));
+    const T z2 = nE2 * Z0 + (E3 * Z1 + (nE4 * Z2 + n2));
+    const T z1 = nE2 * z3 + (E3 * Z0 + (nE4 * Z1 + n1));
+    const T z0 = nE2 * z2 + (E3 * z3 + (nE4 * Z0 + n0));
+    Y0 = n0, Y1 = n1, Y2 = n2, Y3 = n3;
+    Z0 = z0, Z1 = z1, Z2 = z2, Z3 = z3;
+  }
+  // sum_k N_k z_k = sum_j f_j (A + e_j (B + e_j (z_2 + e_j z_3)))
+  const T A = (Z0 - E3 * Z3) + E2 * Z2, B = Z1 + E2 * Z3;
+  T sum = f[0] * (A + e[0] * (B + e[0] * (Z2 + e[0] * Z3)));
+  sum += f[1] * (A + e[1] * (B + e[1] * (Z2 + e[1] * Z3)));
+  sum += f[2] * (A + e[2] * (B + e[2] * (Z2 + e[2] * Z3)));
+  sum += f[3] * (A + e3 * (B + e3 * (Z2 + e3 * Z3)));
+  return sum * ci;
+}
+
+// series_sum's own terms, by a cheaper recurrence (FP32 static weights): the same expansion about
+// the midpoint, cut by the same rule (two successive terms at or below tol), so that the sums agree
+// to rounding.  s_k = [z^k] N(z) / Q(z)^2 with Q = (1 - r^2 z^2)(1 - e1 z)(1 - e2 z), r = -e0 = e3: two
+// divisions by each factor, six multiply-adds per term where the h_k of all four vertices take
+// thirteen operations.  N = n0 + n1 z + n2 z^2 + n3 z^3 from the power sums of f e^i.
+__device__ __forceinline__ float series_sum_short(const float x[4], const float f[4]) {
+  const float c = (x[0] + x[3]) * 0.5f, ci = rcp(c);
+  const float r = (x[3] - x[0]) * 0.5f * ci, e1 = fmaf(x[1], ci, -1.0f), e2 = fmaf(x[2], ci, -1.0f);
+  const float r2 = r * r;
+  // power sums m_i = sum_j f_j e_j^i
+  const float fs = f[0] + f[3], fd = (f[3] - f[0]) * r;
+  const float g1 = f[1] * e1, g2 = f[2] * e2, h1 = g1 * e1, h2 = g2 * e2;
+  const float m0 = fs + (f[1] + f[2]), m1 = fd + (g1 + g2), m2 = fmaf(r2, fs, h1 + h2);
+  const float m3 = fmaf(r2, fd, fmaf(h1, e1, h2 * e2));
+  // elementary symmetric polynomials of the offsets (-r, e1, e2, r)
+  const float E1 = e1 + e2, P = e1 * e2, E2 = P - r2, E3 = -r2 * E1;
+  const float n1 = m1 - E1 * m0, n2 = fmaf(E2, m0, m2 - E1 * m1), n3 = fmaf(E2, m1, m3) - fmaf(E3, m0, E1 * m2);
+  // stage by stage: x = N/(1 - r2 z2), y = x/(1 - r2 z2), then twice 1/(1 - e1 z), twice 1/(1 - e2 z)
+  float xa = m0, xb = n1, ya = m0, yb = n1;  // the last two of x and y (even, odd)
+  float v = m0, vv = m0, u = m0, uu = m0;
+  auto step = [&](float y) {
+    v = fmaf(e1, v, y);
+    vv = fmaf(e1, vv, v);
+    u = fmaf(e2, u, vv);
+    uu = fmaf(e2, uu, u);
+    return uu;
+  };
+  float sum = 0.25f * m0, big = tabs(sum);
+  float tp = series_coef<float>(1) * step(yb);
+  sum += tp;
+  xa = fmaf(r2, xa, n2);
+  ya = fmaf(r2, ya, xa);
+  float t = series_coef<float>(2) * step(ya);
+  sum += t;
+  big = fmaxf(fmaxf(big, tabs(sum)), fmaxf(tabs(tp), tabs(t)));
+  const float thr = Num<float>::tol * big;  // (the sum moves little after the second term)
+  if (tabs(t) + tabs(tp) > thr) {
+    xb = fmaf(r2, xb, n3);
+#pragma unroll 1
+    for (int k = 3; k < Num<float>::kmax; k += 2) {
+      yb = fmaf(r2, yb, xb);
+      tp = series_coef<float>(k) * step(yb);
+      sum += tp;
+      if (tabs(t) + tabs(tp) <= thr) break;
+      xb *= r2;
+      xa *= r2;
+      ya = fmaf(r2, ya, xa);
+      t = series_coef<float>(k + 1) * step(ya);
+      sum += t;
+      if (tabs(t) + tabs(tp) <= thr) break;
+    }
   }
   return sum * ci;
 }
@@ -750,6 +980,114 @@ __device__ __forceinline__ int cut_piece(const Vt<T> in[4], int idx, Vt<T> P[4],
     r = (T(1) - s0) * (T(1) - s1) * s2;
   }
   return 3;
+}
+
+// ------------------------------------------------------------------------------------
+// The same cut without branches (static weights).  Every piece of a cut has at most three
+// vertices on the cut plane, and its volume ratio is the product, over them, of the cut fraction
+// t or of 1 - t.  A recipe names them: three slots (i, j, flip) for the point where the key
+// vanishes on edge i (key < 0) - j, and the original vertex of the fourth slot; a slot with i = j
+// stands for vertex i itself (t = 0, flip: factor 1).  One table of recipes, indexed by the set of
+// vertices with key < 0 and the piece number: the lanes of a warp all run the same code, where
+// cut_piece runs its one-, two- and three-vertex cases one after the other (ten cut points for a
+// piece's three), and the vertices need no sorting (only which side they are on matters: FP64; the FP32 caller
+// sorts them by key all the same, which keeps its pieces, and with them the rounding errors of
+// its near-degenerate ones, what cut_piece makes).
+// ------------------------------------------------------------------------------------
+constexpr unsigned cut_recipe(int mask, int idx) {
+  int N[4] = {}, P[4] = {}, nn = 0, np = 0;
+  for (int i = 0; i < 4; ++i)
+    if ((mask >> i) & 1) N[nn++] = i;
+    else P[np++] = i;
+  int s[3][3] = {}, last = 0;
+  auto set = [&](int k, int i, int j, int flip) {
+    s[k][0] = i;
+    s[k][1] = j;
+    s[k][2] = flip;
+  };
+  const int a = N[0], b = N[1], c = N[2], p = P[0], q = P[1], r = P[2];
+  if (nn == 1) {  // corner tetrahedron
+    set(0, a, p, 0);
+    set(1, a, q, 0);
+    set(2, a, r, 0);
+    last = a;
+  } else if (nn == 2) {  // prism (a, ap, aq) - (b, bp, bq)
+    last = b;
+    if (idx == 0) {
+      set(0, a, p, 0);
+      set(1, a, q, 0);
+      set(2, a, a, 1);
+    } else if (idx == 1) {
+      set(0, a, p, 1);
+      set(1, a, q, 0);
+      set(2, b, p, 0);
+    } else {
+      set(0, a, q, 1);
+      set(1, b, p, 0);
+      set(2, b, q, 0);
+    }
+  } else if (nn == 3) {  // prism (a, b, c) - (ap, bp, cp)
+    last = c;
+    set(0, a, p, idx == 0 ? 0 : 1);
+    if (idx == 0) set(1, a, a, 1);
+    else set(1, b, p, idx == 1 ? 0 : 1);
+    if (idx < 2) set(2, b, b, 1);
+    else set(2, c, p, 0);
+  } else {  // nothing cut
+    set(0, 0, 0, 1);
+    set(1, 1, 1, 1);
+    set(2, 2, 2, 1);
+    last = 3;
+  }
+  unsigned v = 0;
+  for (int k = 0; k < 3; ++k) v |= (unsigned)(s[k][0] | (s[k][1] << 2) | (s[k][2] << 4)) << (5 * k);
+  return v | ((unsigned)last << 15);
+}
+struct CutTab {
+  unsigned v[64];
+  constexpr CutTab() : v() {
+    for (int m = 0; m < 16; ++m)
+      for (int i = 0; i < 3; ++i) v[m * 4 + i] = cut_recipe(m, i);
+  }
+};
+__constant__ constexpr CutTab kCutTab{};  // (copied to shared memory: lanes index it apart)
+// pieces of a cut by the number of vertices kept
+__device__ __forceinline__ int cut_count(unsigned mask) {
+  const int n = (int)((0x4332322132212110ull >> (4 * mask)) & 7ull);  // bits set
+  return n == 0 ? 0 : ((n == 1 || n == 4) ? 1 : 3);
+}
+template <typename T> __device__ __forceinline__ T sel4(const T v[4], unsigned i) {
+  const T a = (i & 1u) ? v[1] : v[0], b = (i & 1u) ? v[3] : v[2];
+  return (i & 2u) ? b : a;
+}
+__device__ __forceinline__ float cut_quot(float a, float b) { return quot(a, b); }
+__device__ __forceinline__ double cut_quot(double a, double b) { return a * rcp_nr(b); }
+// cut fraction of slot k (0 for an unused slot) and the values at its vertex
+template <typename T> __device__ __forceinline__ T cut_frac(unsigned rec, int k, const T key[4]) {
+  const unsigned sl = rec >> (5 * k);
+  const T ki = sel4(key, sl & 3u), den = ki - sel4(key, (sl >> 2) & 3u);
+  return den != T(0) ? cut_quot(ki, den) : T(0);
+}
+template <typename T> __device__ __forceinline__ T cut_mix(unsigned rec, int k, const T v[4], T t) {
+  const unsigned sl = rec >> (5 * k);
+  return (T(1) - t) * sel4(v, sl & 3u) + t * sel4(v, (sl >> 2) & 3u);
+}
+__device__ __forceinline__ bool cut_used(unsigned rec, int k) {
+  const unsigned sl = rec >> (5 * k);
+  return (sl & 3u) != ((sl >> 2) & 3u);
+}
+template <typename T> __device__ __forceinline__ T cut_factor(unsigned rec, int k, T t) {
+  return ((rec >> (5 * k + 4)) & 1u) ? T(1) - t : t;
+}
+// x < 0 (FP64: on the integer pipe; false for -0 and NaN)
+__device__ __forceinline__ bool is_neg(float x) { return x < 0.0f; }
+__device__ __forceinline__ bool is_neg(double x) {
+#ifdef __CUDA_ARCH__
+  const long long b = __double_as_longlong(x);
+  return b < 0 && ((unsigned long long)b << 1) - 1ull < 0xFFE0000000000000ull;
+#else
+  return x < 0.0;
+#endif
 }
 
 // Both carvings of one (tetrahedron, band pair): emit(vol_ratio, d[4], f[4]) for every

@@ -33,7 +33,10 @@ static __device__ __align__(256) unsigned char g_chi0_scratch[CHI0_NOALLOC_SCRAT
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr int kNoallocTabCap = 16;  // queue entries per batch (overflow is evaluated in place)
+// the array's work region per batch of 32 tetrahedra: 640 (FP32) or 1280 (FP64) bytes, of which
+// the unit partials (at most 64 per batch) and the band bounds beyond occ and emp (16 per
+// corner, at most 8 corners per cube) take less than half
+constexpr size_t kNoallocWork32 = 640, kNoallocWork64 = 1280;
 unsigned char *g_scratch_ptr[kMaxDevices] = {nullptr};
 std::mutex g_scratch_mu;
 
@@ -72,7 +75,7 @@ size_t mul_sat(size_t a, size_t b) { return (b != 0 && a > kSat / b) ? kSat : a 
 size_t align256(size_t x) { return x > kSat - 255 ? kSat : (x + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t occ, emp, occq, empq, E32, Eq32, C32, W2, next, counters, tq, tq_n, part, dos, total;
+  size_t bounds, E32, Eq32, C32, W2, next, counters, work, dos, total;
 };
 
 Layout layout(const Grid &g, int w, int fp64, int cma, int dtype) {
@@ -87,19 +90,19 @@ Layout layout(const Grid &g, int w, int fp64, int cma, int dtype) {
   };
   const size_t nc = (size_t)g.nc, nb = (size_t)g.nb, no = (size_t)g.norb, ww = (size_t)w;
   const size_t nbatch = (size_t)static_batches(g.ntet);
-  L.occ = take(mul_sat(sizeof(short), nc));
-  L.emp = take(mul_sat(sizeof(short), nc));
-  L.occq = take(mul_sat(sizeof(short), nc));
-  L.empq = take(mul_sat(sizeof(short), nc));
+  L.bounds = take(mul_sat(sizeof(short), nc));  // occ, emp, and the same at k+q
+  take(mul_sat(sizeof(short), nc));
+  take(mul_sat(sizeof(short), nc));
+  take(mul_sat(sizeof(short), nc));
   L.E32 = take(fp64 ? 0 : mul_sat(mul_sat(sizeof(float), nc), nb));
   L.Eq32 = take(fp64 ? 0 : mul_sat(mul_sat(sizeof(float), nc), nb));
   L.C32 = take((!fp64 && !cma && dtype == CHI0_C128) ? mul_sat(mul_sat(mul_sat(8, nc), no), nb) : 0);
   L.W2 = take(cma ? 0 : mul_sat(mul_sat(mul_sat(fp64 ? 8 : 4, nc), ww), ww));
   L.next = take(sizeof(int));
   L.counters = take(4 * sizeof(unsigned long long));
-  L.tq = take(mul_sat(mul_sat(static_piece_bytes(fp64), nbatch), kNoallocTabCap));
-  L.tq_n = take(mul_sat(sizeof(int), nbatch));
-  L.part = take(mul_sat(sizeof(double), mul_sat(2, nbatch)));
+  L.work = take(mul_sat(fp64 ? kNoallocWork64 : kNoallocWork32, nbatch));
+  take(mul_sat(sizeof(int), nbatch));
+  take(mul_sat(sizeof(double), mul_sat(2, nbatch)));
   L.dos = take(mul_sat(sizeof(double), (size_t)static_blocks()));
   L.total = o;
   return L;
@@ -142,7 +145,6 @@ extern "C" int chi0_static_noalloc(const chi0_kgrid_t *kg, chi0_band_window_t wi
   if (g.nc >= (1LL << 31) || g.ntet >= (1LL << 31)) return err(CHI0_EINVAL, "mesh too large");
   const int dtype = op.cma ? CHI0_C128 : kg->evec_dtype;
   const int w = win.hi - win.lo;
-  const long long nbatch = static_batches(g.ntet);
   const Layout L = layout(g, w, fp64, op.cma, dtype);
   if (L.total > (size_t)CHI0_NOALLOC_SCRATCH_BYTES)
     return err(CHI0_EINVAL, "this mesh needs %zu bytes of scratch; chi0_static_noalloc has %zu", L.total,
@@ -160,15 +162,16 @@ extern "C" int chi0_static_noalloc(const chi0_kgrid_t *kg, chi0_band_window_t wi
   int rc = scratch_base(&base);
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)op.stream;
-  short *occ = (short *)(base + L.occ), *emp = (short *)(base + L.emp);
-  short *occq = (short *)(base + L.occq), *empq = (short *)(base + L.empq);
+  // band bounds: occ, emp (k and k+q) in their own region, occf, empf in the work region
+  const size_t cs = align256(sizeof(short) * (size_t)g.nc) / sizeof(short);
+  short *bb = (short *)(base + L.bounds), *wb = (short *)(base + L.work);
+  const BandBounds kb{bb, bb + cs, wb, wb + g.nc}, qb{bb + 2 * cs, bb + 3 * cs, wb + 2 * g.nc, wb + 3 * g.nc};
   float *E32 = fp64 ? nullptr : (float *)(base + L.E32), *Eq32 = fp64 ? nullptr : (float *)(base + L.Eq32);
   void *C32 = (!fp64 && !op.cma && dtype == CHI0_C128) ? (void *)(base + L.C32) : nullptr;
   void *W2 = op.cma ? nullptr : (void *)(base + L.W2);
   int *next = (int *)(base + L.next);
-  unsigned long long *counters = (unsigned long long *)(base + L.counters);
-  double *part = (double *)(base + L.part), *dos = (double *)(base + L.dos);
-  StaticBufs sb{base + L.tq, (int *)(base + L.tq_n), part, next, kNoallocTabCap};
+  double *part = (double *)(base + L.work + ((4 * sizeof(short) * (size_t)g.nc + 7) & ~(size_t)7));
+  double *dos = (double *)(base + L.dos);
   Tet tet{nullptr, nullptr, 1.0 / (6.0 * g.n[0] * g.n[1] * g.n[2])};
   const double scale = op.sign == CHI0_SIGN_PAPER ? -2.0 : 2.0;
   cudaError_t e;
@@ -176,8 +179,11 @@ extern "C" int chi0_static_noalloc(const chi0_kgrid_t *kg, chi0_band_window_t wi
   do {                                                                                               \
     if ((e = (call)) != cudaSuccess) return err(CHI0_ECUDA, "%s: %s", #call, cudaGetErrorString(e)); \
   } while (0)
-  NA_CK(cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned long long), s));
-  NA_CK(launch_bands(kg->energies, g.nc, g.nb, g.ef, occ, emp, E32, s));
+  BandArgs ba{};
+  ba.E[0] = kg->energies;
+  ba.out = kb;
+  ba.E32 = E32;
+  NA_CK(launch_bands(ba, 1, g.nc, g.nb, g.ef, s));
   if (C32) NA_CK(launch_c128_to_c64(kg->evecs, C32, g.nc * (long long)g.norb * g.nb, s));
   const int grid = static_persistent_blocks(fp64);
   for (int iq = 0; iq < nq; ++iq) {
@@ -199,18 +205,42 @@ extern "C" int chi0_static_noalloc(const chi0_kgrid_t *kg, chi0_band_window_t wi
       }
       if (zero) q.gamma = 1;
     }
-    if (!op.cma) NA_CK(launch_overlap(g, kg->energies, kg->evecs, dtype, q, W2, fp64, s, C32));
-    if (q.gamma) NA_CK(launch_dos(g, tet, kg->energies, q.lo, q.hi, dos, static_blocks(), s));
-    const short *empq_use = emp;
-    const void *Ek = fp64 ? (const void *)kg->energies : (const void *)E32, *Ekq = Ek;
-    if (q.Eq) {
-      NA_CK(launch_bands(q.Eq, g.nc, g.nb, g.ef, occq, empq, fp64 ? nullptr : Eq32, s));
-      empq_use = empq;
-      Ekq = fp64 ? (const void *)q.Eq : (const void *)Eq32;
+    if (!op.cma) {
+      OverlapArgs oa{};
+      oa.g = g;
+      oa.nq = 1;
+      oa.q[0] = q;
+      oa.W2[0] = W2;
+      NA_CK(launch_overlap(oa, kg->evecs, dtype, fp64, s, C32));
     }
-    NA_CK(launch_static(g, tet, Ek, Ekq, q, W2, op.cma, fp64, (float)op.tau, occ, empq_use, sb, grid, counters, s));
-    NA_CK(launch_reduce(part, (int)(2 * nbatch), 1, scale, q.gamma ? dos : nullptr, static_blocks(), nullptr,
-                        chi + iq, s));
+    if (q.gamma) NA_CK(launch_dos(g, tet, kg->energies, q.lo, q.hi, dos, static_blocks(), s));
+    if (q.Eq) {
+      BandArgs bq{};
+      bq.E[0] = q.Eq;
+      bq.out = qb;
+      bq.E32 = Eq32;
+      NA_CK(launch_bands(bq, 1, g.nc, g.nb, g.ef, s));
+    }
+    StaticArgs a{};
+    a.g = g;
+    a.tet = tet;
+    a.Ek = fp64 ? (const void *)kg->energies : (const void *)E32;
+    a.occ = kb.occ;
+    a.occf = kb.occf;
+    a.cma = op.cma;
+    a.tau = (float)op.tau;
+    a.next = next;
+    a.nq = 1;
+    StaticQ &d = a.q[0];
+    d.q = q;
+    d.Ekq = !q.Eq ? a.Ek : (fp64 ? (const void *)q.Eq : (const void *)Eq32);
+    d.W2 = W2;
+    d.emp = q.Eq ? qb.emp : kb.emp;
+    d.empf = q.Eq ? qb.empf : kb.empf;
+    d.partial = part;
+    d.dos = q.gamma ? dos : nullptr;
+    NA_CK(launch_static(a, fp64, grid, s));
+    NA_CK(launch_static_reduce(a, scale, static_blocks(), chi + iq, s));
   }
 #undef NA_CK
   return CHI0_OK;
