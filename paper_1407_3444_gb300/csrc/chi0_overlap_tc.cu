@@ -43,10 +43,17 @@
 // KB * 128 bytes along M/N.  One thread issues the MMAs and commits them to an mbarrier; every
 // wait on it is bounded (the plan's wait budget, in clock cycles) and a wait that runs out
 // sets the error word, frees the tensor memory and ends the kernel.
+//
+// Bound: the round's serial chain of staging, MMAs and epilogue in each CTA (the floor is HBM:
+// 32^3 corners of 40 bands read and write 1.05 GB, 0.16 ms; 80 bands 4.3 GB, 0.64 ms).  Measured
+// before (two-byte staging stores, no loads ahead, the issuing thread's index arithmetic between
+// MMAs) and now, 32^3 corners: 40 bands BF16X3 2.9 -> 0.86 ms, 20 of 40 bands 1.5 -> 0.46 ms,
+// 80 bands BF16X6 5.7 -> 2.8 ms.  Results are bitwise the same.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "chi0_grid.cuh"
 #include "chi0_internal.h"
 
 namespace chi0int {
@@ -137,17 +144,23 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint3
         "l"(a), "l"(b), "r"(id), "r"(acc));
 }
 
-// 8 consecutive FP32 columns of this thread's tensor-memory lane (load and wait in one block)
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
-  uint32_t r[8];
+// 8 consecutive FP32 columns at each of two addresses of this thread's tensor-memory lane (both
+// loads in flight together; loads and wait in one block)
+__device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, float v[8], float u[8]) {
+  uint32_t r[8], q[8];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n"
       "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-      : "r"(taddr)
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(q[0]),
+        "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7])
+      : "r"(ta), "r"(tb)
       : "memory");
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 8; ++i) {
+    v[i] = __uint_as_float(r[i]);
+    u[i] = __uint_as_float(q[i]);
+  }
 }
 
 __device__ __forceinline__ uint32_t tf32_rn(float x) {
@@ -195,50 +208,98 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
   }
 }
 
-// Stages orbitals [o0, o1) of the round's corners c0 .. c0 + G - 1 into one operand buffer
-// (P pieces of A, then P pieces of B; KB 16-byte columns per row): element (g, o, band) goes
-// to A row g*w + m and B rows g*2NW + n, g*2NW + NW + n at K columns 2(o - o0) and 2(o - o0) + 1.
-// kUnroll elements per thread and pass: all their loads are issued before the first store.
+// Staging moves one 16-byte column of K at a time: kOrb orbitals of one band of one corner (4 in
+// the BF16 forms, 2 in TF32), which is one 16-byte store per piece into each of the three operand
+// rows that the band fills (A row gg*w + m; B rows gg*2NW + n and gg*2NW + NW + n).  Threads of a
+// warp take neighbouring bands: their loads are contiguous and their stores fall on different
+// rows of a core matrix (no bank conflicts).  Two-byte stores, element by element, took 2 P x 6
+// stores where this takes 3 P / 4.
+template <int MODE> struct TcItem {
+  static constexpr int kOrb = MODE == TC_TF32 ? 2 : 4;
+};
+constexpr int kAhead = 3;  // items per thread whose loads are issued a step ahead
+
+__device__ __forceinline__ float2 as_float2(float2 v) { return v; }
+__device__ __forceinline__ float2 as_float2(double2 v) { return make_float2(grid::d2f_int(v.x), grid::d2f_int(v.y)); }
+
+// one item's loads (zeros past the last orbital of the chunk); row < 0: no such item
+template <int MODE, typename CTq> struct Staged {
+  float2 x[TcItem<MODE>::kOrb];
+  CTq y[TcItem<MODE>::kOrb];
+  int ra, rb, kb;
+};
+
 template <int MODE, typename CTq>
-__device__ __forceinline__ void stage_orbitals(const Grid &g, const float2 *__restrict__ C,
-                                               const CTq *__restrict__ Cb, int explicit_q, const Q &q,
-                                               const TcShape &sh, long long c0, int o0, int o1,
-                                               unsigned char *sA, unsigned char *sB, size_t a_piece,
-                                               size_t b_piece, int KB) {
-  const int w = sh.w, NW = sh.NW, no = g.norb, nob = o1 - o0;
-  const int per = nob * w, tot = sh.G * per;
-  constexpr int kUnroll = 4;
-  for (int i0 = threadIdx.x; i0 < tot; i0 += kUnroll * kTcThreads) {
-    float2 xv[kUnroll];
-    CTq yv[kUnroll];
-    int ra[kUnroll], rb[kUnroll], kk[kUnroll];
+__device__ __forceinline__ void load_item(const Grid &g, const float2 *__restrict__ C, const CTq *__restrict__ Cb,
+                                          int explicit_q, const Q &q, const TcShape &sh, long long c0, int o0, int o1,
+                                          int i, Staged<MODE, CTq> &t) {
+  constexpr int kOrb = TcItem<MODE>::kOrb;
+  const int w = sh.w, no = g.norb, nob = (o1 - o0 + kOrb - 1) / kOrb, per = nob * w;
+  const int gg = i / per, rem = i - gg * per;
+  const long long c = c0 + gg;
+  t.ra = -1;
+  if (gg >= sh.G || c >= g.nc) return;
+  const int ob = rem / w, mm = rem - ob * w, o = o0 + ob * kOrb;
+  const long long ck = explicit_q ? c : shift_corner(g, c, q.shift);
+  const float2 *px = C + (c * no + o) * g.nb + q.lo + mm;
+  const CTq *py = Cb + (ck * no + o) * g.nb + q.lo + mm;
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int i = i0 + u * kTcThreads;
-      const int gg = i / per, rem = i - gg * per;
-      const long long c = c0 + gg;
-      ra[u] = -1;
-      if (i >= tot || c >= g.nc) continue;
-      const int ol = rem / w, mm = rem - ol * w;
-      const int o = o0 + ol;
-      const long long ck = explicit_q ? c : shift_corner(g, c, q.shift);
-      xv[u] = C[(c * no + o) * g.nb + q.lo + mm];
-      yv[u] = Cb[(ck * no + o) * g.nb + q.lo + mm];
-      ra[u] = gg * w + mm;
-      rb[u] = gg * 2 * NW + mm;
-      kk[u] = 2 * ol;
+  for (int j = 0; j < kOrb; ++j) {
+    const bool in = o + j < o1;
+    t.x[j] = in ? px[(long long)j * g.nb] : make_float2(0.f, 0.f);
+    t.y[j] = CTq{};
+    if (in) t.y[j] = py[(long long)j * g.nb];
+  }
+  t.ra = gg * w + mm;
+  t.rb = gg * 2 * sh.NW + mm;
+  t.kb = ob;
+}
+
+// 16 bytes of K at (row r, 16-byte column kb) of every piece: (re, im) pairs of the item's orbitals
+__device__ __forceinline__ uint32_t row_off(int r, int kb, int KB) {
+  return (uint32_t)(((r >> 3) * KB + kb) * 128 + (r & 7) * 16);
+}
+__device__ __forceinline__ uint32_t bf16_pair(float2 v) {  // low half: v.x
+  const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+  return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+template <int MODE, typename CTq>
+__device__ __forceinline__ void store_item(const TcShape &sh, const Staged<MODE, CTq> &t, unsigned char *sA,
+                                           unsigned char *sB, size_t a_piece, size_t b_piece, int KB) {
+  if (t.ra < 0) return;
+  const uint32_t oa = row_off(t.ra, t.kb, KB), ob = row_off(t.rb, t.kb, KB), oi = row_off(t.rb + sh.NW, t.kb, KB);
+  if constexpr (MODE == TC_TF32) {
+    const float2 y0 = as_float2(t.y[0]), y1 = as_float2(t.y[1]);
+    *(uint4 *)(sA + oa) = make_uint4(tf32_rn(t.x[0].x), tf32_rn(t.x[0].y), tf32_rn(t.x[1].x), tf32_rn(t.x[1].y));
+    *(uint4 *)(sB + ob) = make_uint4(tf32_rn(y0.x), tf32_rn(y0.y), tf32_rn(y1.x), tf32_rn(y1.y));
+    *(uint4 *)(sB + oi) = make_uint4(tf32_rn(y0.y), tf32_rn(-y0.x), tf32_rn(y1.y), tf32_rn(-y1.x));
+  } else {
+    constexpr int P = MODE == TC_BF16X3 ? 2 : 3;
+    float2 x[4], y[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      x[j] = t.x[j];
+      y[j] = as_float2(t.y[j]);
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      if (ra[u] < 0) continue;
-      const float yr = (float)yv[u].x, yi = (float)yv[u].y;
-      const int k = kk[u];
-      put<MODE>(sA, a_piece, ra[u], k, KB, xv[u].x);
-      put<MODE>(sA, a_piece, ra[u], k + 1, KB, xv[u].y);
-      put<MODE>(sB, b_piece, rb[u], k, KB, yr);
-      put<MODE>(sB, b_piece, rb[u], k + 1, KB, yi);
-      put<MODE>(sB, b_piece, rb[u] + NW, k, KB, yi);
-      put<MODE>(sB, b_piece, rb[u] + NW, k + 1, KB, -yr);
+    for (int p = 0; p < P; ++p) {
+      uint32_t hx[4], hy[4], hi[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        hx[j] = bf16_pair(x[j]);
+        hy[j] = bf16_pair(y[j]);
+        hi[j] = __byte_perm(hy[j], 0u, 0x1032) ^ 0x80000000u;  // (im, -re)
+        if (p + 1 < P) {  // the rest, for the next piece
+          x[j].x -= __uint_as_float(hx[j] << 16);
+          x[j].y -= __uint_as_float(hx[j] & 0xFFFF0000u);
+          y[j].x -= __uint_as_float(hy[j] << 16);
+          y[j].y -= __uint_as_float(hy[j] & 0xFFFF0000u);
+        }
+      }
+      *(uint4 *)(sA + p * a_piece + oa) = make_uint4(hx[0], hx[1], hx[2], hx[3]);
+      *(uint4 *)(sB + p * b_piece + ob) = make_uint4(hy[0], hy[1], hy[2], hy[3]);
+      *(uint4 *)(sB + p * b_piece + oi) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
     }
   }
 }
@@ -258,7 +319,7 @@ __device__ __forceinline__ void zero_columns(const TcShape &sh, int k0, int k1, 
 }
 
 template <int MODE, typename CTq>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kTcThreads, sizeof(CTq) == 8 ? 2 : 1)
     k_overlap_tc(Grid g, const float2 *__restrict__ C, const CTq *__restrict__ Cb, int explicit_q, Q q,
                  float *__restrict__ W2, long long budget, int test_stall, int gcap, int *__restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -296,46 +357,81 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   const uint32_t id = idesc(MODE, sh.N);
+  const bool vec = (w & 3) == 0 && ((size_t)W2 & 15) == 0;  // every row of W2 starts on 16 bytes
   const long long nround = (g.nc + G - 1) / G;
   uint32_t parity = 0;
   bool ok = true;
-  // stages chunk j of the round starting at corner c0 into buffer j % nbuf
+  constexpr int kOrb = TcItem<MODE>::kOrb;
+  // Chunk j of the round at corner c0 goes to buffer j % nbuf.  The loads of a thread's first
+  // kAhead items are issued a chunk ahead (fetch), before the wait for the MMAs and the epilogue,
+  // and stored here; the rest are loaded here.
+  Staged<MODE, CTq> ahead[kAhead];
+  auto fetch = [&](long long c0, int j) {
+    const int o0 = j * ostep, o1 = min(g.norb, o0 + ostep);
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+      load_item<MODE, CTq>(g, C, Cb, explicit_q, q, sh, c0, o0, o1, tid + k * kTcThreads, ahead[k]);
+  };
   auto stage = [&](long long c0, int j) {
     unsigned char *sA = smem + (j % nbuf) * buf_bytes;
     unsigned char *sB = sA + sh.P * a_piece;
     const int o0 = j * ostep, o1 = min(g.norb, o0 + ostep);
-    stage_orbitals<MODE, CTq>(g, C, Cb, explicit_q, q, sh, c0, o0, o1, sA, sB, a_piece, b_piece, KB);
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) store_item<MODE, CTq>(sh, ahead[k], sA, sB, a_piece, b_piece, KB);
+    const int tot = G * ((o1 - o0 + kOrb - 1) / kOrb) * w;
+#pragma unroll 1
+    for (int i = tid + kAhead * kTcThreads; i < tot; i += kAhead * kTcThreads) {
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k)
+        load_item<MODE, CTq>(g, C, Cb, explicit_q, q, sh, c0, o0, o1, i + k * kTcThreads, ahead[k]);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) store_item<MODE, CTq>(sh, ahead[k], sA, sB, a_piece, b_piece, KB);
+    }
     // the last chunk of three or more may sit in a buffer whose K padding (inside its last K
-    // step) an earlier, longer chunk filled
+    // step) an earlier, longer chunk filled (an item writes whole 16-byte columns)
     if (sh.chunked && sh.nch >= 3 && j == sh.nch - 1) {
-      const int kstep = 32 / sh.ES, kused = 2 * (o1 - o0);
+      const int kstep = 32 / sh.ES, kcol = 16 / sh.ES, kused = (2 * (o1 - o0) + kcol - 1) / kcol * kcol;
       const int kpad = (kused + kstep - 1) / kstep * kstep;
       if (kused < kpad) zero_columns<MODE>(sh, kused, kpad, sA, sB, a_piece, b_piece, KB);
     }
     // generic-proxy stores must be visible to the tensor core's (async-proxy) reads
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   };
-  // one thread issues chunk j's MMAs and commits them to the mbarrier
+  // One thread issues chunk j's MMAs and commits them to the mbarrier.  The loops below are that
+  // thread's serial chain, so they hold nothing but the MMAs and descriptor sums (a K step is 256
+  // bytes further on: 16 in the descriptor's address field): with a modulo per K step to find the
+  // accumulator and descriptors built anew, the chain took 0.65 us per MMA, four fifths of the
+  // kernel at 40 bands.
+  constexpr int P = MODE == TC_TF32 ? 1 : (MODE == TC_BF16X3 ? 2 : 3);
   auto issue = [&](int j) {
     if (tid != 0 || test_stall) return;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned char *sA = smem + (j % nbuf) * buf_bytes;
-    const unsigned char *sB = sA + sh.P * a_piece;
-    const int s0 = j * sh.kc, s1 = min(sh.nks, s0 + sh.kc);  // global K steps of the chunk
-    for (int ia = 0; ia < sh.NACC; ++ia) {
-      // unchunked: K step s goes to accumulator s % NACC; chunked: chunk j to j * NACC / nch
-      if (sh.chunked && ia != j * sh.NACC / sh.nch) continue;
-      // the first MMA into an accumulator in this round overwrites it
-      uint32_t acc = (sh.chunked && j > 0 && (j - 1) * sh.NACC / sh.nch == ia) ? 1u : 0u;
+    const unsigned char *sB = sA + P * a_piece;
+    uint64_t da[P], db[P];
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      da[k] = sdesc(smem_u32(sA + k * a_piece), 128, KB * 128);
+      db[k] = sdesc(smem_u32(sB + k * b_piece), 128, KB * 128);
+    }
+    const int s0 = j * sh.kc, ns = min(sh.nks, s0 + sh.kc) - s0;  // K steps of the chunk
+    // unchunked: K step s goes to accumulator s % NACC; chunked: chunk j to j * NACC / nch
+    const int ia0 = sh.chunked ? j * sh.NACC / sh.nch : 0, ia1 = sh.chunked ? ia0 + 1 : sh.NACC;
+    const int sstep = sh.chunked ? 1 : sh.NACC;
+    // the first MMA into an accumulator in this round overwrites it
+    const uint32_t first = (sh.chunked && j > 0 && (j - 1) * sh.NACC / sh.nch == ia0) ? 1u : 0u;
+#pragma unroll 1
+    for (int ia = ia0; ia < ia1; ++ia) {
+      uint32_t acc = first;
+      const uint32_t at = tmem + (uint32_t)(ia * sh.N);
       // products of pieces a, b with a + b = lvl < P, smallest level first
-      for (int lvl = sh.P - 1; lvl >= 0; --lvl)
+#pragma unroll
+      for (int lvl = P - 1; lvl >= 0; --lvl)
+#pragma unroll
         for (int pa = 0; pa <= lvl; ++pa)
-          for (int s = s0; s < s1; ++s) {
-            if (!sh.chunked && s % sh.NACC != ia) continue;
-            const uint32_t kb = (uint32_t)(s - s0) * 256u;  // 32 bytes of K = 2 core-matrix columns
-            const uint64_t da = sdesc(smem_u32(sA + pa * a_piece) + kb, 128, KB * 128);
-            const uint64_t db = sdesc(smem_u32(sB + (lvl - pa) * b_piece) + kb, 128, KB * 128);
-            mma(tmem + (uint32_t)(ia * sh.N), da, db, id, acc, MODE);
+#pragma unroll 1
+          for (int s = sh.chunked ? 0 : ia; s < ns; s += sstep) {
+            mma(at, da[pa] + 16u * (uint32_t)s, db[lvl - pa] + 16u * (uint32_t)s, id, acc, MODE);
             acc = 1;
           }
     }
@@ -343,13 +439,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                      smem_u32(bar))
                  : "memory");
   };
+  if (blockIdx.x < nround) fetch((long long)blockIdx.x * G, 0);
   for (long long rd = blockIdx.x; rd < nround && ok; rd += gridDim.x) {
     const long long c0 = rd * G;
     stage(c0, 0);
+    if (sh.nch > 1) fetch(c0, 1);
     __syncthreads();
     for (int j = 0; j < sh.nch; ++j) {
       issue(j);
       if (j + 1 < sh.nch) stage(c0, j + 1);  // the other buffer: chunk j - 1's MMAs are done
+      if (j + 2 < sh.nch) fetch(c0, j + 2);
+      else if (j + 1 == sh.nch && rd + gridDim.x < nround) fetch((rd + gridDim.x) * G, 0);
       // test_stall: nothing arrives, so the bounded wait below runs out (error path test).  The
       // CTA agrees on the outcome before any warp-wide tensor-memory load or buffer reuse.
       const int got = mbar_wait(smem_u32(bar), parity, budget) ? 1 : 0;
@@ -369,25 +469,33 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int gg = r / (w > 0 ? w : 1), m = r - gg * w;
     const long long c = c0 + gg;
     const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    for (int blk = 0; blk < G; ++blk) {  // warp-uniform loops: every lane takes part in tcgen05.ld
+    // (the corner blocks that this warp's 32 rows belong to; rows past G*w belong to none)
+    const int blk0 = quarter * 32 / w, blk1 = min(G - 1, (quarter * 32 + 31) / w);
+    for (int blk = blk0; blk <= blk1; ++blk) {  // warp-uniform loops: every lane takes part in tcgen05.ld
       for (int n0 = half * 8; n0 < NW; n0 += 16) {
         float re[8], im[8];
-        tmem_ld8(trow + blk * 2 * NW + n0, re);
-        tmem_ld8(trow + blk * 2 * NW + NW + n0, im);
+        tmem_ld8x2(trow + blk * 2 * NW + n0, trow + blk * 2 * NW + NW + n0, re, im);
         for (int ia = 1; ia < sh.NACC; ++ia) {  // partial accumulators, added in FP32
           float r2[8], i2[8];
-          tmem_ld8(trow + ia * sh.N + blk * 2 * NW + n0, r2);
-          tmem_ld8(trow + ia * sh.N + blk * 2 * NW + NW + n0, i2);
+          tmem_ld8x2(trow + ia * sh.N + blk * 2 * NW + n0, trow + ia * sh.N + blk * 2 * NW + NW + n0, r2, i2);
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             re[j] += r2[j];
             im[j] += i2[j];
           }
         }
-        if (blk == gg && gg < G && c < g.nc) {
+        if (blk == gg && c < g.nc) {
+          float *out = W2 + (c * w + m) * w + n0;
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (n0 + j < w) W2[(c * w + m) * w + n0 + j] = re[j] * re[j] + im[j] * im[j];
+          for (int j = 0; j < 8; ++j) re[j] = re[j] * re[j] + im[j] * im[j];
+          if (vec) {
+            *(float4 *)out = make_float4(re[0], re[1], re[2], re[3]);
+            if (n0 + 4 < w) *(float4 *)(out + 4) = make_float4(re[4], re[5], re[6], re[7]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              if (n0 + j < w) out[j] = re[j];
+          }
         }
       }
     }
