@@ -60,10 +60,9 @@ struct chi0_plan {
   cudaGraphExec_t gexec = nullptr;
   std::vector<unsigned char> gkey;
   long long gkernels = 0;
-  void *box_tab_d = nullptr;                  // dynamic weights: box table of the pass,
-  double *box_part_d = nullptr;               // per-warp box moments, their totals and the
-  double *box_tot_d = nullptr;                // boxes' share of Re per frequency
-  double *far_d = nullptr;
+  void *box_tab_d = nullptr;                  // dynamic weights: boxes and sorted frequencies of the pass,
+  double *box_part_d = nullptr;               // box moments per warp or CTA, and their totals
+  double *box_tot_d = nullptr;
   void *fb_d = nullptr;                       // dynamic weights: per-warp fallback entries,
   unsigned long long *fx_d = nullptr;         // per-CTA fixed-point sums (FP32) and the
   unsigned long long *ctr_d = nullptr;        // batch counter
@@ -77,7 +76,6 @@ struct chi0_plan {
   int static_grid = 0, dynamic_grid = 0;  // persistent CTAs of the weight kernels
   int static_variant = 0;                  // block shape of the static weight kernel
   int tc_gcap = 0;                         // corners per tensor-core round (0: most that fit)
-  size_t part_cap = 0;
   chi0_stats_t stats;
   char err[512];
 };
@@ -178,7 +176,6 @@ static void release(chi0_plan_t *p) {
   cudaFree(p->box_tab_d);
   cudaFree(p->box_part_d);
   cudaFree(p->box_tot_d);
-  cudaFree(p->far_d);
   cudaFree(p->fb_d);
   cudaFree(p->fx_d);
   cudaFree(p->ctr_d);
@@ -315,10 +312,11 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
   }
   const size_t G = (size_t)p->group;
   if (!op.cma) CK(p, cudaMalloc(&p->W2_d, G * w2b));
-  const size_t np = (size_t)static_batches(g.ntet) * dynamic_max_nw();
+  // unit partials of the static weights; per-warp sums of the FP64 dynamic weights
+  const size_t np = op.precision == CHI0_PREC_FP64 ? (size_t)dynamic_max_ctas_per_sm(1) * device_sms() *
+                                                         dynamic_warps_per_cta(1) * dynamic_max_nw() : 1;
   const size_t ns = G * (size_t)static_max_units(g.ntet);
-  p->part_cap = np > ns ? np : ns;
-  CK(p, cudaMalloc(&p->partR, sizeof(double) * p->part_cap));
+  CK(p, cudaMalloc(&p->partR, sizeof(double) * (np > ns ? np : ns)));
   CK(p, cudaMalloc(&p->partI, sizeof(double) * np));
   CK(p, cudaMalloc(&p->dos_d, sizeof(double) * G * static_blocks()));
   CK(p, cudaMalloc(&p->counters_d, sizeof(unsigned long long) * 4));
@@ -350,7 +348,6 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
     CK(p, cudaMalloc(&p->box_tab_d, dynamic_box_tab_bytes()));
     CK(p, cudaMalloc(&p->box_part_d, sizeof(double) * warps * dynamic_box_slots(fp64)));
     CK(p, cudaMalloc(&p->box_tot_d, sizeof(double) * dynamic_box_slots(fp64)));
-    CK(p, cudaMalloc(&p->far_d, sizeof(double) * dynamic_max_nw()));
     CK(p, cudaMalloc(&p->fb_d, warps * dynamic_fb_bytes(fp64)));
     CK(p, cudaMalloc(&p->fx_d, dynamic_fx_bytes(dynamic_max_ctas_per_sm(fp64) * device_sms())));
     CK(p, cudaMalloc(&p->ctr_d, sizeof(unsigned long long)));
@@ -650,57 +647,41 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
     const int ndos = static_blocks();
     if (q.gamma && (rc = enqueue_dos(p, q, 0, nullptr, tm))) return rc;
     if (q.Eq && (rc = enqueue_bands(p, &q, 1, tm))) return rc;
-    const int nb = (int)static_batches(p->g.ntet);
     const size_t ncb = (size_t)p->g.nc * p->g.nb;
-    const short *occ = bounds_at(p->bounds_d, p->g.nc).occ;
-    const short *empq = bounds_at(q.Eq ? p->boundsq_d : p->bounds_d, p->g.nc).emp;
-    const void *Ek = fp64 ? (const void *)p->E_d : (const void *)p->E32_d;
-    const void *Ekq = !q.Eq ? Ek : (fp64 ? (const void *)q.Eq : (const void *)p->Eq32_d);
-    const float *Eklo = fp64 ? nullptr : p->E32_d + ncb, *Ekqlo = fp64 || !q.Eq ? Eklo : p->Eq32_d + ncb;
-    unsigned long long *counters = op.profile ? p->counters_d : nullptr;
-    if (kk_du > 0.0) {
-      // Kramers-Kronig route: Im alone on the uniform grid (passes of at most maxw nodes), then
-      // Re from Im over the whole grid
-      const int maxw = dynamic_max_nw();
-      for (int w0 = 0; w0 < nw; w0 += maxw) {
-        const int nwc = nw - w0 < maxw ? nw - w0 : maxw;
-        DynBufs db{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->far_d, p->fb_d, p->fx_d,
-                   p->ctr_d};
-        int rows = nb;
-        tm.start(CHI0_K_DYNAMIC);
-        CK(p, launch_dynamic_im(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, occ, empq,
-                                om_d + w0, nwc, db, p->dynamic_grid, counters, s, Eklo, Ekqlo, &rows));
-        p->stats.kernels += fp64 ? 1 : 2;
-        tm.stop();
-        tm.start(CHI0_K_REDUCE);
-        CK(p, launch_reduce(p->partI, rows, nwc, scale, nullptr, 0, nullptr, outI + (size_t)iq * nw + w0, s));
-        p->stats.kernels += 1;
-        tm.stop();
-      }
+    const BandBounds kb = bounds_at(p->bounds_d, p->g.nc), qb = q.Eq ? bounds_at(p->boundsq_d, p->g.nc) : kb;
+    DynArgs a{};
+    a.g = p->g;
+    a.tet = p->tet;
+    a.q = q;
+    a.Ek = fp64 ? (const void *)p->E_d : (const void *)p->E32_d;
+    a.Ekq = !q.Eq ? a.Ek : (fp64 ? (const void *)q.Eq : (const void *)p->Eq32_d);
+    a.W2 = p->W2_d;
+    a.Eklo = fp64 ? nullptr : p->E32_d + ncb;
+    a.Ekqlo = fp64 || !q.Eq ? a.Eklo : p->Eq32_d + ncb;
+    a.occ = kb.occ;
+    a.occf = kb.occf;
+    a.emp = qb.emp;
+    a.empf = qb.empf;
+    a.cma = op.cma;
+    a.tau = (float)op.tau;
+    a.db = DynBufs{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->fb_d, p->fx_d, p->ctr_d};
+    a.counters = op.profile ? p->counters_d : nullptr;
+    const bool kk = kk_du > 0.0;
+    const double *dos = q.gamma ? p->dos_d : nullptr;
+    const int maxw = dynamic_max_nw();
+    for (int w0 = 0; w0 < nw; w0 += maxw) {  // frequency passes
+      const int nwc = nw - w0 < maxw ? nw - w0 : maxw;
+      const size_t at = (size_t)iq * nw + w0;
+      tm.start(CHI0_K_DYNAMIC);
+      CK(p, launch_dynamic(a, fp64, kk, om_d + w0, nwc, p->dynamic_grid, scale, dos, ndos, outR + at, outI + at, s));
+      p->stats.kernels += kk ? 3 : 4;  // setup, weights, box sums, output
+      tm.stop();
+    }
+    if (kk) {  // Kramers-Kronig route: Re from Im over the whole grid
       tm.start(CHI0_K_REDUCE);
-      CK(p, launch_kk(outI + (size_t)iq * nw, nw, kk_du, scale, q.gamma ? p->dos_d : nullptr, ndos,
-                      outR + (size_t)iq * nw, s));
+      CK(p, launch_kk(outI + (size_t)iq * nw, nw, kk_du, scale, dos, ndos, outR + (size_t)iq * nw, s));
       p->stats.kernels += 1;
       tm.stop();
-    } else {
-      const int maxw = dynamic_max_nw();
-      for (int w0 = 0; w0 < nw; w0 += maxw) {
-        const int nwc = nw - w0 < maxw ? nw - w0 : maxw;
-        DynBufs db{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->far_d, p->fb_d, p->fx_d,
-                   p->ctr_d};
-        int rows = nb;
-        tm.start(CHI0_K_DYNAMIC);
-        CK(p, launch_dynamic(p->g, p->tet, Ek, Ekq, q, p->W2_d, op.cma, fp64, (float)op.tau, occ, empq,
-                             om_d + w0, nwc, db, p->dynamic_grid, counters, s, Eklo, Ekqlo, &rows));
-        p->stats.kernels += fp64 ? 4 : 5;  // box table, weights, box sums, box evaluation (+ row sums)
-        tm.stop();
-        tm.start(CHI0_K_REDUCE);
-        CK(p, launch_reduce(p->partR, rows, nwc, scale, q.gamma ? p->dos_d : nullptr, ndos, om_d + w0,
-                            outR + (size_t)iq * nw + w0, s, p->far_d));
-        CK(p, launch_reduce(p->partI, rows, nwc, scale, nullptr, 0, nullptr, outI + (size_t)iq * nw + w0, s));
-        p->stats.kernels += 2;
-        tm.stop();
-      }
     }
     if (slot >= 0) CK(p, cudaEventRecord(p->ev_free[slot], s));  // its staging buffer is free again
   }

@@ -11,43 +11,53 @@
 // far from a piece they are gathered per box of D instead of per (piece, frequency):
 //
 //   box b: centre C_b, radius R_b; every piece assigned to it has |d_j - C_b| <= R_b, and adds
-//     its moments  M_k += v sum_j f_j (1/V) int_S lambda_j eps^k,  eps = (D - C_b)/R_b,
-//     = v 6 k!/(k+4)! sum_j f_j h_k(e_1..e_4, e_j)  (e = (d - C_b)/R_b; Dirichlet moments of
-//     the simplex, h_k the complete homogeneous symmetric polynomials);
-//   1/(D -+ u) = 1/(C_b -+ u) sum_k (-z)^k eps^k,  z = R_b/(C_b -+ u),  |z| <= 1/2 where the
-//     box stands in for its pieces (1/3 in FP64), so the box's share of Re(u) is
-//     sum_k M_k (-z)^k/(C_b -+ u),
-//     evaluated once per (box, frequency) in FP64 after the moments of all warps are summed.
+//     its moments  M_k += v a_k s_k,  a_k = (-1)^k 6 k!/(k+4)!,  s_k = sum_j f_j h_k(e_1..e_4, e_j),
+//     e = (d - C_b)/R_b (Dirichlet moments of the simplex, h_k the complete homogeneous symmetric
+//     polynomials).  With eps = (D - C_b)/R_b and z = R_b/(C_b -+ u),
+//     1/(D -+ u) = (1/(C_b -+ u)) / (1 + z eps), and 1/(1 + t) is replaced on |t| <= z_max by a
+//     polynomial sum_k p_k t^k (the Chebyshev series of chi0_math.cuh), so the box's share of Re(u)
+//     is sum_k (-1)^k p_k M_k z^k/(C_b -+ u), evaluated once per (box, frequency) in FP64 after the
+//     moments of all warps are summed.  Against the Taylor series the same accuracy takes 20
+//     moments instead of 24 at z = 1/2 (FP32), 40 instead of 90 at z = 2/3 (FP64).
 //
 // Boxes (rebuilt each pass from u_max = max |w| of the pass):
 //   fine boxes, levels l = 0..3 of width w_l = (u_max/32) 2^l: centres (j + 1/2) w_l, radius
-//     w_l; a piece of half-width s <= w_l/2 whose centre lies in [j w_l, (j+1) w_l) fits.  For a
-//     frequency with |C_b - u| < F R_b (the - term) or C_b + u < F R_b (the + term), F = 2 in
-//     the FP32 kernel and 3 in the FP64 kernel (|z| <= 1/F elsewhere), the box does not stand
-//     in: its pieces evaluate that term themselves (own far-field series about their midpoint,
-//     or the divided-difference table near their knots);
-//   geometric boxes past u_max: x = c - u_max in [x_b, 1.25 x_b), x_0 = 5 u_max/32, centre
-//     u_max + 1.125 x_b, radius x_b/4, pieces with s <= x_b/8; every frequency of the pass is
-//     far (|z| <= 2/9), so their pieces evaluate nothing per frequency;
+//     w_l; a piece of half-width s <= w_l/2 whose centre lies in [j w_l, (j+1) w_l) fits.  The box
+//     stands in where |C_b - u| >= F R_b (the - term) or C_b + u >= F R_b (the + term); for the
+//     other frequencies its pieces evaluate that term themselves: by their own moments about
+//     their midpoint c where |c -+ u| >= F s, by the closed form nearer.  F = 2 (FP32), 1.5 (FP64);
+//   past u_max, x = c - u_max in [x_b, 1.25 x_b), x_0 = 5 u_max/32, every frequency of the pass is
+//     far and pieces evaluate nothing per frequency: geometric boxes (centre u_max + 1.125 x_b,
+//     radius x_b/4, pieces with s <= x_b/8, |z| <= 2/9), and, for pieces without a fine box, wide
+//     ones up to s = x_b/2 (radius 0.625 x_b, |z| <= 5/9): on coarse meshes a quarter of all pieces
+//     are that wide, and without a box each cost two closed forms at every frequency;
 //   pieces wider than any box, or past the last one, are evaluated at every frequency.
-// Every (piece, frequency, term) is taken exactly once, either by the piece or by its box;
-// the predicate that decides is computed in the kernels' precision from the same table.
+// Every (piece, frequency, term) is taken exactly once, either by the piece or by its box.
 //
-// Work layout.  A warp takes a batch of 32 tetrahedra; the batch's (m, n) items are sorted
-// into whole-tetrahedron and cut lists and carved 32 at a time, one item per lane, in warp-
-// uniform steps that emit at most one final tetrahedron per lane.  Each piece finds its box
-// and moments in its lane (one lane per moment index adds them to the box sums).  Pieces that
-// evaluate frequencies themselves (fine boxes, or no box) go to a per-warp ring queue that the
-// whole warp drains 32 pieces at a time: own series with lanes owning frequencies, then the
-// near-field (piece, frequency, term) entries of all of them packed one per lane; entries the
-// shared divided-difference table leaves go to a per-warp fallback buffer in global memory,
-// evaluated in full rounds when it fills.
-// Sums.  FP32 kernel: per-CTA sums in 64-bit fixed point (units of 2^-44) in shared memory,
-// added with integer atomics and written once per CTA: integer sums are exact in any order, so
-// the warps take batches from a launch-wide counter (balanced loads) and the results are
-// bitwise reproducible for any launch shape.  FP64 kernel: per-warp compensated FP64 sums per
-// batch, batches assigned statically (batch = warp + k * warps), every sum in a fixed order:
-// bitwise reproducible for a given launch shape.
+// Work layout.  Frequencies are sorted by |w| once per pass (k_box_setup), so that the
+// frequencies a piece evaluates are index ranges.  A warp takes a run of 2^tlog tetrahedra; its
+// (m, n) items are whole or cut by band index alone and carved 32 pieces at a time, one final
+// tetrahedron per lane, as in the static weights (chi0_static.cu).  Each piece finds its box and
+// adds its moments in its lane.  Pieces that evaluate frequencies themselves go to a per-warp ring
+// queue that the whole warp drains DC pieces at a time: each lane finds one piece's frequency
+// ranges and own moments, then all (piece, frequency, term) pairs of the drain are evaluated packed,
+// one per lane, first the own-moment pairs, then the near ones.  Near pairs that the shared
+// divided-difference table leaves go to a per-warp fallback buffer in global memory, evaluated in
+// full rounds when it fills.
+// Sums.  FP32 kernel: per-CTA sums in 64-bit fixed point (units of 2^-44) in shared memory, added
+// with integer atomics and written once per CTA: integer sums are exact in any order, so the warps
+// take units from a launch-wide counter and the results are bitwise reproducible for any launch
+// shape.  FP64 kernel: units assigned statically (unit = warp + k * warps); Re and Im in per-warp
+// compensated FP64 sums, box moments added to a row of the warp's own in global memory (one
+// reduction per moment, in the warp's order; 26 KB of shared memory per warp for them had kept an
+// SM at four warps): bitwise reproducible for a given launch shape.
+//
+// Bound: instruction issue and dependent latency (FP32: 12 warps per SM, 1.6 instructions per
+// cycle), the FP64 pipe (FP64: 74% busy while an SM has work).  Measured per 256-frequency pass,
+// before (one (piece, frequency range) at a time, 64-bit float conversions and atomics, batches of
+// 32 tetrahedra) and now: 64 x 64 x 16 mesh, 10 bands FP32 10.5 -> 7.0 ms, 32^3, 80 bands FP32 836
+// -> 590 ms; 16 x 16 x 8, 10 bands, 128 frequencies FP64 58-100 -> 13 ms; Im alone, 32^3, 12 bands
+// FP32 3.3 -> 0.8 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -63,23 +73,21 @@ using namespace chi0dev;
 namespace chi0int {
 namespace {
 
-using grid::div_small;
 using grid::kFull;
+using grid::quick_div;
 using grid::tet_corners;
 
 constexpr int kNWPass = 256;   // frequencies per dynamic pass
 // FP32 kernel: sums in 64-bit fixed point, units of 2^-44 (exact and order-independent; every
 // per-CTA total stays far below 2^19, and one rounding of 2^-45 per term is far below the
 // FP32 terms' own error)
-constexpr float kFxScale = 17592186044416.0f;  // 2^44
 constexpr double kFxUnit = 1.0 / 17592186044416.0;
-constexpr int kNearCap = 1024;  // near-field (piece, frequency, term) entries listed per warp
 constexpr int kFbCap = 4096;   // near-field entries left to the per-vertex table, per warp
-static_assert(kFbCap >= 4 * kNearCap, "the fallback buffer holds several near lists' leftovers");
-static_assert(kNearCap >= 4 * kNWPass, "the near list keeps room for two pieces' entries");
+constexpr int kQC = 64;        // queue of final tetrahedra that evaluate frequencies themselves
+constexpr int kCodes = 128;    // listed pieces of cut items per warp: < 32 left over + 3 x 32
 
 // a near-field entry the shared table leaves: knots x (sorted), values f, weight v, and
-// code = frequency index << 2 | term << 1 | (w < 0)
+// code = frequency index << 1 | term
 template <typename T> struct FbEnt {
   T x[4], f[4], v;
   int code;
@@ -88,60 +96,107 @@ template <typename T> struct FbEnt {
 template <bool FP64> struct DynShape {
   static constexpr int threads = FP64 ? 64 : 128;
   static constexpr int warps = threads / 32;
+  static constexpr int minb = FP64 ? 4 : 3;
   static constexpr int DC = FP64 ? 16 : 32;  // queued pieces evaluated per round
-  static constexpr int KM = FP64 ? 64 : 32;  // own far-field moments kept per queued piece
-  static constexpr int NF = FP64 ? 3 : 2;    // a fine box stands in beyond NF radii
-  static constexpr int KF = FP64 ? 28 : 24;  // moments of a fine box   (truncation NF^-KF)
-  static constexpr int KG = FP64 ? 22 : 12;  // moments of a geometric box ((2/9)^KG)
+  static constexpr double far = FP64 ? 1.5 : 2.0;  // a box or a piece's own moments stand in from here on (radii)
+  static constexpr int KF = FP64 ? 40 : 20;  // moments of a fine box (z <= 1/far)
+  static constexpr int KO = FP64 ? 40 : 32;  // own moments of a queued piece, at most
+  static constexpr int KG = FP64 ? 18 : 12;  // moments of a geometric box (z <= 2/9)
+  static constexpr int KW = FP64 ? 32 : 20;  // moments of a wide box (z <= 5/9)
 };
+template <bool FP64> constexpr bool poly_ok(double tol) {
+  using S = DynShape<FP64>;
+  return mean_err(1.0 / S::far, S::KF) <= tol && mean_err(2.0 / 9.0, S::KG) <= tol && mean_err(5.0 / 9.0, S::KW) <= tol;
+}
+static_assert(poly_ok<false>(2.5e-9) && poly_ok<true>(1e-16), "too few moments");
+// The boxes' moments carry Taylor's coefficients (6 k!/(k+4)! with the sign of (-1)^k), and
+// p_k (-1)^k is applied in FP64 where the boxes are evaluated: rounding it to FP32 in every moment
+// would be a bias common to all pieces.  An FP64 piece's own moments carry the polynomial's.
+__constant__ constexpr ChebInv<double, DynShape<true>::KO> kOwn(1.0 / DynShape<true>::far);
+template <bool FP64> struct BoxPoly {
+  using S = DynShape<FP64>;
+  double v[S::KF + S::KG + S::KW];
+  constexpr BoxPoly() : v() {
+    const ChebInv<double, S::KF> f(1.0 / S::far);
+    const ChebInv<double, S::KG> g(2.0 / 9.0);
+    const ChebInv<double, S::KW> w(5.0 / 9.0);
+    for (int k = 0; k < S::KF; ++k) v[k] = (k & 1) ? -f.p_[k] : f.p_[k];
+    for (int k = 0; k < S::KG; ++k) v[S::KF + k] = (k & 1) ? -g.p_[k] : g.p_[k];
+    for (int k = 0; k < S::KW; ++k) v[S::KF + S::KG + k] = (k & 1) ? -w.p_[k] : w.p_[k];
+  }
+};
+__constant__ constexpr BoxPoly<false> kBoxPolyF{};
+__constant__ constexpr BoxPoly<true> kBoxPolyD{};
 
 // box geometry
 constexpr int kBoxL = 4;      // fine levels
 constexpr int kBoxJ0 = 32;    // finest boxes across [0, u_max]
 constexpr int kBoxExtra = 6;  // fine boxes per level past u_max
 constexpr int kBoxG = 40;     // geometric boxes (x_0 1.25^40 = 7500 x_0)
+constexpr int kBoxW = 24;     // wide boxes (x_0 1.25^24 = 212 x_0)
 constexpr int kMinBoxNw = 8;  // fewer frequencies: every piece evaluates all of them
 __host__ __device__ constexpr int box_J(int l) { return (kBoxJ0 >> l) + kBoxExtra; }
 constexpr int kBoxFine = box_J(0) + box_J(1) + box_J(2) + box_J(3);
-constexpr int kBoxes = kBoxFine + kBoxG;
+constexpr int kBoxes = kBoxFine + kBoxG + kBoxW;
 template <bool FP64> __host__ __device__ constexpr int box_slots() {
-  return kBoxFine * DynShape<FP64>::KF + kBoxG * DynShape<FP64>::KG;
+  return kBoxFine * DynShape<FP64>::KF + kBoxG * DynShape<FP64>::KG + kBoxW * DynShape<FP64>::KW;
+}
+template <bool FP64> __host__ __device__ constexpr int box_terms(int b) {
+  return b < kBoxFine ? DynShape<FP64>::KF : (b < kBoxFine + kBoxG ? DynShape<FP64>::KG : DynShape<FP64>::KW);
 }
 template <bool FP64> __host__ __device__ constexpr int slot_base(int b) {
-  return b < kBoxFine ? b * DynShape<FP64>::KF
-                      : kBoxFine * DynShape<FP64>::KF + (b - kBoxFine) * DynShape<FP64>::KG;
+  using S = DynShape<FP64>;
+  return b < kBoxFine ? b * S::KF
+                      : (b < kBoxFine + kBoxG ? kBoxFine * S::KF + (b - kBoxFine) * S::KG
+                                              : kBoxFine * S::KF + kBoxG * S::KG + (b - kBoxFine - kBoxG) * S::KW);
 }
 
-// the pass's boxes in the kernels' precision (written by k_box_setup, read by both kernels)
+// the pass's boxes and its frequencies in ascending |w|, in the kernels' precision (written by
+// k_box_setup)
 template <typename T> struct BoxTab {
   T C[kBoxes], R[kBoxes];  // centre and radius
   T lowG[kBoxG + 1];       // lower edges x_b of the geometric boxes (x = c - u_max)
   T W0, x0, umax;
   int on;
+  T om[kNWPass];      // |w| ascending
+  T oml[kNWPass];     // |w| - (T)|w|
+  short rank[kNWPass];  // place of frequency i in that order
 };
 
 template <typename T> __device__ __forceinline__ void kadd_t(T &sum, T &comp, T x) {
   const T t = sum + x;
-  if (tabs(sum) >= tabs(x)) comp += (sum - t) + x;
-  else comp += (x - t) + sum;
+  const bool big = Mean<T>::bits(sum) >= Mean<T>::bits(x);
+  const T a = big ? sum : x, b = big ? x : sum;
+  comp += (a - t) + b;
   sum = t;
 }
 
-// one block: u_max of the pass and the box table
+// one block: the sorted frequencies, u_max of the pass and the box table (boxes = 0: none)
 template <typename T>
-__global__ void __launch_bounds__(256) k_box_setup(const double *__restrict__ omega, int nw, BoxTab<T> *tab) {
+__global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict__ omega, int nw, int boxes,
+                                                       BoxTab<T> *tab) {
   __shared__ double red[8];
-  double u = 0.0;
-  for (int i = threadIdx.x; i < nw; i += blockDim.x) u = fmax(u, fabs(omega[i]));
+  __shared__ unsigned long long key[kNWPass];
+  const int i = threadIdx.x;
+  const double a = i < nw ? fabs(omega[i]) : 0.0;
+  key[i] = (unsigned long long)__double_as_longlong(a);  // ascends with a; a NaN comes last
+  double u = a;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) u = fmax(u, __shfl_xor_sync(kFull, u, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = u;
+  if ((i & 31) == 0) red[i >> 5] = u;
   __syncthreads();
+  if (i < nw) {
+    int r = 0;
+    for (int j = 0; j < nw; ++j) r += key[j] < key[i] || (key[j] == key[i] && j < i);
+    tab->rank[i] = (short)r;
+    tab->om[r] = (T)a;
+    tab->oml[r] = (T)(a - (double)(T)a);
+  }
   double umax = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) umax = fmax(umax, red[i]);
+  for (int k = 0; k < kNWPass / 32; ++k) umax = fmax(umax, red[k]);
   const T W0 = (T)(umax / kBoxJ0), um = (T)umax, x0 = W0 * T(5);
-  const int on = (nw >= kMinBoxNw && umax > 1e-30 && umax < 1e30 && W0 > T(0)) ? 1 : 0;
-  if (threadIdx.x == 0) {
+  const int on = (boxes && nw >= kMinBoxNw && umax > 1e-30 && umax < 1e30 && W0 > T(0)) ? 1 : 0;
+  if (i == 0) {
     tab->W0 = W0;
     tab->x0 = x0;
     tab->umax = um;
@@ -153,20 +208,20 @@ __global__ void __launch_bounds__(256) k_box_setup(const double *__restrict__ om
     }
   }
   __syncthreads();
-  const int b = threadIdx.x;
-  if (b < kBoxFine) {
-    int l = 0, j = b;
+  if (i < kBoxFine) {
+    int l = 0, j = i;
     while (j >= box_J(l)) {
       j -= box_J(l);
       ++l;
     }
     const T w = W0 * (T)(1 << l);
-    tab->C[b] = ((T)j + T(0.5)) * w;
-    tab->R[b] = w;
-  } else if (b < kBoxes) {
-    const T xb = tab->lowG[b - kBoxFine];
-    tab->C[b] = um + xb * T(1.125);
-    tab->R[b] = xb * T(0.25);
+    tab->C[i] = ((T)j + T(0.5)) * w;
+    tab->R[i] = w;
+  } else if (i < kBoxes) {
+    const bool wide = i >= kBoxFine + kBoxG;
+    const T xb = tab->lowG[i - kBoxFine - (wide ? kBoxG : 0)];
+    tab->C[i] = um + xb * T(1.125);
+    tab->R[i] = xb * (wide ? T(0.625) : T(0.25));
   }
 }
 
@@ -174,12 +229,17 @@ __global__ void __launch_bounds__(256) k_box_setup(const double *__restrict__ om
 template <typename T> __device__ __forceinline__ int box_of(T c, T s, const BoxTab<T> &tb) {
   if (!tb.on) return -1;
   const T x = c - tb.umax;
+  int wide = -1;
   if (x >= tb.x0) {
-    int b = (int)(__log2f((float)quot(x, tb.x0)) * 3.1062837f);  // log base 1.25 (a first guess)
+    int b = (int)(__log2f(__fdividef((float)x, (float)tb.x0)) * 3.1062837f);  // log base 1.25 (a first guess)
     b = b < 0 ? 0 : (b > kBoxG - 1 ? kBoxG - 1 : b);
     while (b > 0 && x < tb.lowG[b]) --b;
     while (b < kBoxG - 1 && x >= tb.lowG[b + 1]) ++b;
-    if (x >= tb.lowG[b] && x < tb.lowG[b + 1] && s <= T(0.125) * tb.lowG[b]) return kBoxFine + b;
+    const T lo = tb.lowG[b];
+    if (x >= lo && x < tb.lowG[b + 1]) {
+      if (s <= T(0.125) * lo) return kBoxFine + b;
+      if (b < kBoxW && s <= T(0.5) * lo) wide = kBoxFine + kBoxG + b;
+    }
   }
   T w = tb.W0;
   int off = 0;
@@ -187,75 +247,121 @@ template <typename T> __device__ __forceinline__ int box_of(T c, T s, const BoxT
   for (int l = 0; l < kBoxL; ++l) {
     if (s <= T(0.5) * w) {
       const T jf = floor(quot(c, w));
-      return jf < (T)box_J(l) ? off + (int)jf : -1;
+      return jf < (T)box_J(l) ? off + (int)jf : wide;
     }
     off += box_J(l);
     w *= T(2);
   }
-  return -1;
+  return wide;
 }
 
-// moments m_k = v 6 k!/(k+4)! sum_j f_j h_k(e, e_j), k < K, of a piece about a box (e = (d - C)/R)
-template <typename T> __device__ __noinline__ void box_moments_ol(const T e[4], const T f[4], T v, T *m, int K) {
-  T H[4] = {T(1), T(1), T(1), T(1)};
-  T P[4] = {T(1), T(1), T(1), T(1)};
-  m[0] = v * T(0.25) * (f[0] + f[1] + f[2] + f[3]);
-  for (int k = 1; k < K; ++k) {
+// s_k = [z^k] N(z)/Q(z)^2 of a piece, one after the other (k = 0, 1, ...): Q in the quadratic
+// factors of the end and of the middle knots, two divisions by each
+template <typename T> struct Moments {
+  T A, B, C, D;        // 1 - A z + B z^2 (e_0, e_3), 1 - C z + D z^2 (e_1, e_2)
+  T n[4];
+  T x1, x2, y1, y2, u1, u2, v1, v2;  // the stages' last two values
+  __device__ __forceinline__ Moments(const T e[4], const T f[4]) {
+    A = e[0] + e[3];
+    B = e[0] * e[3];
+    C = e[1] + e[2];
+    D = e[1] * e[2];
+    const T E1 = A + C, E2 = (B + D) + A * C, E3 = B * C + D * A;
+    const T g0 = f[0] * e[0], g1 = f[1] * e[1], g2 = f[2] * e[2], g3 = f[3] * e[3];
+    const T h0 = g0 * e[0], h1 = g1 * e[1], h2 = g2 * e[2], h3 = g3 * e[3];
+    const T m0 = (f[0] + f[1]) + (f[2] + f[3]), m1 = (g0 + g1) + (g2 + g3), m2 = (h0 + h1) + (h2 + h3);
+    const T m3 = (h0 * e[0] + h1 * e[1]) + (h2 * e[2] + h3 * e[3]);
+    n[0] = m0;
+    n[1] = m1 - E1 * m0;
+    n[2] = m2 + (E2 * m0 - E1 * m1);
+    n[3] = m3 + (E2 * m1 - E1 * m2) - E3 * m0;
+    x1 = x2 = y1 = y2 = u1 = u2 = v1 = v2 = T(0);
+  }
+  __device__ __forceinline__ T next(T in) {
+    const T x = in + (A * x1 - B * x2);
+    const T y = x + (A * y1 - B * y2);
+    const T u = y + (C * u1 - D * u2);
+    const T v = u + (C * v1 - D * v2);
+    x2 = x1, x1 = x;
+    y2 = y1, y1 = y;
+    u2 = u1, u1 = u;
+    v2 = v1, v1 = v;
+    return v;
+  }
+};
+
+// The same s_k (k = 1, 2, ...) by the complete homogeneous polynomials h_k(e_1..e_4, e_j) of every
+// vertex: the FP32 kernel's form.  Thirteen operations a moment instead of eight, but shorter
+// chains and fewer registers: the 64 x 64 x 16 pass takes 6.8 ms with it, 7.4 ms with Moments.
+template <typename T> struct MomentsH {
+  T e[4], f[4], H[4], P[4];
+  __device__ __forceinline__ MomentsH(const T e_[4], const T f_[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      e[i] = e_[i];
+      f[i] = f_[i];
+      H[i] = P[i] = T(1);
+    }
+  }
+  __device__ __forceinline__ T next() {
     H[0] = e[0] * H[0];
 #pragma unroll
     for (int l = 1; l < 4; ++l) H[l] = H[l - 1] + e[l] * H[l];
-    T sj = T(0);
+    T s = T(0);
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      P[jj] = H[3] + e[jj] * P[jj];
-      sj += f[jj] * P[jj];
+    for (int j = 0; j < 4; ++j) {
+      P[j] = H[3] + e[j] * P[j];
+      s += f[j] * P[j];
     }
-    m[k] = v * tabs(series_coef<T>(k)) * sj;
+    return s;
   }
+};
+
+// v as 64-bit fixed point (units of 2^-44, round to nearest even): the same integer as
+// __float2ll_rn(v 2^44), from two 32-bit conversions (the 64-bit conversion runs at the FP64 rate,
+// 16 cycles of the SM per warp; these take 4)
+__device__ __forceinline__ long long fx_of(float v) {
+  const float xs = v * 262144.0f;  // 2^18
+  if (!(fabsf(xs) < 1.0e9f)) return __float2ll_rn(v * 17592186044416.0f);
+  const int h = __float2int_rn(xs);
+  const int l = __float2int_rn((xs - (float)h) * 67108864.0f);  // exact difference, 2^26
+  return ((long long)h << 26) + (long long)l;
+}
+// a 64-bit sum in shared memory as two 32-bit words (native 32-bit atomics; the 64-bit add of shared
+// memory took 17 to 42 cycles of the SM per warp, by how many lanes shared an address)
+__device__ __forceinline__ void fx_add(unsigned *lo, unsigned *hi, int i, float v) {
+  const long long t = fx_of(v);
+  if (t == 0) return;
+  const unsigned l = (unsigned)t;
+  const unsigned old = atomicAdd(&lo[i], l);
+  atomicAdd(&hi[i], (unsigned)((unsigned long long)t >> 32) + (old + l < old ? 1u : 0u));
 }
 
-// the same moments added straight into fixed-point box sums dst[0..K) (shared-memory atomics)
-__device__ __forceinline__ void box_moments_fx(const float e[4], const float f[4], float v, unsigned long long *dst,
-                                               int K) {
-  float H[4] = {1.f, 1.f, 1.f, 1.f};
-  float P[4] = {1.f, 1.f, 1.f, 1.f};
-  // (terms that round to 0 in fixed point are skipped: high moments of small pieces)
-  long long t0 = __float2ll_rn(v * 0.25f * (f[0] + f[1] + f[2] + f[3]) * kFxScale);
-  if (t0) atomicAdd(&dst[0], (unsigned long long)t0);
-#pragma unroll 1
-  for (int k = 1; k < K; ++k) {
-    H[0] = e[0] * H[0];
-#pragma unroll
-    for (int l = 1; l < 4; ++l) H[l] = H[l - 1] + e[l] * H[l];
-    float sj = 0.f;
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      P[jj] = H[3] + e[jj] * P[jj];
-      sj += f[jj] * P[jj];
-    }
-    const long long t = __float2ll_rn(v * tabs(series_coef<float>(k)) * sj * kFxScale);
-    if (t) atomicAdd(&dst[k], (unsigned long long)t);
-  }
-}
-
-// Out-of-line copy of the fallback's delta term: inlined copies of the helpers at several call
-// sites made the kernel's body overflow the instruction cache (ncu: 45% of the issue stalls
-// waiting for instructions).  Helpers with one call site (the near drain's divided-difference
-// table and de Boor recursion, the own and the box moments) are inlined there: 8% and 3%
-// faster than calling them.
+// Out-of-line copy of the fallback's delta term (rare: kept out of the hot code's instruction cache)
 template <typename T> __device__ __noinline__ T delta_sum_ol(const T d[4], const T f[4]) { return delta_sum(d, f, T(0)); }
 
+// the delta term of a near pair: FP64 by the plane section; FP32 by the cubic recursion, whose
+// rounding (a relative 2.9e-8 common to every piece, from its 4/3) its results have always carried
+__device__ __forceinline__ double delta_term(const double x[4], const double e[4], const double f[4]) {
+  return delta_section(x, e, f);
+}
+__device__ __forceinline__ float delta_term(const float x[4], const float e[4], const float f[4]) {
+  const float rs[6] = {rcp(e[1] - e[0]), rcp(e[2] - e[1]), rcp(e[3] - e[2]),
+                       rcp(e[2] - e[0]), rcp(e[3] - e[1]), rcp(e[3] - e[0])};
+  return delta_sum_pre(x, f, rs);
+}
+
 // does box b stand in for term (0: 1/(D - u), 1: 1/(D + u)) at frequency u = om?  Fine boxes
-// only near themselves; geometric boxes always.  Same expression in both kernels.
+// only near themselves; the others always.  Same expression in all kernels.
 template <typename T> __device__ __forceinline__ bool box_far(T C, T R, int b, T om, int term) {
   if (b >= kBoxFine) return true;
-  const T r2 = R * T(DynShape<sizeof(T) == 8>::NF);
+  const T r2 = R * T(DynShape<sizeof(T) == 8>::far);
   if (term) return !(C + om < r2);
   return !(tabs(C - om) < r2);
 }
 
 // sum_j f_j (1/V) int lambda_j / X for knots x of X near 0: divided-difference table (principal
-// value across X = 0); one out-of-line copy shared by every call site
+// value across X = 0); one out-of-line copy
 template <bool FP64>
 __device__ __noinline__ typename std::conditional<FP64, double, float>::type near_term(
     const typename std::conditional<FP64, double, float>::type *x,
@@ -289,167 +395,128 @@ __device__ __forceinline__ float near_shift(float D0h, float D0l, float wh, floa
 }
 __device__ __forceinline__ double near_shift(double D0h, double, double wh, double) { return D0h - wh; }
 
-// knots of near-field entry ent (= 2 * frequency index + term) of a piece with knots
-// d = D0 + e (sorted), D0 = D0h + D0l: term 0 is 1/(D - |w|) with knots (D0 - |w|) + e, term 1
-// is 1/(D + |w|) with knots d + |w|
-template <bool FP64, typename T>
-__device__ __forceinline__ void near_knots(int ent, const T d[4], const T e[4], T D0h, T D0l, const T *s_w,
-                                           const T *s_wl, T x[4], bool &neg) {
-  const int iw = ent >> 1, sgn = ent & 1;
-  const T w = s_w[iw];
-  neg = w < T(0);
-  const T om = neg ? -w : w;
-  if (sgn) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = d[i] + om;
-  } else {
-    const T sh = near_shift(D0h, D0l, om, FP64 ? T(0) : (neg ? -s_wl[iw] : s_wl[iw]));
-#pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = sh + e[i];
+// first index of the ascending om[0..n) with om[i] > v (strict) or >= v
+template <bool STRICT, typename T> __device__ __forceinline__ int first_above(const T *om, int n, T v) {
+  int a = 0, z = n;
+  while (a < z) {
+    const int mid = (a + z) >> 1;
+    if (STRICT ? om[mid] > v : om[mid] >= v) z = mid;
+    else a = mid + 1;
   }
+  return a;
 }
 
-// IMO: Im only (the delta term of Eq. 2 on an ascending grid of w >= 0; no principal value,
-// no boxes) for the Kramers-Kronig route to Re
+// a queued piece's frequency ranges (indices of the sorted frequencies): the - term from f0 to f1,
+// its near part n0 to n1; the + term up to p1, its near part up to np
+struct Range {
+  short f0, n0, n1, f1, np, p1;
+};
+
+// IMO: Im only (the delta term of Eq. 2; no principal value, no boxes) for the Kramers-Kronig route
 template <bool FP64, bool IMO = false>
-__global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
-    k_dynamic(Grid g, Tet tet, const void *__restrict__ Ek, const void *__restrict__ Ekq, Q q,
-              const void *__restrict__ W2, int cma, float tau, const short *__restrict__ occ,
-              const short *__restrict__ empq, const double *__restrict__ omega, int nw, DynBufs db,
-              const float *__restrict__ Eklo, const float *__restrict__ Ekqlo,
-              unsigned long long *__restrict__ counters) {
+__global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
+    k_dynamic(const __grid_constant__ DynArgs A, int nw, int tlog) {
   using T = typename std::conditional<FP64, double, float>::type;
   using S = DynShape<FP64>;
-  constexpr int W = S::warps, KM = S::KM, KF = S::KF, KG = S::KG, DC = S::DC;
-  constexpr int QC = 64;  // queue of final tetrahedra that evaluate frequencies themselves
+  constexpr int W = S::warps, KO = S::KO, DC = S::DC;
   constexpr int NS = box_slots<FP64>();
-  // per-piece strides of the scratch: odd (conflict-free lane-parallel writes), except the FP32
-  // own moments, even so that the own series reads them in aligned pairs (2-way write conflicts)
-  constexpr int SKM = FP64 ? KM + 1 : KM + 2, SKF = KF + 1;
-  constexpr int KU = DC * SKM > 32 * SKF ? DC * SKM : 32 * SKF;  // per-warp scratch (T elements)
-  static_assert(QC >= DC + 32, "one carving step adds at most 32 queued pieces");
-  __shared__ int s_c[W][32][4], s_cq[W][32][4];
-  __shared__ T s_vol[W][32];
-  __shared__ int s_nlo[W][32], s_nn[W][32], s_pre[W][33];
-  __shared__ int s_list[W][2][64], s_nl[W][2];  // item lists (whole / cut): l << 24 | m << 12 | n
-  // scratch: box moments of one carving step's pieces (32 x KF), or the own far-field moments
-  // of the queued pieces being evaluated (DC x KM)
-  __shared__ T s_scr[W][KU];
-  __shared__ int s_pk[W][DC];
-  // ring queue: offsets e from D0 (sorted), values f, (weight, D0h, D0l), box
-  __shared__ __align__(16) T s_qe[W][QC][4];
-  __shared__ __align__(16) T s_qf[W][QC][4];
-  __shared__ T s_qv[W][QC][3];
-  __shared__ int s_qb[W][QC];
-  // FP64 kernel: per-warp compensated sums of the batch (static batch order); FP32 kernel:
-  // per-CTA fixed-point sums of the whole launch (s_fx; batches in any order)
+  constexpr int SK = KO + 2;  // own moments per queued piece (even: read in aligned pairs)
+  static_assert(kQC >= DC + 32, "one carving step adds at most 32 queued pieces");
   constexpr bool FX = !FP64;
+  __shared__ int4 s_ck[W][32], s_cq[W][32];
+  __shared__ T s_vol[W][32];
+  __shared__ int s_pw[W][33], s_pc[W][33];               // prefix sums: whole items, cut items
+  __shared__ int s_wm[W][32], s_wn[W][32], s_nn[W][32];  // whole columns m, whole and all rows n
+  __shared__ int s_code[W][kCodes];                      // l << 24 | (m - lo) << 12 | (n - lo)
+  __shared__ unsigned char s_sub[W][kCodes];             // first-cut piece << 6 | second-cut piece << 4 | mask
+  __shared__ unsigned s_rec[64];
+  __shared__ __align__(16) T s_mom[IMO ? 1 : W][IMO ? 1 : DC][IMO ? 1 : SK];  // own moments of the drain's pieces
+  __shared__ unsigned char s_mk[W][DC];  // their count (FP32)
+  // ring queue: offsets e from D0 (sorted), values f, (weight, D0h, D0l), box
+  __shared__ __align__(16) T s_qe[W][kQC][4];
+  __shared__ __align__(16) T s_qf[W][kQC][4];
+  __shared__ T s_qv[W][kQC][3];
+  __shared__ short s_qb[W][kQC];
+  __shared__ Range s_rg[W][DC];
+  __shared__ int s_po[W][DC + 1], s_pn[W][DC + 1];  // prefix sums: own pairs, near pairs
+  // FP64 kernel: per-warp compensated sums; FP32 kernel: per-CTA fixed-point sums (two words)
   constexpr int WA = FX ? 1 : W, NA = FX ? 1 : kNWPass;
-  __shared__ T sR[WA][NA], sI[WA][NA];
-  __shared__ T cR[WA][NA], cI[WA][NA];  // compensation terms
-  __shared__ unsigned long long s_fx[FX ? 2 : 1][FX ? kNWPass : 1];
-  __shared__ T s_w[kNWPass];
-  __shared__ T s_wl[FP64 ? 1 : kNWPass];  // FP32 path: w - (float)w
-  // near-field entries of the drain's pieces: ring slot << 9 | 2 * frequency index + term
-  __shared__ unsigned short s_near[W][kNearCap];
-  __shared__ short s_rng[kBoxFine][2];  // frequencies a fine box leaves to its pieces: [lo, hi)
+  __shared__ T sR[WA][IMO ? 1 : NA], sI[WA][NA];
+  __shared__ T cR[WA][IMO ? 1 : NA], cI[WA][NA];  // compensation terms
+  __shared__ unsigned s_fxl[FX ? 2 * kNWPass : 1], s_fxh[FX ? 2 * kNWPass : 1];
+  __shared__ T s_w[kNWPass];                 // |w| ascending
+  __shared__ T s_wl[FP64 ? 1 : kNWPass];     // FP32 path: |w| - (float)|w|
+  __shared__ short s_rng[kBoxFine][3];  // frequencies a fine box leaves to its pieces: - term [lo, hi), + term [0, p)
   __shared__ BoxTab<T> s_tab;
-  extern __shared__ __align__(16) unsigned char s_dyn[];  // box sums: [W][NS] (FP64), [NS] fixed point
+  extern __shared__ __align__(16) unsigned char s_dyn[];  // FP32: box sums, low and high words [NS]
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
-  T *acc = (T *)s_dyn + (size_t)wib * NS;
-  unsigned long long *bfx = (unsigned long long *)s_dyn;
-  T *scr = s_scr[wib];
-  const int w = q.hi - q.lo;
-  const long long nbatch = (g.ntet + 31) / 32;
+  unsigned *bl = (unsigned *)s_dyn, *bh = bl + NS;
+  const Grid &g = A.g;
+  const Q &q = A.q;
+  const DynBufs &db = A.db;
+  const int lo = q.lo, w = q.hi - q.lo, nb = g.nb;
+  const T *W2 = (const T *)A.W2;
+  const long long units = (g.ntet + (1LL << tlog) - 1) >> tlog;
   const long long gwarp = (long long)blockIdx.x * W + wib, nwarps = (long long)gridDim.x * W;
-  double *gpart = db.box_part + gwarp * NS;
+  double *gbox = db.box_part + gwarp * NS;  // FP64: the warp's box moments
   FbEnt<T> *gfb = (FbEnt<T> *)db.fb + gwarp * kFbCap;
-#pragma unroll 1
-  for (int iw = threadIdx.x; iw < nw; iw += blockDim.x) {
-    s_w[iw] = (T)omega[iw];
-    if constexpr (!FP64) s_wl[iw] = (float)(omega[iw] - (double)s_w[iw]);
-  }
   {
-    if constexpr (IMO) {
-      if (threadIdx.x == 0) s_tab.on = 0;  // every piece evaluates its own frequencies
-    } else {
-      const BoxTab<T> *src = (const BoxTab<T> *)db.box_tab;
-      const int nwords = (int)(sizeof(BoxTab<T>) / 4);
+    const BoxTab<T> *src = (const BoxTab<T> *)db.box_tab;
+    constexpr int nwords = (int)(offsetof(BoxTab<T>, om) / 4);
 #pragma unroll 1
-      for (int i = threadIdx.x; i < nwords; i += blockDim.x) ((int *)&s_tab)[i] = ((const int *)src)[i];
+    for (int i = threadIdx.x; i < nwords; i += blockDim.x) ((int *)&s_tab)[i] = ((const int *)src)[i];
+#pragma unroll 1
+    for (int i = threadIdx.x; i < nw; i += blockDim.x) {
+      s_w[i] = src->om[i];
+      if constexpr (!FP64) s_wl[i] = src->oml[i];
     }
   }
+  for (int i = threadIdx.x; i < 64; i += blockDim.x) s_rec[i] = kCutTab.v[i];
   if constexpr (FX) {
     if constexpr (!IMO) {
 #pragma unroll 1
-      for (int i = threadIdx.x; i < NS; i += blockDim.x) bfx[i] = 0ull;
+      for (int i = threadIdx.x; i < 2 * NS; i += blockDim.x) bl[i] = 0u;
     }
 #pragma unroll 1
-    for (int i = threadIdx.x; i < 2 * kNWPass; i += blockDim.x) s_fx[i / kNWPass][i % kNWPass] = 0ull;
+    for (int i = threadIdx.x; i < 2 * kNWPass; i += blockDim.x) s_fxl[i] = s_fxh[i] = 0u;
   } else {
 #pragma unroll 1
-    for (int i = lane; i < (IMO ? 0 : NS); i += 32) acc[i] = T(0);
+    for (int i = lane; i < nw; i += 32) {
+      if constexpr (!IMO) sR[wib][i] = cR[wib][i] = T(0);
+      sI[wib][i] = cI[wib][i] = T(0);
+    }
   }
   __syncthreads();
-  // frequency ranges of the fine boxes: contiguous when |w| ascends along the grid (an
-  // interval for the - term, a prefix for the + term); otherwise the whole grid, the
-  // predicate deciding each frequency
-  bool sorted = true;
+  if constexpr (!IMO) {
 #pragma unroll 1
-  for (int i = threadIdx.x; i + 1 < nw; i += blockDim.x) sorted = sorted && tabs(s_w[i]) <= tabs(s_w[i + 1]);
-  sorted = __syncthreads_and(sorted) != 0;
-#pragma unroll 1
-  for (int b = threadIdx.x; b < (IMO ? 0 : kBoxFine); b += blockDim.x) {
-    int lo = 0, hi = nw;
-    if (sorted) {
-      lo = nw;
-      hi = 0;
+    for (int b = threadIdx.x; b < kBoxFine; b += blockDim.x) {
+      int a = nw, z = 0, p = 0;  // (intervals: |w| ascends)
 #pragma unroll 1
       for (int i = 0; i < nw; ++i) {
-        const T om = tabs(s_w[i]);
-        if (!box_far(s_tab.C[b], s_tab.R[b], b, om, 0) || !box_far(s_tab.C[b], s_tab.R[b], b, om, 1)) {
-          lo = lo < i ? lo : i;
-          hi = i + 1;
+        if (!box_far(s_tab.C[b], s_tab.R[b], b, s_w[i], 0)) {
+          a = a < i ? a : i;
+          z = i + 1;
         }
+        if (!box_far(s_tab.C[b], s_tab.R[b], b, s_w[i], 1)) p = i + 1;
       }
-      if (hi <= lo) lo = hi = 0;
+      s_rng[b][0] = (short)(z > a ? a : 0);
+      s_rng[b][1] = (short)(z > a ? z : 0);
+      s_rng[b][2] = (short)p;
     }
-    s_rng[b][0] = (short)lo;
-    s_rng[b][1] = (short)hi;
+    __syncthreads();
   }
-  __syncthreads();
-  const bool boxes = s_tab.on != 0;
+  const bool boxes = !IMO && s_tab.on != 0;
   int nfp64 = 0, npieces = 0, nboxed = 0;
   int qh = 0, qt = 0;  // ring queue head and tail (warp-uniform)
-  // one queued final tetrahedron (sorted offsets ee from D0 = D0h + D0l, values ff, weight vr,
-  // own far-field moments am[0..K)) on the frequencies its box (b >= 0) leaves to it, or on
-  // all of them (b < 0); lanes own frequencies
-  // one term of Re / Im at frequency iw
-  auto add_re = [&](int iw, T v) {
-    if constexpr (FX) {
-      const long long t = __float2ll_rn(v * kFxScale);
-      if (t) atomicAdd(&s_fx[0][iw], (unsigned long long)t);
-    } else {
-      kadd_t(sR[wib][iw], cR[wib][iw], v);
-    }
-  };
-  auto add_im = [&](int iw, T v) {
-    if constexpr (FX) {
-      const long long t = __float2ll_rn(v * kFxScale);
-      if (t) atomicAdd(&s_fx[1][iw], (unsigned long long)t);
-    } else {
-      kadd_t(sI[wib][iw], cI[wib][iw], v);
-    }
-  };
+  int nfb = 0;         // entries in the warp's fallback buffer (warp-uniform)
   // one round of per-lane results (iw < 0: nothing).  Fixed point: atomic adds (exact, any
-  // order).  FP64: lanes that share a frequency add one at a time in lane order (the lists are
-  // built in a fixed order, so the sums are reproducible), the others at once.
+  // order).  FP64: lanes that share a frequency add one at a time in lane order, the others at once.
   auto round_add = [&](int iw, T re, T im) {
     if constexpr (FX) {
       if (iw >= 0) {
-        if (re != T(0)) add_re(iw, re);
-        if (im != T(0)) add_im(iw, im);
+        if (!IMO && re != T(0)) fx_add(s_fxl, s_fxh, iw, re);
+        if (im != T(0)) fx_add(s_fxl + kNWPass, s_fxh + kNWPass, iw, im);
       }
     } else {
       const unsigned grp = __match_any_sync(kFull, iw >= 0 ? iw : -1 - lane);
@@ -458,25 +525,22 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
 #pragma unroll 1
       for (int r = 0; r <= nr; ++r) {
         if (iw >= 0 && rank == r) {
-          add_re(iw, re);
-          if (im != T(0)) add_im(iw, im);
+          if constexpr (!IMO) kadd_t(sR[wib][iw], cR[wib][iw], re);
+          if (im != T(0)) kadd_t(sI[wib][iw], cI[wib][iw], im);
         }
         __syncwarp();
       }
     }
   };
-  int nfb = 0;  // entries in the warp's fallback buffer
   // the fallback buffer: per-vertex table, one entry per lane and round (full rounds: the
-  // buffer collects the entries of many pieces).  Lanes that share a frequency add one at a
-  // time in lane order (the buffer's order is fixed, so the sums are reproducible), the others
-  // at once.
+  // buffer collects the entries of many pieces, in a fixed order)
   auto fallback_flush = [&]() {
     __syncwarp();
 #pragma unroll 1
     for (int base = 0; base < nfb; base += 32) {
       const int k = base + lane;
       T re = T(0), im = T(0);
-      int iw = -1 - lane;  // inactive lanes: keys of their own
+      int iw = -1;
       if (k < nfb) {
         const FbEnt<T> &o = gfb[k];
         T x[4], ff[4];
@@ -486,37 +550,136 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
           ff[i] = o.f[i];
         }
         const T vr = o.v;
-        const int code = o.code;
-        iw = code >> 2;
-        re = vr * near_term<FP64>(x, ff, tau, nfp64);
-        if ((code & 2) == 0 && x[0] < T(0) && x[3] > T(0)) {
-          im = vr * delta_sum_ol(x, ff) * T(3.141592653589793);
-          if (code & 1) im = -im;
-        }
+        iw = o.code >> 1;
+        re = vr * near_term<FP64>(x, ff, A.tau, nfp64);
+        if ((o.code & 1) == 0 && x[0] < T(0) && x[3] > T(0)) im = vr * delta_sum_ol(x, ff) * T(3.141592653589793);
       }
       round_add(iw, re, im);
     }
     nfb = 0;
+    __syncwarp();
   };
-  int nnear = 0;  // entries in the drain's near list
-  // the drain's near list: the shared divided-difference table, one entry per lane and round
-  // (the entries of all queued pieces packed together); lanes that share a frequency add one
-  // at a time in lane order (the list's order is fixed, so the sums are reproducible).  Entries
-  // the table leaves (three clustered knots, three zero knots) go, knots and all, to the
-  // fallback buffer (the caller keeps room for the whole list).
-  auto near_drain = [&]() {
+  // evaluates n <= DC queued pieces: ranges and own moments one piece per lane, then their
+  // (piece, frequency, term) pairs packed over the lanes
+  auto drain = [&](int n) {
+    int no = 0, nn = 0;
+    if (lane < n) {
+      const int sl = (qh + lane) % kQC;
+      const T D0h = s_qv[wib][sl][1];
+      const T e0 = s_qe[wib][sl][0], e3 = s_qe[wib][sl][3];
+      Range r;
+      if constexpr (IMO) {  // the frequencies inside the knots, one more on each side (the pair's own test decides)
+        const int a = first_above<true>(s_w, nw, D0h + e0), z = first_above<false>(s_w, nw, D0h + e3);
+        r = Range{0, (short)(a > 0 ? a - 1 : 0), (short)(z < nw ? z + 1 : nw), 0, 0, 0};
+        nn = r.n1 - r.n0;
+      } else {
+        const int b = s_qb[wib][sl];
+        const T half = (e3 - e0) * T(0.5), c = D0h + (e0 + e3) * T(0.5), near = half * T(S::far);
+        const int f0 = b >= 0 ? s_rng[b][0] : 0, f1 = b >= 0 ? s_rng[b][1] : nw, p1 = b >= 0 ? s_rng[b][2] : nw;
+        const int a = min(max(first_above<true>(s_w, nw, c - near), f0), f1);
+        const int z = max(min(first_above<false>(s_w, nw, c + near), f1), a);
+        const int p = p1 > 0 ? min(first_above<false>(s_w, nw, near - c), p1) : 0;
+        r = Range{(short)f0, (short)a, (short)z, (short)f1, (short)p, (short)p1};
+        nn = (z - a) + p;
+        no = (f1 - f0) - (z - a) + (p1 - p);
+        if (no > 0) {
+          T ff[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) ff[i] = s_qf[wib][sl][i];
+          if constexpr (FP64) {  // about the midpoint, offsets in units of the half-width
+            const T ri = half > T(0) ? rcp_nr(half) : T(0), mid = (e0 + e3) * T(0.5), vr = s_qv[wib][sl][0];
+            T e[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = (s_qe[wib][sl][i] - mid) * ri;
+            Moments<T> m(e, ff);
+            T *out = s_mom[wib][lane];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) out[k] = vr * kOwn.v[k] * m.next(m.n[k]);
+#pragma unroll 4
+            for (int k = 4; k < KO; ++k) out[k] = vr * kOwn.v[k] * m.next(T(0));
+          } else {  // in units of the midpoint, as many as the widest ratio needs
+            T d[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[i] = D0h + s_qe[wib][sl][i];
+            s_mk[wib][lane] = far_moments<T, KO>(d, ff, s_mom[wib][lane]);
+          }
+        }
+      }
+      s_rg[wib][lane] = r;
+    }
+    int po = no, pn = nn;  // inclusive prefix sums over the lanes
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(kFull, po, o), y = __shfl_up_sync(kFull, pn, o);
+      if (lane >= o) {
+        po += x;
+        pn += y;
+      }
+    }
+    if (lane < n) {
+      s_po[wib][lane + 1] = po;
+      s_pn[wib][lane + 1] = pn;
+    }
+    if (lane == 0) s_po[wib][0] = s_pn[wib][0] = 0;
+    const int own = __shfl_sync(kFull, po, 31), near = __shfl_sync(kFull, pn, 31);
+    __syncwarp();
+    if constexpr (!IMO) {
+      int p = 0;
 #pragma unroll 1
-    for (int base = 0; base < nnear; base += 32) {
-      const int k = base + lane;
+      for (int base = 0; base < own; base += 32) {  // warp-uniform
+        const int it = base + lane;
+        T v = T(0);
+        int iw = -1;
+        if (it < own) {
+          while (s_po[wib][p + 1] <= it) ++p;
+          const int sl = (qh + p) % kQC;
+          const Range r = s_rg[wib][p];
+          int k = it - s_po[wib][p];
+          const int k1 = r.n0 - r.f0, k2 = k1 + (r.f1 - r.n1);
+          const bool plus = k >= k2;
+          iw = k < k1 ? r.f0 + k : (plus ? r.np + (k - k2) : r.n1 + (k - k1));
+          const T e0 = s_qe[wib][sl][0], e3 = s_qe[wib][sl][3];
+          const T om = s_w[iw], c = s_qv[wib][sl][1] + (e0 + e3) * T(0.5);
+          const T *m = s_mom[wib][p];
+          if constexpr (FP64) {
+            const T rd = rcp_nr(plus ? c + om : c - om), z = (e3 - e0) * T(0.5) * rd, z2 = z * z;
+            // even and odd powers as two chains (the loop is bound by dependent latency)
+            const double2 m0 = *reinterpret_cast<const double2 *>(m + KO - 2);
+            T se = m0.x, so = m0.y;
+#pragma unroll 4
+            for (int j = KO - 4; j >= 0; j -= 2) {
+              const double2 mj = *reinterpret_cast<const double2 *>(m + j);
+              so = so * z2 + mj.y;
+              se = se * z2 + mj.x;
+            }
+            v = (se + z * so) * rd;
+          } else {
+            v = s_qv[wib][sl][0] * far_eval_k(m, s_mk[wib][p], c, plus ? -om : om);
+          }
+        }
+        round_add(iw, v, T(0));
+      }
+    }
+    // near pairs: the shared divided-difference table and the delta term.  Pairs the table leaves
+    // (three clustered knots, three zero knots) go, knots and all, to the fallback buffer.
+    int p = 0;
+#pragma unroll 1
+    for (int base = 0; base < near; base += 32) {  // warp-uniform
+      if (!IMO && nfb > kFbCap - 32) fallback_flush();
+      const int it = base + lane;
       T re = T(0), im = T(0), x[4], ff[4], vr = T(0);
-      int iw = -1 - lane, ent = 0;  // inactive lanes: keys of their own
-      bool left = false, neg = false;
-      if (k < nnear) {
-        const int code = s_near[wib][k], sl = code >> 9;
-        ent = code & 511;
-        T ee[4], d[4];
+      int iw = -1, code = 0;
+      bool left = false;
+      if (it < near) {
+        while (s_pn[wib][p + 1] <= it) ++p;
+        const int sl = (qh + p) % kQC;
+        const Range r = s_rg[wib][p];
+        const int k = it - s_pn[wib][p], k1 = r.n1 - r.n0;
+        const bool plus = k >= k1;
+        const int jw = plus ? k - k1 : r.n0 + k;
         const T D0h = s_qv[wib][sl][1], D0l = s_qv[wib][sl][2];
         vr = s_qv[wib][sl][0];
+        T ee[4];
         if constexpr (FP64) {
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -529,205 +692,112 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
           ee[0] = e4.x, ee[1] = e4.y, ee[2] = e4.z, ee[3] = e4.w;
           ff[0] = f4.x, ff[1] = f4.y, ff[2] = f4.z, ff[3] = f4.w;
         }
+        // - term: knots (D0 - |w|) + e; + term: knots d + |w|
+        const T om = s_w[jw];
+        if (plus) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = D0h + ee[i];
-        near_knots<FP64>(ent, d, ee, D0h, D0l, s_w, s_wl, x, neg);
-        // (a near entry has the frequency within two half-widths of the piece's midpoint,
-        // where the moment series about the knot midpoint does not apply)
-        T v;
-        if constexpr (IMO) {  // the delta term alone
-          if (x[0] < T(0) && x[3] > T(0)) {
-            iw = ent >> 1;
-            const T rs[6] = {rcp(ee[1] - ee[0]), rcp(ee[2] - ee[1]), rcp(ee[3] - ee[2]),
-                             rcp(ee[2] - ee[0]), rcp(ee[3] - ee[1]), rcp(ee[3] - ee[0])};
-            im = vr * delta_sum_pre(x, ff, rs) * T(3.141592653589793);
-          }
-        } else if (inv_sum_shared(x, ff, v)) {
-          iw = ent >> 1;
-          re = vr * v;
-          if ((ent & 1) == 0 && x[0] < T(0) && x[3] > T(0)) {
-            // reciprocal knot spans 01, 12, 23, 02, 13, 03 for the de Boor recursion (from the
-            // unshifted offsets: nonnegative terms, no cancellation)
-            const T rs[6] = {rcp(ee[1] - ee[0]), rcp(ee[2] - ee[1]), rcp(ee[3] - ee[2]),
-                             rcp(ee[2] - ee[0]), rcp(ee[3] - ee[1]), rcp(ee[3] - ee[0])};
-            im = vr * delta_sum_pre(x, ff, rs) * T(3.141592653589793);
-            if (neg) im = -im;
+          for (int i = 0; i < 4; ++i) x[i] = (D0h + ee[i]) + om;
+        } else {
+          const T sh = near_shift(D0h, D0l, om, FP64 ? T(0) : s_wl[FP64 ? 0 : jw]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i] = sh + ee[i];
+        }
+        const bool in = !plus && x[0] < T(0) && x[3] > T(0);
+        code = (jw << 1) | (plus ? 1 : 0);
+        if constexpr (IMO) {
+          if (in) {
+            iw = jw;
+            im = vr * delta_term(x, ee, ff) * T(3.141592653589793);
           }
         } else {
-          left = true;
+          T v;
+          if (inv_sum_shared(x, ff, v)) {
+            iw = jw;
+            re = vr * v;
+            if (in) im = vr * delta_term(x, ee, ff) * T(3.141592653589793);
+          } else {
+            left = true;
+          }
         }
       }
       round_add(iw, re, im);
-      const unsigned bal = __ballot_sync(kFull, left);
-      if (bal) {  // warp-uniform
-        if (left) {
-          FbEnt<T> &o = gfb[nfb + __popc(bal & lt)];
+      if constexpr (!IMO) {
+        const unsigned bal = __ballot_sync(kFull, left);
+        if (bal) {  // warp-uniform
+          if (left) {
+            FbEnt<T> &o = gfb[nfb + __popc(bal & lt)];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            o.x[i] = x[i];
-            o.f[i] = ff[i];
+            for (int i = 0; i < 4; ++i) {
+              o.x[i] = x[i];
+              o.f[i] = ff[i];
+            }
+            o.v = vr;
+            o.code = code;
           }
-          o.v = vr;
-          o.code = ((ent >> 1) << 2) | ((ent & 1) << 1) | (neg ? 1 : 0);
-        }
-        nfb += __popc(bal);
-        __syncwarp();
-      }
-    }
-    nnear = 0;
-  };
-  auto eval_piece = [&](const T ee[4], const T ff[4], T vr, T D0h, T D0l, const T *am, int K, int b, int slot) {
-    if constexpr (IMO) {
-      // the grid frequencies inside the knot range (ascending grid: one index range, widened
-      // by one on each side; the delta term's own test decides each entry)
-      const T lo_d = D0h + ee[0], hi_d = D0h + ee[3];
-      int a = 0, z = nw;  // first index with w > lo_d
-#pragma unroll 1
-      while (a < z) {
-        const int mid = (a + z) >> 1;
-        if (s_w[mid] > lo_d) z = mid;
-        else a = mid + 1;
-      }
-      int c = a, e = nw;  // first index with w >= hi_d
-#pragma unroll 1
-      while (c < e) {
-        const int mid = (c + e) >> 1;
-        if (s_w[mid] >= hi_d) e = mid;
-        else c = mid + 1;
-      }
-      const int lo = a > 0 ? a - 1 : 0, hi = c < nw ? c + 1 : nw;
-#pragma unroll 1
-      for (int iw = lo + lane; iw < hi; iw += 32) s_near[wib][nnear + iw - lo] = (unsigned short)((slot << 9) | (iw * 2));
-      nnear += hi - lo;
-      __syncwarp();
-    } else {
-      T d[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) d[i] = D0h + ee[i];
-      const T c = D0h + (ee[0] + ee[3]) * T(0.5), half = (ee[3] - ee[0]) * T(0.5);
-      const T Cb = b >= 0 ? s_tab.C[b] : T(0), Rb = b >= 0 ? s_tab.R[b] : T(0);
-      const int lo = b >= 0 ? s_rng[b][0] : 0, hi = b >= 0 ? s_rng[b][1] : nw;
-      // far field for both terms (Horner on the moments); near-field frequencies are
-      // recorded per lane (bit it of nearm / nearp) and evaluated below in full warps
-      unsigned nearm = 0u, nearp = 0u;
-#pragma unroll 1
-      for (int iw = lo + lane, itn = 0; iw < hi; iw += 32, ++itn) {
-        const T om = s_w[iw] < T(0) ? -s_w[iw] : s_w[iw];
-        T re = T(0);
-        // (the + term is near only for boxes that reach below u = 0 + F R: most boxes skip it)
-        const int t_hi = (b >= 0 && !(Cb < Rb * T(DynShape<FP64>::NF))) ? 0 : 1;
-#pragma unroll 1
-        for (int t = t_hi; t >= 0; --t) {  // the + term (t = 1), then the - term
-          int kk = 0;  // own-series terms this lane needs for this term (0: none)
-          if (b < 0 || !box_far(Cb, Rb, b, om, t)) {
-            const T den = t ? c + om : c - om;
-            const T r = quot(half, den < T(0) ? -den : den);
-            if (r <= T(Num<T>::kappa_far)) kk = own_terms<T>(K, r);
-            else if (t) nearp |= 1u << itn;
-            else nearm |= 1u << itn;
-          }
-          // one trip count for the lanes of the warp (extra terms only add what lies below the
-          // truncation tolerance): a convergent loop
-          const int km = __reduce_max_sync(__activemask(), kk);
-          if (kk > 0) re += far_eval_k(am, km, c, t ? -om : om);
-        }
-        if (re != T(0)) add_re(iw, vr * re);
-      }
-      // near field: the (frequency, term) pairs go to the drain's near list (the caller keeps
-      // room for them)
-      const int nit = (hi - lo + 31) >> 5;
-#pragma unroll 1
-      for (int itn = 0; itn < nit; ++itn) {
-#pragma unroll
-        for (int sgn = 0; sgn < 2; ++sgn) {
-          const bool mine = ((sgn ? nearp : nearm) >> itn) & 1u;
-          const unsigned bal = __ballot_sync(kFull, mine);
-          if (mine) s_near[wib][nnear + __popc(bal & lt)] = (unsigned short)((slot << 9) | ((lo + itn * 32 + lane) * 2 + sgn));
-          nnear += __popc(bal);
+          nfb += __popc(bal);
         }
       }
-      __syncwarp();
-    }
-  };
-  // evaluates n <= DC queued pieces: own far-field moments one piece per lane, then each piece
-  // on its frequencies with the whole warp
-  auto drain = [&](int n) {
-    if (!IMO && lane < n) {
-      const int sl = (qh + lane) % QC;
-      T d[4], ff[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        d[i] = s_qv[wib][sl][1] + s_qe[wib][sl][i];
-        ff[i] = s_qf[wib][sl][i];
-      }
-      s_pk[wib][lane] = far_moments<T, KM>(d, ff, scr + lane * SKM);
-    }
-    __syncwarp();
-    // pieces one by one (p < n), the near list whenever it might not hold another piece's
-    // entries and after the last piece (p == n; one call site), with room for its leftovers
-#pragma unroll 1
-    for (int p = 0; p <= n; ++p) {
-      if (p == n ? nnear > 0 : nnear > kNearCap - 2 * kNWPass) {  // warp-uniform
-        if (nfb > kFbCap - kNearCap) fallback_flush();
-        near_drain();
-      }
-      if (p == n) break;
-      const int sl = (qh + p) % QC;
-      T ee[4], ff[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        ee[i] = s_qe[wib][sl][i];
-        ff[i] = s_qf[wib][sl][i];
-      }
-      eval_piece(ee, ff, s_qv[wib][sl][0], s_qv[wib][sl][1], s_qv[wib][sl][2], scr + p * SKM, s_pk[wib][p],
-                 s_qb[wib][sl], sl);
     }
     qh += n;
     __syncwarp();
   };
-  int dthr = DC;  // queued pieces that trigger a drain (1: drain them all; warp-uniform)
-  // one carving step: at most one final tetrahedron per lane (has).  Its box and moments, the
-  // box sums (one moment index per lane, pieces in lane order), and the queue for pieces that
-  // evaluate frequencies themselves.
-  auto piece = [&](bool has, T ee[4], T ff[4], T vr, T D0h, T D0l) {
+  // one carving step: at most one final tetrahedron per lane (has).  Its box and moments, and the
+  // queue for pieces that evaluate frequencies themselves.  last: the queue is emptied.
+  auto piece = [&](bool has, T ee[4], T ff[4], T vr, T D0h, T D0l, bool last) {
     int b = -1;
     if (has) {
       sort4(ee, ff);
       ++npieces;
       has = D0h + ee[3] > T(0);
     }
-    if (has) {
-      const T c = D0h + (ee[0] + ee[3]) * T(0.5), half = (ee[3] - ee[0]) * T(0.5);
-      b = boxes ? box_of(c, half, s_tab) : -1;
-      if (b >= 0) {
-        const T ri = rcp(s_tab.R[b]), base = (D0h - s_tab.C[b]) + D0l;
+    if (has && boxes) b = box_of(D0h + (ee[0] + ee[3]) * T(0.5), (ee[3] - ee[0]) * T(0.5), s_tab);
+    if constexpr (!IMO) {
+      const bool in = has && b >= 0;
+      if constexpr (FX) {
+        if (in) {
+          ++nboxed;
+          const T ri = rcp(s_tab.R[b]), base = (D0h - s_tab.C[b]) + D0l;
+          T e[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) e[i] = (base + ee[i]) * ri;
+          const int K = box_terms<FP64>(b), at = slot_base<FP64>(b);
+          fx_add(bl, bh, at, vr * T(0.25) * (ff[0] + ff[1] + ff[2] + ff[3]));
+          MomentsH<T> m(e, ff);
+#pragma unroll 2
+          for (int k = 1; k < K; ++k) fx_add(bl, bh, at + k, vr * series_coef<T>(k) * m.next());
+        }
+      } else if (__any_sync(kFull, in)) {
+        // lanes in the same box add one at a time, in lane order
+        const unsigned grp = __match_any_sync(kFull, in ? b : -1 - lane);
+        const int rank = __popc(grp & lt), nr = __reduce_max_sync(kFull, in ? rank : 0);
+        nboxed += in;
+        const int bb = in ? b : 0;
+        const T ri = rcp_nr(s_tab.R[bb]), base = D0h - s_tab.C[bb];
         T e[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) e[i] = (base + ee[i]) * ri;
-        if constexpr (FX) box_moments_fx(e, ff, vr, bfx + slot_base<FP64>(b), b < kBoxFine ? KF : KG);
-        else box_moments_ol(e, ff, vr, scr + lane * SKF, b < kBoxFine ? KF : KG);
-        ++nboxed;
-      }
-    }
-    if constexpr (!FX) {  // FP64 box sums: one moment index per lane, pieces in lane order
-      __syncwarp();
-      unsigned mask = __ballot_sync(kFull, has && b >= 0);
+        for (int i = 0; i < 4; ++i) e[i] = in ? (base + ee[i]) * ri : T(0);
+        const int K = in ? box_terms<FP64>(bb) : 0, Kmax = __reduce_max_sync(kFull, K);
+        double *out = gbox + slot_base<FP64>(bb);
+        Moments<T> m(e, ff);
+        T in4[4] = {m.n[0], m.n[1], m.n[2], m.n[3]};
 #pragma unroll 1
-      while (mask) {  // warp-uniform
-        const int p = __ffs(mask) - 1;
-        mask &= mask - 1u;
-        const int bp = __shfl_sync(kFull, b, p);
-        const int K = bp < kBoxFine ? KF : KG, base = slot_base<FP64>(bp);
+        for (int k = 0; k < Kmax; ++k) {
+          const T v = m.next(in4[0]);
+          in4[0] = in4[1], in4[1] = in4[2], in4[2] = in4[3], in4[3] = T(0);
+          const T t = k < K ? vr * series_coef<T>(k) * v : T(0);
 #pragma unroll 1
-        for (int k = lane; k < K; k += 32) acc[base + k] += scr[p * SKF + k];
+          for (int r = 0; r <= nr; ++r) {
+            if (k < K && rank == r) atomicAdd(out + k, t);
+            __syncwarp();
+          }
+        }
       }
     }
     // (Im only: pieces whose knot range meets the pass's frequencies)
-    const bool queue = has && b < kBoxFine &&
-                       (!IMO || (D0h + ee[3] > s_w[0] && D0h + ee[0] < s_w[nw - 1]));
+    const bool queue = has && (IMO ? (D0h + ee[3] > s_w[0] && D0h + ee[0] < s_w[nw - 1]) : b < kBoxFine);
     const unsigned qm = __ballot_sync(kFull, queue);
     if (queue) {
-      const int sl = (qt + __popc(qm & lt)) % QC;
+      const int sl = (qt + __popc(qm & lt)) % kQC;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         s_qe[wib][sl][i] = ee[i];
@@ -736,38 +806,40 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
       s_qv[wib][sl][0] = vr;
       s_qv[wib][sl][1] = D0h;
       s_qv[wib][sl][2] = D0l;
-      s_qb[wib][sl] = b;
+      s_qb[wib][sl] = (short)b;
     }
     qt += __popc(qm);
     __syncwarp();
-    while (qt - qh >= dthr) drain(qt - qh < DC ? qt - qh : DC);
+#pragma unroll 1
+    while (qt - qh >= (last ? 1 : DC)) drain(qt - qh < DC ? qt - qh : DC);
   };
-  // item data of (tetrahedron l of the batch, bands m, n): a = e^m_k - eF, D = D0 + e (e_0 = 0)
-  // and |M|^2 at the corners.  Mixed path: energies as FP32 hi + lo pairs, so that D0 (hi + lo)
-  // and the corner offsets e come out to full FP32 relative precision whatever the size of a, b
-  auto load_item = [&](int l, int m, int n, T a[4], T e[4], T f[4], T &D0h, T &D0l) {
+  // item data: a = e^m_k - eF, D = D0 + e (e_0 = 0) and |M|^2 at the corners.  Mixed path:
+  // energies as FP32 hi + lo pairs, so that D0 (hi + lo) and the corner offsets e come out to full
+  // FP32 relative precision whatever the size of a, b
+  auto load_item = [&](int l, int mo, int no, T a[4], T e[4], T &D0h, T &D0l) {
+    const int4 k4 = s_ck[wib][l], q4 = s_cq[wib][l];
+    const int ck[4] = {k4.x, k4.y, k4.z, k4.w}, cq[4] = {q4.x, q4.y, q4.z, q4.w};
     D0h = T(0);
     D0l = T(0);
     if constexpr (FP64) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int ck = s_c[wib][l][i], cq = s_cq[wib][l][i];
-        a[i] = ((const double *)Ek)[(long long)ck * g.nb + m] - g.ef;
-        e[i] = (((const double *)Ekq)[(long long)cq * g.nb + n] - g.ef) - a[i];
+        a[i] = ((const double *)A.Ek)[(long long)ck[i] * nb + lo + mo] - g.ef;
+        e[i] = (((const double *)A.Ekq)[(long long)cq[i] * nb + lo + no] - g.ef) - a[i];
       }
     } else {
-      float al[4], bh[4], bl[4];
+      float al[4], bh_[4], bl_[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const long long ik = (long long)s_c[wib][l][i] * g.nb + m, iq = (long long)s_cq[wib][l][i] * g.nb + n;
-        a[i] = ((const float *)Ek)[ik];
-        al[i] = Eklo[ik];
-        bh[i] = ((const float *)Ekq)[iq];
-        bl[i] = Ekqlo[iq];
+        const long long ik = (long long)ck[i] * nb + lo + mo, iq = (long long)cq[i] * nb + lo + no;
+        a[i] = ((const float *)A.Ek)[ik];
+        al[i] = A.Eklo[ik];
+        bh_[i] = ((const float *)A.Ekq)[iq];
+        bl_[i] = A.Ekqlo[iq];
       }
       float sv, tv;
-      two_diff(bh[0], a[0], sv, tv);
-      const float corr = tv + (bl[0] - al[0]);
+      two_diff(bh_[0], a[0], sv, tv);
+      const float corr = tv + (bl_[0] - al[0]);
       D0h = sv + corr;
       D0l = corr - (D0h - sv);
       e[0] = 0.0f;
@@ -775,93 +847,82 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
       for (int i = 1; i < 4; ++i) {
         float sa, ta, sb, tb;
         two_diff(a[i], a[0], sa, ta);
-        two_diff(bh[i], bh[0], sb, tb);
-        e[i] = (sb - sa) + ((tb - ta) + ((bl[i] - bl[0]) - (al[i] - al[0])));
+        two_diff(bh_[i], bh_[0], sb, tb);
+        e[i] = (sb - sa) + ((tb - ta) + ((bl_[i] - bl_[0]) - (al[i] - al[0])));
       }
     }
-    const T *W2t = (const T *)W2;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      f[i] = cma ? T(1) : W2t[((long long)s_c[wib][l][i] * w + (m - q.lo)) * w + (n - q.lo)];
   };
-  // up to 32 items, one per lane: both carvings of Sec. II as warp-uniform loops over the
-  // pieces of the first and second cut, one final tetrahedron per lane and step
-  // (force: at least one step, so that piece() runs and drains the queue)
-  auto carve_items = [&](bool has, int l, int m, int n, bool force) {
-    T a[4] = {T(0), T(0), T(0), T(0)}, e[4] = {T(0), T(0), T(0), T(0)}, f[4] = {T(0), T(0), T(0), T(0)};
-    T D0h = T(0), D0l = T(0);
-    if (has) load_item(l, m, n, a, e, f, D0h, D0l);
-    const T vol = has ? s_vol[wib][l] : T(0);
-    bool whole = false;
-    if (has) {
-      const T amax = fmax(fmax(a[0], a[1]), fmax(a[2], a[3]));
-      const T bmin = fmin(fmin(a[0] + D0h + e[0], a[1] + D0h + e[1]), fmin(a[2] + D0h + e[2], a[3] + D0h + e[3]));
-      whole = amax < T(0) && bmin > T(0);  // occupied at k and empty at k+q everywhere: no cut
-    }
-    // whole items emit their one piece at the first step
-    Vt<T> V[4];
+  auto load_f = [&](int l, int mo, int no, T f[4]) {
+    const int4 k4 = s_ck[wib][l];
+    const int ck[4] = {k4.x, k4.y, k4.z, k4.w};
+    const T *pw = W2 + (mo * w + no);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) V[i] = Vt<T>{a[i], e[i], f[i]};
-    const bool cut = has && !whole;
-    Vt<T> P0[4];
-    T r0 = T(0);
-    const int n1 = cut ? cut_piece<0>(V, 0, P0, r0) : 0;
-    const int n1max = max(__reduce_max_sync(kFull, whole ? 1 : n1), force ? 1 : 0);
-#pragma unroll 1
-    for (int i1 = 0; i1 < n1max; ++i1) {
-      Vt<T> P[4];
-      T r1 = T(0);
-      bool ok1 = false;
-      if (cut && i1 < n1) {
-        cut_piece<0>(V, i1, P, r1);
-        ok1 = r1 > T(0);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) P[i].a += D0h;  // second-cut key -(a + e) is now -b
-      }
-      int n2 = 0;
-      if (ok1) {
-        Vt<T> Qd[4];
-        T rd;
-        n2 = cut_piece<1>(P, 0, Qd, rd);
-      }
-      const int n2max = max(__reduce_max_sync(kFull, (whole && i1 == 0) ? 1 : n2), (force && i1 == 0) ? 1 : 0);
-#pragma unroll 1
-      for (int i2 = 0; i2 < n2max; ++i2) {
-        T ee[4], ff[4], vr = T(0);
-        bool okp = false;
-        if (whole) {
-          okp = i1 == 0 && i2 == 0;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            ee[i] = e[i];
-            ff[i] = f[i];
+    for (int i = 0; i < 4; ++i) f[i] = A.cma ? T(1) : pw[(long long)ck[i] * w * w];
+  };
+  // FP32: the vertices in ascending order of the key, as cut_piece takes them
+  auto sort_key = [&](T key[4], T x[4], T y[4]) {
+    if constexpr (!FP64) {
+      auto sw = [&](int i, int j) {
+        if (key[j] < key[i]) {
+          T t = key[i];
+          key[i] = key[j], key[j] = t;
+          t = x[i];
+          x[i] = x[j], x[j] = t;
+          if (y != x) {
+            t = y[i];
+            y[i] = y[j], y[j] = t;
           }
-          vr = vol;
-        } else if (ok1 && i2 < n2) {
-          Vt<T> Qv[4];
-          T r2 = T(0);
-          cut_piece<1>(P, i2, Qv, r2);
-          const T r = r1 * r2;
-          okp = r > T(0);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            ee[i] = Qv[i].D > -D0h ? Qv[i].D : -D0h;  // clamped to D >= 0
-            ff[i] = Qv[i].f;
-          }
-          vr = vol * r;
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) ee[i] = ff[i] = T(0);
         }
-        piece(okp, ee, ff, vr, D0h, D0l);
-      }
+      };
+      sw(0, 1);
+      sw(2, 3);
+      sw(0, 2);
+      sw(1, 3);
+      sw(1, 2);
     }
   };
-  bool first = true;  // this warp's first batch writes its box partials, later ones add to them
-  // batches: FP64 kernel in a fixed order per warp (batch = warp + k x warps: its FP64 sums are
-  // reproducible); FP32 kernel from a launch-wide counter (its sums are exact integers, whatever
-  // the order), which balances the warps' loads
-  auto next_batch = [&](long long cur) -> long long {
+  // a listed piece of a cut item (mask: the second cut's sides): offsets, values, volume ratio
+  auto cut_item = [&](unsigned cd, unsigned sub, T ee[4], T ff[4], T &vr, T &D0h, T &D0l) -> bool {
+    const int tl = (int)(cd >> 24), mo = (int)((cd >> 12) & 0xFFFu), no = (int)(cd & 0xFFFu);
+    T a[4], e[4], fv[4];
+    load_item(tl, mo, no, a, e, D0h, D0l);
+    load_f(tl, mo, no, fv);
+    sort_key(a, e, fv);
+    unsigned m = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m |= (is_neg(a[i]) ? 1u : 0u) << i;
+    T key[4], e1[4], f1[4], r = T(1);
+    unsigned rec = s_rec[m * 4 + (sub >> 6)];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T t = cut_frac(rec, k, a);
+      e1[k] = cut_mix(rec, k, e, t);
+      f1[k] = cut_mix(rec, k, fv, t);
+      key[k] = -((cut_used(rec, k) ? D0h : sel4(a, (rec >> (5 * k)) & 3u) + D0h) + e1[k]);
+      r *= cut_factor(rec, k, t);
+    }
+    e1[3] = sel4(e, (rec >> 15) & 3u);
+    f1[3] = sel4(fv, (rec >> 15) & 3u);
+    key[3] = -((sel4(a, (rec >> 15) & 3u) + D0h) + e1[3]);
+    sort_key(key, e1, f1);
+    rec = s_rec[(sub & 15u) * 4 + ((sub >> 4) & 3u)];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const T t = cut_frac(rec, k, key);
+      ee[k] = cut_mix(rec, k, e1, t);
+      ff[k] = cut_mix(rec, k, f1, t);
+      r *= cut_factor(rec, k, t);
+    }
+    ee[3] = sel4(e1, (rec >> 15) & 3u);
+    ff[3] = sel4(f1, (rec >> 15) & 3u);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ee[i] = ee[i] > -D0h ? ee[i] : -D0h;  // clamped to D >= 0
+    vr = s_vol[wib][tl] * r;
+    return r > T(0);
+  };
+  // units: FP64 kernel in a fixed order per warp; FP32 kernel from a launch-wide counter (its sums
+  // are exact integers, whatever the order), which balances the warps' loads
+  auto next_unit = [&](long long cur) -> long long {
     if constexpr (FX) {
       unsigned long long b = 0ull;
       if (lane == 0) b = atomicAdd(db.ctr, 1ull);
@@ -870,169 +931,188 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
       return cur < 0 ? gwarp : cur + nwarps;
     }
   };
-#pragma unroll 1
-  for (long long batch = next_batch(-1); batch < nbatch; batch = next_batch(batch)) {
-    if constexpr (!FX) {
-#pragma unroll 1
-      for (int iw = lane; iw < nw; iw += 32) {
-        sR[wib][iw] = T(0);
-        sI[wib][iw] = T(0);
-        cR[wib][iw] = T(0);
-        cI[wib][iw] = T(0);
-      }
-    }
-    const long long t = batch * 32 + lane;
-    int cnt = 0;
-    if (t < g.ntet) {
+  for (long long unit = next_unit(-1);; unit = next_unit(unit)) {
+    const bool end = unit >= units;  // (one more turn: empties the queue)
+    const long long t = (unit << tlog) + lane;
+    int cw = 0, cc = 0;
+    if (!end && lane < (1 << tlog) && t < g.ntet) {
       long long c[4], cq[4];
       double vol;
-      tet_corners(g, tet, q, t, c, cq, vol);
-      int mhi = 0, nlo = g.nb;
+      tet_corners(g, A.tet, q, t, c, cq, vol);
+      int mhi = 0, mf = nb, nlo = nb, nf = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        s_c[wib][lane][i] = (int)c[i];
-        s_cq[wib][lane][i] = (int)cq[i];
-        mhi = max(mhi, (int)occ[c[i]]);
-        nlo = min(nlo, (int)empq[cq[i]]);
+        mhi = max(mhi, (int)A.occ[c[i]]);
+        mf = min(mf, (int)A.occf[c[i]]);
+        nlo = min(nlo, (int)A.emp[cq[i]]);
+        nf = max(nf, (int)A.empf[cq[i]]);
       }
       mhi = min(mhi, q.hi);
-      nlo = max(nlo, q.lo);
-      const int nm = mhi - q.lo, nn = q.hi - nlo;
-      cnt = (nm > 0 && nn > 0) ? nm * nn : 0;
-      s_vol[wib][lane] = (T)vol;
-      s_nlo[wib][lane] = nlo;
-      s_nn[wib][lane] = nn;
+      nlo = max(nlo, lo);
+      const int nm = mhi - lo, nn = q.hi - nlo;
+      if (nm > 0 && nn > 0) {
+        const int wm = max(min(mf, mhi) - lo, 0), wn = max(q.hi - max(nf, nlo), 0);
+        cw = wm * wn;
+        cc = nm * nn - cw;
+        s_ck[wib][lane] = make_int4((int)c[0], (int)c[1], (int)c[2], (int)c[3]);
+        s_cq[wib][lane] = make_int4((int)cq[0], (int)cq[1], (int)cq[2], (int)cq[3]);
+        s_vol[wib][lane] = (T)vol;
+        s_wm[wib][lane] = wm;
+        s_wn[wib][lane] = wn;
+        s_nn[wib][lane] = nn;
+      }
     }
-    int pre = cnt;  // inclusive prefix sum over the lanes
+    int pw = cw, pc = cc;  // inclusive prefix sums over the lanes
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, pre, o);
-      if (lane >= o) pre += v;
-    }
-    s_pre[wib][lane + 1] = pre;
-    if (lane == 0) s_pre[wib][0] = 0;
-    const int total = __shfl_sync(kFull, pre, 31);
-    if (lane < 2) s_nl[wib][lane] = 0;
-    __syncwarp();
-    // Items are sorted into two per-warp lists, whole-tetrahedron items and items whose
-    // tetrahedron a Fermi surface cuts, and each list is carved 32 items at a time, so that the
-    // lanes of a warp mostly run the same path.
-    auto drain_items = [&](bool final) {
-      for (;;) {  // warp-uniform
-        const int nf = s_nl[wib][0], nc = s_nl[wib][1];
-        int which;
-        if (nf >= 32) which = 0;
-        else if (nc >= 32) which = 1;
-        else if (final && nf > 0) which = 0;
-        else if (final && nc > 0) which = 1;
-        else if (final && qt > qh) which = 2;  // the batch's last queued pieces
-        else break;
-        int take = 0, code = 0;
-        if (which < 2) {
-          const int cntl = which ? nc : nf;
-          take = cntl < 32 ? cntl : 32;
-          if (lane < take) code = s_list[wib][which][cntl - take + lane];
-          __syncwarp();
-          if (lane == 0) s_nl[wib][which] = cntl - take;
-          __syncwarp();
-        }
-        dthr = which == 2 ? 1 : DC;
-        const unsigned u = (unsigned)code;
-        carve_items(lane < take, (int)(u >> 24), (int)((u >> 12) & 0xFFFu), (int)(u & 0xFFFu), which == 2);
+      const int a = __shfl_up_sync(kFull, pw, o), b = __shfl_up_sync(kFull, pc, o);
+      if (lane >= o) {
+        pw += a;
+        pc += b;
       }
-      dthr = DC;
-    };
-    for (int base = 0;; base += 32) {  // warp-uniform; the pass after the last items drains
-      const bool last = base >= total;
-      const int it = base + lane;
-      int kind = -1, code = 0;  // 0: whole tetrahedron (likely), 1: cut, -1: nothing to do
-      if (it < total) {
-        int lo_ = 0, hi_ = 32;  // owner: largest l with s_pre[l] <= it
+    }
+    s_pw[wib][lane + 1] = pw;
+    s_pc[wib][lane + 1] = pc;
+    if (lane == 0) s_pw[wib][0] = s_pc[wib][0] = 0;
+    const int total_w = __shfl_sync(kFull, pw, 31), total_c = __shfl_sync(kFull, pc, 31);
+    __syncwarp();
+    // Rounds of 32 final tetrahedra: first the whole items, then the listed pieces of the cut ones
+    // (items are listed 32 at a time whenever fewer than 32 pieces wait); one call site of piece().
+    int lw = 0, lc = 0, base_w = 0, base_c = 0, nc = 0, i1 = 0, n1 = 0, n1max = 0;
+    unsigned m1 = 0u, eb = 0u;
+    int code = 0;
+    bool dpos = true;
+    T a1[4], e1[4], D1h = T(0);
 #pragma unroll
-        for (int step = 0; step < 5; ++step) {
-          const int mid = (lo_ + hi_) >> 1;
-          if (s_pre[wib][mid] <= it) lo_ = mid;
-          else hi_ = mid;
+    for (int i = 0; i < 4; ++i) a1[i] = e1[i] = T(0);
+#pragma unroll 1
+    for (;;) {  // warp-uniform
+      T ee[4], ff[4], vr = T(0), D0h = T(0), D0l = T(0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) ee[i] = ff[i] = T(0);
+      bool has = false, last = false;
+      if (base_w < total_w) {
+        const int it = base_w + lane;
+        base_w += 32;
+        has = it < total_w;
+        if (has) {
+          while (s_pw[wib][lw + 1] <= it) ++lw;  // the item's tetrahedron: items ascend per lane
+          const int wn = s_wn[wib][lw];
+          int no;
+          const int mo = quick_div(it - s_pw[wib][lw], wn, no);
+          no += w - wn;
+          has = !(q.gamma && mo == no);  // intraband at Gamma: replaced by the DOS limit
+          T a[4];
+          load_item(lw, mo, no, a, ee, D0h, D0l);
+          load_f(lw, mo, no, ff);
+          vr = s_vol[wib][lw];
         }
-        const int l = lo_;
-        const int loc = it - s_pre[wib][l];
-        const int nn = s_nn[wib][l];
-        const int mo = div_small(loc, nn, q.hi - q.lo);
-        const int m = q.lo + mo, n = s_nlo[wib][l] + (loc - mo * nn);
-        if (!(q.gamma && m == n)) {  // intraband at Gamma: replaced by the DOS limit
-          T amin = T(1e30), amax = T(-1e30), bmin = T(1e30), bmax = T(-1e30);
+      } else if (nc < 32 && (i1 < n1max || base_c < total_c)) {
+        // list pieces: of the current 32 cut items' next first-cut piece, or take the next items
+        if (i1 >= n1max) {
+          const int it = base_c + lane;
+          base_c += 32;
+          bool on = it < total_c;
+          n1 = 0;
+          if (on) {
+            while (s_pc[wib][lc + 1] <= it) ++lc;
+            const int wm = s_wm[wib][lc], wn = s_wn[wib][lc], nn = s_nn[wib][lc];
+            // rows m < wm hold nn - wn items each, the rows after them nn
+            const int loc = it - s_pc[wib][lc], first = wm * (nn - wn);
+            int mo, no;
+            if (loc < first) mo = quick_div(loc, nn - wn, no);
+            else mo = wm + quick_div(loc - first, nn, no);
+            no += w - nn;
+            if (!(q.gamma && mo == no)) {
+              code = (lc << 24) | (mo << 12) | no;
+              T D1l;
+              load_item(lc, mo, no, a1, e1, D1h, D1l);
+              sort_key(a1, e1, e1);
+              // sides of the vertices: occupied (a < 0), empty (a + D > 0); D > 0 everywhere puts
+              // every point of the first cut plane (b = D there) on the empty side
+              m1 = eb = 0u;
+              dpos = true;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            T a, b;
-            if constexpr (FP64) {
-              a = ((const double *)Ek)[(long long)s_c[wib][l][i] * g.nb + m] - g.ef;
-              b = ((const double *)Ekq)[(long long)s_cq[wib][l][i] * g.nb + n] - g.ef;
-            } else {
-              a = ((const float *)Ek)[(long long)s_c[wib][l][i] * g.nb + m];
-              b = ((const float *)Ekq)[(long long)s_cq[wib][l][i] * g.nb + n];
+              for (int i = 0; i < 4; ++i) {
+                m1 |= (is_neg(a1[i]) ? 1u : 0u) << i;
+                eb |= (is_neg(-((a1[i] + D1h) + e1[i])) ? 1u : 0u) << i;
+                dpos = dpos && is_neg(-(D1h + e1[i]));
+              }
+              n1 = cut_count(m1);
             }
-            amin = a < amin ? a : amin;
-            amax = a > amax ? a : amax;
-            bmin = b < bmin ? b : bmin;
-            bmax = b > bmax ? b : bmax;
           }
-          if (amin < T(0) && bmax > T(0)) {
-            kind = (amax < T(0) && bmin > T(0)) ? 0 : 1;
-            code = (l << 24) | (m << 12) | n;
-          }
+          i1 = 0;
+          n1max = __reduce_max_sync(kFull, n1);
         }
-      }
+        unsigned m2 = 0u;
+        if (i1 < n1) {
+          const unsigned rec = s_rec[m1 * 4 + i1];
+          if (dpos) {
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const unsigned bal = __ballot_sync(kFull, kind == k);
-        if (kind == k) s_list[wib][k][s_nl[wib][k] + __popc(bal & lt)] = code;
-        __syncwarp();
-        if (lane == 0) s_nl[wib][k] += __popc(bal);
-        __syncwarp();
-      }
-      drain_items(last);
-      if (last) break;
-    }
-    qh = qt = 0;  // (the last pass of drain_items emptied the queue)
-    if constexpr (!FX) {
-      if (nfb > 0) fallback_flush();  // warp-uniform
-      __syncwarp();
-#pragma unroll 1
-      for (int iw = lane; iw < nw; iw += 32) {
-        db.partR[batch * nw + iw] = (double)sR[wib][iw] + (double)cR[wib][iw];
-        db.partI[batch * nw + iw] = (double)sI[wib][iw] + (double)cI[wib][iw];
-      }
-      // this batch's box sums into the warp's FP64 partials (a fixed order: bitwise reproducible)
-      if (boxes) {
-#pragma unroll 1
-        for (int i = lane; i < NS; i += 32) {
-          const double v = (double)acc[i];
-          gpart[i] = first ? v : gpart[i] + v;
-          acc[i] = T(0);
+            for (int k = 0; k < 3; ++k) m2 |= (cut_used(rec, k) ? 1u : (eb >> ((rec >> (5 * k)) & 3u)) & 1u) << k;
+          } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              const T x = D1h + cut_mix(rec, k, e1, cut_frac(rec, k, a1));
+              m2 |= (cut_used(rec, k) ? (is_neg(-x) ? 1u : 0u) : (eb >> ((rec >> (5 * k)) & 3u)) & 1u) << k;
+            }
+          }
+          m2 |= ((eb >> ((rec >> 15) & 3u)) & 1u) << 3;
+          if constexpr (!FP64) m2 = (1u << __popc(m2)) - 1u;  // (evaluated in sorted order)
         }
+        const int n2 = cut_count(m2);
+#pragma unroll
+        for (int i2 = 0; i2 < 3; ++i2) {
+          const unsigned bal = __ballot_sync(kFull, i2 < n2);
+          if (i2 < n2) {
+            const int at = nc + __popc(bal & lt);
+            s_code[wib][at] = code;
+            s_sub[wib][at] = (unsigned char)((i1 << 6) | (i2 << 4) | m2);
+          }
+          nc += __popc(bal);
+        }
+        ++i1;
+        __syncwarp();
+        continue;
+      } else if (nc > 0) {
+        const int take = nc < 32 ? nc : 32;
+        nc -= take;
+        has = lane < take;
+        const unsigned cd = has ? (unsigned)s_code[wib][nc + lane] : 0u;
+        const unsigned sub = has ? s_sub[wib][nc + lane] : 0u;
+        __syncwarp();
+        if (has) has = cut_item(cd, sub, ee, ff, vr, D0h, D0l);
+      } else if (end && qt > qh) {
+        last = true;
+      } else {
+        break;
       }
+      piece(has, ee, ff, vr, D0h, D0l, last);
     }
-    first = false;
-    __syncwarp();
+    if (end) break;
   }
+  if (nfb > 0) fallback_flush();  // warp-uniform
   if constexpr (FX) {
-    // the warp's remaining fallback entries, then the CTA's fixed-point sums into its rows
-    if (nfb > 0) fallback_flush();  // warp-uniform
+    // the CTA's fixed-point sums into its rows
     __syncthreads();
     unsigned long long *row = db.fx + (size_t)blockIdx.x * 2 * kNWPass;
     unsigned long long *brow = (unsigned long long *)db.box_part + (size_t)blockIdx.x * NS;
 #pragma unroll 1
-    for (int i = threadIdx.x; i < 2 * kNWPass; i += blockDim.x) row[i] = s_fx[i / kNWPass][i % kNWPass];
+    for (int i = threadIdx.x; i < 2 * kNWPass; i += blockDim.x)
+      row[i] = ((unsigned long long)s_fxh[i] << 32) | s_fxl[i];
     if constexpr (!IMO) {
 #pragma unroll 1
-      for (int i = threadIdx.x; i < NS; i += blockDim.x) brow[i] = bfx[i];
+      for (int i = threadIdx.x; i < NS; i += blockDim.x) brow[i] = ((unsigned long long)bh[i] << 32) | bl[i];
     }
   } else {
-    if (boxes && first)  // a warp without batches
+    __syncwarp();
 #pragma unroll 1
-      for (int i = lane; i < NS; i += 32) gpart[i] = 0.0;
+    for (int iw = lane; iw < nw; iw += 32) {
+      if constexpr (!IMO) db.partR[gwarp * nw + iw] = (double)sR[wib][iw] + (double)cR[wib][iw];
+      db.partI[gwarp * nw + iw] = (double)sI[wib][iw] + (double)cI[wib][iw];
+    }
   }
-  if (counters) {
+  if (A.counters) {
     unsigned long long a = (unsigned long long)npieces, b = (unsigned long long)nfp64,
                        x = (unsigned long long)nboxed;
 #pragma unroll
@@ -1042,9 +1122,9 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
       x += __shfl_xor_sync(kFull, x, o);
     }
     if (lane == 0) {
-      atomicAdd(&counters[0], a);  // each lane counted its own pieces
-      atomicAdd(&counters[1], b);
-      atomicAdd(&counters[3], x);
+      atomicAdd(&A.counters[0], a);  // each lane counted its own pieces
+      atomicAdd(&A.counters[1], b);
+      atomicAdd(&A.counters[3], x);
     }
   }
 }
@@ -1054,77 +1134,150 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, FP64 ? 2 : 3)
 template <bool FP64>
 __global__ void __launch_bounds__(256) k_box_sum(const double *__restrict__ part, int nrows, double *__restrict__ tot) {
   constexpr int NS = box_slots<FP64>();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NS) return;
+  // 8 threads per slot, each a contiguous run of rows, added in run order
+  __shared__ double red[8][32];
+  const int i = blockIdx.x * 32 + (threadIdx.x & 31), run = threadIdx.x >> 5;
+  const int per = (nrows + 7) / 8, r0 = run * per, r1 = min(nrows, r0 + per);
   if constexpr (FP64) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int wv = 0;
-    for (; wv + 3 < nrows; wv += 4) {
-      s0 += part[(size_t)wv * NS + i];
-      s1 += part[(size_t)(wv + 1) * NS + i];
-      s2 += part[(size_t)(wv + 2) * NS + i];
-      s3 += part[(size_t)(wv + 3) * NS + i];
+    if (i < NS) {
+      int r = r0;
+      for (; r + 3 < r1; r += 4) {
+        s0 += part[(size_t)r * NS + i];
+        s1 += part[(size_t)(r + 1) * NS + i];
+        s2 += part[(size_t)(r + 2) * NS + i];
+        s3 += part[(size_t)(r + 3) * NS + i];
+      }
+      for (; r < r1; ++r) s0 += part[(size_t)r * NS + i];
     }
-    for (; wv < nrows; ++wv) s0 += part[(size_t)wv * NS + i];
-    tot[i] = (s0 + s1) + (s2 + s3);
+    red[run][threadIdx.x & 31] = (s0 + s1) + (s2 + s3);
+    __syncthreads();
+    if (run == 0 && i < NS) {
+      double s = 0.0;
+      for (int k = 0; k < 8; ++k) s += red[k][threadIdx.x];
+      tot[i] = s;
+    }
   } else {
     const unsigned long long *fx = (const unsigned long long *)part;
     unsigned long long a = 0ull;
-    for (int r = 0; r < nrows; ++r) a += fx[(size_t)r * NS + i];
-    tot[i] = (double)(long long)a * kFxUnit;
+    if (i < NS) {
+#pragma unroll 4
+      for (int r = r0; r < r1; ++r) a += fx[(size_t)r * NS + i];
+    }
+    red[run][threadIdx.x & 31] = __longlong_as_double((long long)a);
+    __syncthreads();
+    if (run == 0 && i < NS) {
+      a = 0ull;
+      for (int k = 0; k < 8; ++k) a += (unsigned long long)__double_as_longlong(red[k][threadIdx.x]);
+      tot[i] = (double)(long long)a * kFxUnit;
+    }
   }
 }
 
-// FP32 kernel: Re and Im per frequency from the CTAs' fixed-point rows (exact sums) into row 0
-// of the partials
-__global__ void __launch_bounds__(256) k_fx_rows(const unsigned long long *__restrict__ fx, int nrows, int nw,
-                                                 double *__restrict__ partR, double *__restrict__ partI) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 2 * nw) return;
-  const int term = i / nw, iw = i % nw;
-  unsigned long long a = 0ull;
-  for (int r = 0; r < nrows; ++r) a += fx[((size_t)r * 2 + term) * kNWPass + iw];
-  (term ? partI : partR)[iw] = (double)(long long)a * kFxUnit;
-}
-
-// far[iw]: the boxes' share of Re at frequency iw (FP64 evaluation of the multipoles); one
-// block per frequency, fixed-order reduction
+// One block per frequency iw (caller's order): the weight launch's sums of its sorted place and the
+// boxes' share of Re (FP64 evaluation of the multipoles), normalised, into re[iw] and im[iw].
+// FP32 kernel: rows are CTAs' fixed-point sums (added exactly); FP64: per-warp partials.
 template <bool FP64>
-__global__ void __launch_bounds__(128) k_box_eval(const double *__restrict__ omega, const void *__restrict__ tabp,
-                                                  const double *__restrict__ tot, double *__restrict__ far) {
+__global__ void __launch_bounds__(128) k_dyn_out(const double *__restrict__ omega, int nw, const void *__restrict__ tabp,
+                                                 const double *__restrict__ tot, DynBufs db, int nrows, double scale,
+                                                 const double *__restrict__ dos, int ndos, double *__restrict__ re,
+                                                 double *__restrict__ im) {
   using T = typename std::conditional<FP64, double, float>::type;
   using S = DynShape<FP64>;
   const BoxTab<T> &tb = *(const BoxTab<T> *)tabp;
   const int iw = blockIdx.x;
-  const double u = fabs(omega[iw]);
-  const T wT = (T)omega[iw];
-  const T om = wT < T(0) ? -wT : wT;
-  double v = 0.0;
-  if (tb.on) {
+  const double wv = omega[iw], u = fabs(wv);
+  const int rk = tb.rank[iw];
+  const T om = tb.om[rk];
+  double v = 0.0, vi = 0.0;
+  unsigned long long ar = 0ull, ai = 0ull;
+  if constexpr (FP64) {
+    for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
+      if (re) v += db.partR[(size_t)r * nw + rk];
+      vi += db.partI[(size_t)r * nw + rk];
+    }
+  } else {
+    for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
+      ar += db.fx[(size_t)r * 2 * kNWPass + rk];
+      ai += db.fx[((size_t)r * 2 + 1) * kNWPass + rk];
+    }
+  }
+  if (re && tb.on) {
     for (int b = threadIdx.x; b < kBoxes; b += blockDim.x) {
-      const int K = b < kBoxFine ? S::KF : S::KG;
+      const int K = box_terms<FP64>(b);
       const double *M = tot + slot_base<FP64>(b);
+      const double *P = (FP64 ? kBoxPolyD.v : kBoxPolyF.v) +
+                        (b < kBoxFine ? 0 : (b < kBoxFine + kBoxG ? S::KF : S::KF + S::KG));
       const double C = (double)tb.C[b], R = (double)tb.R[b];
       for (int term = 0; term < 2; ++term) {
         if (!box_far(tb.C[b], tb.R[b], b, om, term)) continue;
         const double den = term ? C + u : C - u;
-        const double mz = -R / den;
-        double s = M[K - 1];
-        for (int k = K - 2; k >= 0; --k) s = s * mz + M[k];
+        const double z = R / den;
+        double s = P[K - 1] * M[K - 1];
+        for (int k = K - 2; k >= 0; --k) s = s * z + P[k] * M[k];
         v += s / den;
       }
     }
   }
-  __shared__ double red[4];
+  if (re && dos && wv == 0.0)
+    for (int i = threadIdx.x; i < ndos; i += blockDim.x) v += dos[i];
+  __shared__ double red[2][4];
+  __shared__ unsigned long long rad[2][4];
   v = grid::warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  vi = grid::warp_sum(vi);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ar += __shfl_xor_sync(kFull, ar, o);
+    ai += __shfl_xor_sync(kFull, ai, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = v;
+    red[1][threadIdx.x >> 5] = vi;
+    rad[0][threadIdx.x >> 5] = ar;
+    rad[1][threadIdx.x >> 5] = ai;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) far[iw] = (red[0] + red[1]) + (red[2] + red[3]);
+  if (threadIdx.x == 0) {
+    v = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
+    vi = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+    if constexpr (!FP64) {
+      v += (double)(long long)(rad[0][0] + rad[0][1] + rad[0][2] + rad[0][3]) * kFxUnit;
+      vi = (double)(long long)(rad[1][0] + rad[1][1] + rad[1][2] + rad[1][3]) * kFxUnit;
+    }
+    if (re) re[iw] = scale * v;
+    im[iw] = wv < 0.0 ? -scale * vi : scale * vi;
+  }
 }
 
-template <bool FP64> size_t dyn_smem() {
-  return FP64 ? (size_t)DynShape<FP64>::warps * box_slots<FP64>() * sizeof(double)
-              : (size_t)box_slots<FP64>() * sizeof(unsigned long long);
+template <bool FP64> size_t dyn_smem() { return FP64 ? 0 : (size_t)box_slots<FP64>() * 2 * sizeof(unsigned); }
+
+// Tetrahedra per unit (as log2): 32 at most, fewer on small meshes or wide windows, as long as a
+// unit keeps items (about a quarter of the window's pairs per tetrahedron) for full rounds of 32.
+// FP64 units are assigned statically: a few per warp even them out.
+int dyn_unit_log2(long long ntet, int w, bool fp64) {
+  int t = 5;
+  const long long ww = (long long)w * w, want = fp64 ? 4864 : 20480, least = fp64 ? 256 : 1024;
+  while (t > 0 && (ntet >> t) < want && (ww << t) > least) --t;
+  return t;
+}
+
+template <bool FP64, bool IMO>
+cudaError_t launch_weights(const DynArgs &a, const double *omega, int nw, int nblocks, double scale, const double *dos,
+                           int ndos, double *re, double *im, cudaStream_t s) {
+  using T = typename std::conditional<FP64, double, float>::type;
+  const DynBufs &db = a.db;
+  constexpr int NS = box_slots<FP64>();
+  const int rows = FP64 ? nblocks * DynShape<FP64>::warps : nblocks;
+  cudaError_t e = cudaSuccess;
+  if (!FP64) e = cudaMemsetAsync(db.ctr, 0, sizeof(unsigned long long), s);
+  else if (!IMO) e = cudaMemsetAsync(db.box_part, 0, sizeof(double) * (size_t)rows * NS, s);
+  if (e != cudaSuccess) return e;
+  k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, (BoxTab<T> *)db.box_tab);
+  k_dynamic<FP64, IMO><<<nblocks, DynShape<FP64>::threads, IMO ? 0 : dyn_smem<FP64>(), s>>>(
+      a, nw, dyn_unit_log2(a.g.ntet, a.q.hi - a.q.lo, FP64));
+  if (!IMO) k_box_sum<FP64><<<(NS + 31) / 32, 256, 0, s>>>(db.box_part, rows, db.box_tot);
+  k_dyn_out<FP64><<<nw, 128, 0, s>>>(omega, nw, db.box_tab, db.box_tot, db, rows, scale, dos, ndos, IMO ? nullptr : re, im);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1141,66 +1294,23 @@ size_t dynamic_box_tab_bytes() {
 }
 
 cudaError_t dynamic_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(k_dynamic<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)dyn_smem<true>());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_dynamic<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)dyn_smem<false>());
+  return cudaFuncSetAttribute(k_dynamic<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn_smem<false>());
 }
 
-cudaError_t launch_dynamic(const Grid &g, const Tet &tet, const void *Ek, const void *Ekq, const Q &q,
-                           const void *W2, int cma, int fp64, float tau, const short *occ, const short *empq,
-                           const double *omega, int nw, const DynBufs &db, int nblocks,
-                           unsigned long long *counters, cudaStream_t s, const float *Eklo,
-                           const float *Ekqlo, int *rows) {
+// Re and Im (im_only: Im alone, for the Kramers-Kronig route) of one q and nw <= dynamic_max_nw()
+// frequencies into re[nw], im[nw]
+cudaError_t launch_dynamic(const DynArgs &a, int fp64, int im_only, const double *omega, int nw, int nblocks,
+                           double scale, const double *dos, int ndos, double *re, double *im, cudaStream_t s) {
+  const DynBufs &db = a.db;
   if (nw > kNWPass || nw <= 0 || nblocks <= 0) return cudaErrorInvalidValue;
-  if (!fp64 && (!Eklo || !Ekqlo)) return cudaErrorInvalidValue;
-  if (!db.box_tab || !db.box_part || !db.box_tot || !db.far || !db.fb || !db.fx || !db.ctr)
+  if (!fp64 && (!a.Eklo || !a.Ekqlo)) return cudaErrorInvalidValue;
+  if (!db.box_tab || !db.box_part || !db.box_tot || !db.fb || !db.fx || !db.ctr || !db.partR || !db.partI)
     return cudaErrorInvalidValue;
-  if (fp64) {
-    const int nwarps = nblocks * DynShape<true>::warps;
-    k_box_setup<double><<<1, 256, 0, s>>>(omega, nw, (BoxTab<double> *)db.box_tab);
-    k_dynamic<true><<<nblocks, DynShape<true>::threads, dyn_smem<true>(), s>>>(
-        g, tet, Ek, Ekq, q, W2, cma, tau, occ, empq, omega, nw, db, Eklo, Ekqlo, counters);
-    k_box_sum<true><<<(box_slots<true>() + 255) / 256, 256, 0, s>>>(db.box_part, nwarps, db.box_tot);
-    k_box_eval<true><<<nw, 128, 0, s>>>(omega, db.box_tab, db.box_tot, db.far);
-    *rows = (int)((g.ntet + 31) / 32);
-  } else {
-    cudaError_t e = cudaMemsetAsync(db.ctr, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    k_box_setup<float><<<1, 256, 0, s>>>(omega, nw, (BoxTab<float> *)db.box_tab);
-    k_dynamic<false><<<nblocks, DynShape<false>::threads, dyn_smem<false>(), s>>>(
-        g, tet, Ek, Ekq, q, W2, cma, tau, occ, empq, omega, nw, db, Eklo, Ekqlo, counters);
-    k_box_sum<false><<<(box_slots<false>() + 255) / 256, 256, 0, s>>>(db.box_part, nblocks, db.box_tot);
-    k_box_eval<false><<<nw, 128, 0, s>>>(omega, db.box_tab, db.box_tot, db.far);
-    k_fx_rows<<<(2 * nw + 255) / 256, 256, 0, s>>>(db.fx, nblocks, nw, db.partR, db.partI);
-    *rows = 1;
-  }
-  return cudaGetLastError();
-}
-
-// Im only (the Kramers-Kronig route): the delta term on an ascending grid of w >= 0
-cudaError_t launch_dynamic_im(const Grid &g, const Tet &tet, const void *Ek, const void *Ekq, const Q &q,
-                              const void *W2, int cma, int fp64, float tau, const short *occ, const short *empq,
-                              const double *omega, int nw, const DynBufs &db, int nblocks,
-                              unsigned long long *counters, cudaStream_t s, const float *Eklo,
-                              const float *Ekqlo, int *rows) {
-  if (nw > kNWPass || nw <= 0 || nblocks <= 0) return cudaErrorInvalidValue;
-  if (!fp64 && (!Eklo || !Ekqlo)) return cudaErrorInvalidValue;
-  if (!db.fb || !db.fx || !db.ctr) return cudaErrorInvalidValue;
-  if (fp64) {
-    k_dynamic<true, true><<<nblocks, DynShape<true>::threads, 0, s>>>(g, tet, Ek, Ekq, q, W2, cma, tau, occ, empq,
-                                                                       omega, nw, db, Eklo, Ekqlo, counters);
-    *rows = (int)((g.ntet + 31) / 32);
-  } else {
-    cudaError_t e = cudaMemsetAsync(db.ctr, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
-    k_dynamic<false, true><<<nblocks, DynShape<false>::threads, 0, s>>>(g, tet, Ek, Ekq, q, W2, cma, tau, occ, empq,
-                                                                         omega, nw, db, Eklo, Ekqlo, counters);
-    k_fx_rows<<<(2 * nw + 255) / 256, 256, 0, s>>>(db.fx, nblocks, nw, db.partR, db.partI);
-    *rows = 1;
-  }
-  return cudaGetLastError();
+  if (fp64)
+    return im_only ? launch_weights<true, true>(a, omega, nw, nblocks, scale, dos, ndos, re, im, s)
+                   : launch_weights<true, false>(a, omega, nw, nblocks, scale, dos, ndos, re, im, s);
+  return im_only ? launch_weights<false, true>(a, omega, nw, nblocks, scale, dos, ndos, re, im, s)
+                 : launch_weights<false, false>(a, omega, nw, nblocks, scale, dos, ndos, re, im, s);
 }
 
 int dynamic_max_ctas_per_sm(int fp64) {

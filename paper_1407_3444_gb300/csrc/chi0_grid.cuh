@@ -12,15 +12,18 @@ namespace grid {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// x / d for 0 <= x < qmax * d (small quotients): binary search, no division sequence
-__device__ __forceinline__ int div_small(int x, int d, int qmax) {
-  int lo = 0, hi = qmax;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (mid * d <= x) lo = mid;
-    else hi = mid;
+// x / d for x < 2^24, d < 2^13 (and the remainder), without a division sequence
+__device__ __forceinline__ int quick_div(int x, int d, int &rem) {
+  int k = (int)__fdividef((float)x + 0.5f, (float)d);
+  rem = x - k * d;
+  if (rem < 0) {
+    --k;
+    rem += d;
+  } else if (rem >= d) {
+    ++k;
+    rem -= d;
   }
-  return lo;
+  return k;
 }
 
 // Corners of tetrahedron t at k and at k+q, and its fractional volume.  Builtin mesh:

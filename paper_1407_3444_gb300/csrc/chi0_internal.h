@@ -123,34 +123,37 @@ long long static_max_units(long long ntet);      // ... of any window
 // message of the last failed call made without a plan (chi0_last_error(NULL))
 void set_global_error(const char *msg);
 
-// Work buffers of the dynamic weights: one partial per (batch of 32 tetrahedra, frequency) for
-// the pieces evaluated directly, and the far-field box moments (per warp, then summed)
+// Work buffers of the dynamic weights
 struct DynBufs {
-  double *partR, *partI;  // [nbatch][nw]
-  void *box_tab;          // box centres and radii of the pass (dynamic_box_tab_bytes())
-  double *box_part;       // [warps of the launch][dynamic_box_slots(fp64)] (FP32 kernel: int64 per CTA)
-  double *box_tot;        // [dynamic_box_slots(fp64)]
-  double *far;            // [nw]: Re contribution of the box multipoles per frequency
-  void *fb;               // [warps of the launch][dynamic_fb_bytes(fp64)]: near-field entries
-                          // left to the per-vertex table (scratch)
+  double *partR, *partI;    // FP64 kernel: [warps of the launch][nw]
+  void *box_tab;            // boxes and sorted frequencies of the pass (dynamic_box_tab_bytes())
+  double *box_part;         // box moments: FP64 [warps of the launch][dynamic_box_slots(1)], FP32 int64 per CTA
+  double *box_tot;          // [dynamic_box_slots(fp64)]
+  void *fb;                 // [warps of the launch][dynamic_fb_bytes(fp64)]: near-field entries
+                            // left to the per-vertex table (scratch)
   unsigned long long *fx;   // FP32 kernel: [CTAs of the launch][2][dynamic_max_nw()] fixed-point sums
-  unsigned long long *ctr;  // FP32 kernel: batch counter (reset by the launch)
+  unsigned long long *ctr;  // FP32 kernel: unit counter (reset by the launch)
+};
+// one q of a dynamic launch: energies FP64 absolute, or FP32 relative to eF (hi and lo parts), their
+// band bounds, |M|^2
+struct DynArgs {
+  Grid g;
+  Tet tet;
+  Q q;
+  const void *Ek, *Ekq, *W2;
+  const float *Eklo, *Ekqlo;
+  const short *occ, *occf, *emp, *empf;
+  int cma;
+  float tau;
+  DynBufs db;
+  unsigned long long *counters;  // profile (or none)
 };
 
-// dynamic weights for one q and nw <= dynamic_max_nw() frequencies: partR/partI in *rows rows
-// of nw (FP64: one per batch; FP32: one) and far[nw] (add far to the sum of partR)
-cudaError_t launch_dynamic(const Grid &g, const Tet &tet, const void *Ek, const void *Ekq, const Q &q,
-                           const void *W2, int cma, int fp64, float tau, const short *occ, const short *empq,
-                           const double *omega, int nw, const DynBufs &db, int nblocks,
-                           unsigned long long *counters, cudaStream_t s, const float *Eklo,
-                           const float *Ekqlo, int *rows);
+// dynamic weights of one q and nw <= dynamic_max_nw() frequencies: re[nw], im[nw] = scale times the
+// sums (at w = 0 the sum of dos[0..ndos) is added to re); im_only: Im alone (the Kramers-Kronig route)
+cudaError_t launch_dynamic(const DynArgs &a, int fp64, int im_only, const double *omega, int nw, int nblocks,
+                           double scale, const double *dos, int ndos, double *re, double *im, cudaStream_t s);
 size_t dynamic_fx_bytes(int nblocks);
-// Im only, for the Kramers-Kronig route: partI in *rows rows of nw (omega ascending, >= 0)
-cudaError_t launch_dynamic_im(const Grid &g, const Tet &tet, const void *Ek, const void *Ekq, const Q &q,
-                              const void *W2, int cma, int fp64, float tau, const short *occ, const short *empq,
-                              const double *omega, int nw, const DynBufs &db, int nblocks,
-                              unsigned long long *counters, cudaStream_t s, const float *Eklo,
-                              const float *Ekqlo, int *rows);
 // energies and eigenvectors at k+q (fractional q) by linear interpolation from the periodic
 // mesh (chi0_interp.cu): Eq [nc][nb], Cq [nc][norb][nb] (C == nullptr: energies only), c64:
 // complex64 vectors, else complex128
@@ -172,11 +175,6 @@ cudaError_t launch_dos(const Grid &g, const Tet &tet, const double *E, int lo, i
                        int nblocks, cudaStream_t s, unsigned long long *pairs = nullptr);
 // band-pair output: out[i] = scale * pairs[i] in FP64 (pairs: fixed-point totals of the static kernels)
 cudaError_t launch_pairs_out(const unsigned long long *pairs, int n, double scale, double *out, cudaStream_t s);
-
-// out[k] = scale * (sum_b partial[b*nw + k] (+ sum dos where omega == 0) (+ extra[k]))
-cudaError_t launch_reduce(const double *partial, int nblocks, int nw, double scale, const double *dos,
-                          int ndos, const double *omega, double *out, cudaStream_t s,
-                          const double *extra = nullptr);
 
 int static_blocks();
 int dynamic_max_nw();

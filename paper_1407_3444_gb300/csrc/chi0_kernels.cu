@@ -8,7 +8,6 @@
 //  (the static weights, Eq. 1 at w = 0, are in chi0_static.cu)
 //  (the dynamic weights, Eqs. 1-3, are in chi0_dynamic.cu)
 //  k_dos      Gamma: the intraband q -> 0 limit, tetrahedron DOS at eF (Sec. III).
-//  k_reduce   deterministic fixed-order sum of the batch partials.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -206,38 +205,6 @@ __global__ void __launch_bounds__(kThreads) k_pairs_out(const unsigned long long
   if (i < n) out[i] = scale * ((double)(long long)pairs[i] / kPairScale);
 }
 
-// ---------------------------------------------------------------- reduction
-constexpr int kRedThreads = 1024;
-__global__ void __launch_bounds__(kRedThreads) k_reduce(const double *__restrict__ partial, int nblocks, int nw,
-                                                         double scale, const double *__restrict__ dos, int ndos,
-                                                         const double *__restrict__ omega,
-                                                         const double *__restrict__ extra,
-                                                         double *__restrict__ out) {
-  const int k = blockIdx.x;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0, sd = 0.0;
-  int b = threadIdx.x;
-  for (; b + 3 * kRedThreads < nblocks; b += 4 * kRedThreads) {  // independent loads in flight
-    s0 += partial[(long long)b * nw + k];
-    s1 += partial[(long long)(b + kRedThreads) * nw + k];
-    s2 += partial[(long long)(b + 2 * kRedThreads) * nw + k];
-    s3 += partial[(long long)(b + 3 * kRedThreads) * nw + k];
-  }
-  for (; b < nblocks; b += kRedThreads) s0 += partial[(long long)b * nw + k];
-  const bool add_dos = dos && (omega == nullptr || omega[k] == 0.0);
-  if (add_dos)
-    for (int i = threadIdx.x; i < ndos; i += kRedThreads) sd += dos[i];
-  double v = ((s0 + s1) + (s2 + s3)) + sd;
-  __shared__ double red[kRedThreads / 32];
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    v = red[threadIdx.x];
-    v = warp_sum(v);
-    if (threadIdx.x == 0) out[k] = scale * (extra ? v + extra[k] : v);
-  }
-}
-
 }  // namespace
 
 // ======================================================================= launchers
@@ -309,12 +276,6 @@ cudaError_t launch_dos(const Grid &g, const Tet &tet, const double *E, int lo, i
 
 cudaError_t launch_pairs_out(const unsigned long long *pairs, int n, double scale, double *out, cudaStream_t s) {
   k_pairs_out<<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(pairs, n, scale, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reduce(const double *partial, int nblocks, int nw, double scale, const double *dos,
-                          int ndos, const double *omega, double *out, cudaStream_t s, const double *extra) {
-  k_reduce<<<nw, kRedThreads, 0, s>>>(partial, nblocks, nw, scale, dos, ndos, omega, extra, out);
   return cudaGetLastError();
 }
 

@@ -303,6 +303,42 @@ constexpr double mean_err(double R, int K) {  // the Chebyshev truncation bound 
   for (int i = 0; i < K; ++i) t *= q;
   return t;
 }
+// the polynomial for radius R: p_0 .. p_{K-1}, and a_0 .. a_{K-1} in T
+template <typename T, int K> struct ChebInv {
+  T v[K];
+  double p_[K];
+  constexpr explicit ChebInv(double R) : v(), p_() {
+    // sum_n c_n T_n(t/R), c_0 = 1/s, c_n = 2 (-q)^n / s, collected in powers of u = t/R
+    const double s = mean_sqrt(1.0 - R * R), q = R / (1.0 + s);
+    double p[K + 1] = {}, t0[K + 1] = {}, t1[K + 1] = {};
+    t0[0] = 1.0;
+    t1[1] = 1.0;
+    double c = 1.0 / s;
+    p[0] = c;
+    c *= -2.0 * q;
+    for (int n = 1; n < K; ++n) {
+      for (int k = 0; k <= n; ++k) p[k] += c * t1[k];
+      c *= -q;
+      double t2[K + 1] = {};
+      for (int k = 0; k <= n; ++k) t2[k + 1] = 2.0 * t1[k];
+      for (int k = 0; k <= n; ++k) {
+        t2[k] -= t0[k];
+        t0[k] = t1[k];
+      }
+      for (int k = 0; k <= K; ++k) t1[k] = t2[k];
+    }
+    double rk = 1.0;
+    for (int k = 0; k < K; ++k) {
+      // p_k differs from Taylor's (-1)^k by the truncation; a difference of a few roundings is
+      // this computation's own and is dropped (it would be a bias common to all pieces)
+      const double one = (k & 1) ? -1.0 : 1.0, dp = p[k] / rk - one;
+      const double pk = dp < 1e-15 && dp > -1e-15 ? one : p[k] / rk;
+      p_[k] = pk;
+      v[k] = (T)(pk * 6.0 / ((k + 1.0) * (k + 2.0) * (k + 3.0) * (k + 4.0)));  // a_k
+      rk *= R;
+    }
+  }
+};
 constexpr int mean_off(int tier) { return 2 * tier * (tier + 1); }  // a tier's first coefficient
 // threshold on the high word of max|e| (FP32: its bits): bits <= thr implies max|e| <= R
 constexpr int mean_bits(double x, bool dbl) {
@@ -317,43 +353,23 @@ constexpr int mean_bits(double x, bool dbl) {
 template <typename T, int NT> struct MeanTab {
   T a[2 * NT * (NT + 1)];
   int thr[NT];
-  constexpr MeanTab(const double (&R)[NT], double tol) : a(), thr() {
-    for (int i = 0; i < NT; ++i) {
-      const int K = 4 * (i + 1);
-      thr[i] = mean_bits(R[i], sizeof(T) == 8);
-      if (mean_err(R[i], K) > tol) thr[i] = -1 / (K - K);  // (compile error: R too large for K)
-      const double s = mean_sqrt(1.0 - R[i] * R[i]), q = R[i] / (1.0 + s);
-      // sum_n c_n T_n(t/R), c_0 = 1/s, c_n = 2 (-q)^n / s, collected in powers of u = t/R
-      double p[4 * NT] = {}, t0[4 * NT] = {}, t1[4 * NT] = {};
-      t0[0] = 1.0;
-      t1[1] = 1.0;
-      double c = 1.0 / s;
-      p[0] = c;
-      c *= -2.0 * q;
-      for (int n = 1; n < K; ++n) {
-        for (int k = 0; k <= n; ++k) p[k] += c * t1[k];
-        c *= -q;
-        double t2[4 * NT] = {};
-        for (int k = 0; k <= n && k + 1 < 4 * NT; ++k) t2[k + 1] = 2.0 * t1[k];
-        for (int k = 0; k <= n; ++k) {
-          t2[k] -= t0[k];
-          t0[k] = t1[k];
-        }
-        for (int k = 0; k < 4 * NT; ++k) t1[k] = t2[k];
-      }
-      double rk = 1.0;
-      for (int k = 0; k < K; ++k) {
-        // p_k differs from Taylor's (-1)^k by the truncation; a difference of a few roundings is
-        // this computation's own and is dropped (it would be a bias common to all pieces)
-        const double one = (k & 1) ? -1.0 : 1.0, dp = p[k] / rk - one;
-        const double pk = dp < 1e-15 && dp > -1e-15 ? one : p[k] / rk;
-        a[mean_off(i) + k] = (T)(pk * 6.0 / ((k + 1.0) * (k + 2.0) * (k + 3.0) * (k + 4.0)));
-        rk *= R[i];
-      }
+  template <int I> constexpr void tier(const double (&R)[NT]) {
+    if constexpr (I < NT) {
+      const ChebInv<T, 4 * (I + 1)> c(R[I]);
+      for (int k = 0; k < 4 * (I + 1); ++k) a[mean_off(I) + k] = c.v[k];
+      thr[I] = mean_bits(R[I], sizeof(T) == 8);
+      tier<I + 1>(R);
     }
   }
+  constexpr explicit MeanTab(const double (&R)[NT]) : a(), thr() { tier<0>(R); }
 };
-__constant__ constexpr MeanTab<double, kMeanTiersD> kMeanD{kMeanRD, kMeanTolD};
+constexpr bool mean_tiers_ok() {
+  for (int i = 0; i < kMeanTiersD; ++i)
+    if (mean_err(kMeanRD[i], 4 * (i + 1)) > kMeanTolD) return false;
+  return true;
+}
+static_assert(mean_tiers_ok(), "a tier's R is too large for its K");
+__constant__ constexpr MeanTab<double, kMeanTiersD> kMeanD{kMeanRD};
 template <typename T> struct Mean;
 template <> struct Mean<float> {
   static __device__ __forceinline__ int bits(float x) {
@@ -546,7 +562,7 @@ template <typename T> __device__ T inv_sum_table(const T xin[4], const T f[4]) {
 // G[p..r] are common to all j, and the entries with knot j doubled follow the same recursion,
 //   H_j[p..r] = ((p < j ? H_j[p+1..r] : G[p..r]) - (r > j ? H_j[p..r-1] : G[p..r])) / (u_r - u_p),
 //   H_j[j..j] = g'(u_j) = 3 u_j^2 ln|u_j| + u_j^2,
-// so all four fourth divided differences g[u, u_j] = H_j[0..3] take four logarithms and six
+// so all four fourth divided differences g[u, u_j] = H_j[0..3] take four logarithms (FP64: three) and six
 // reciprocals (the per-vertex table below takes twenty and forty divisions).  The result is
 // sum_j f_j H_j[0..3] / s.
 // A pair of adjacent knots a < b of one sign with y = (b - a)/a small (|y| <= 1/8, ties
@@ -584,10 +600,20 @@ template <typename T> __device__ __forceinline__ bool inv_sum_shared(const T x[4
   }
   if ((cl[0] && cl[1]) || (cl[1] && cl[2])) return false;  // three knots together
   T g[4], gp[4], L[4];
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) L[i] = u[i] == T(0) ? T(0) : Num<T>::lg(tabs(u[i]));
+  } else {  // (the end knot of largest magnitude is +-1 to rounding: no logarithm)
+    const bool low = tabs(x[0]) > tabs(x[3]);
+    const T o = low ? u[3] : u[0], Lo = o == T(0) ? T(0) : Num<T>::lg(tabs(o));
+    L[0] = low ? T(0) : Lo;
+    L[3] = low ? Lo : T(0);
+#pragma unroll
+    for (int i = 1; i < 3; ++i) L[i] = u[i] == T(0) ? T(0) : Num<T>::lg(tabs(u[i]));
+  }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const T t = u[i], t2 = t * t;
-    L[i] = t == T(0) ? T(0) : Num<T>::lg(tabs(t));
     g[i] = t2 * t * L[i];
     gp[i] = T(3) * t2 * L[i] + t2;
   }
@@ -859,6 +885,31 @@ template <typename T> __device__ __forceinline__ T delta_sum_pre(const T x[4], c
     acc += f[jj] * M[0];
   }
   return T(0.25) * acc;
+}
+
+// sum_j f_j (1/V) int_S lambda_j delta(X) for sorted knots x with x_0 < 0 < x_3, spans e_j - e_i from
+// the unshifted knots e: the plane X = 0 cuts S in a triangle around vertex 0 (x_1 >= 0) or 3
+// (x_2 <= 0), or in a quadrilateral, split by the diagonal between edges 03 and 12; f is linear,
+// so each triangle contributes its share of the density (the nonnegative terms of the quadratic
+// B-spline's recursion) times the mean of f at its three vertices.  A quarter of the operations of
+// the per-vertex cubic recursions of delta_sum_pre.
+template <typename T> __device__ __forceinline__ T delta_section(const T x[4], const T e[4], const T f[4]) {
+  const T r30 = rcp_nr(e[3] - e[0]);
+  const T f03 = f[0] - x[0] * r30 * (f[3] - f[0]);  // f on edge 03 (fraction (0 - x_0)/(x_3 - x_0))
+  if (x[1] < T(0) && x[2] > T(0)) {
+    const T r20 = rcp_nr(e[2] - e[0]), r21 = rcp_nr(e[2] - e[1]), r31 = rcp_nr(e[3] - e[1]);
+    const T f02 = f[0] - x[0] * r20 * (f[2] - f[0]), f12 = f[1] - x[1] * r21 * (f[2] - f[1]);
+    const T f13 = f[1] - x[1] * r31 * (f[3] - f[1]);
+    const T a = -x[0] * x[2] * r20, b = -x[1] * x[3] * r31, m = f03 + f12;
+    return (a * (f02 + m) + b * (f13 + m)) * r21 * r30;
+  }
+  // around vertex 0 or 3: edges to the other three
+  const bool lo = x[1] >= T(0);
+  const T p = lo ? x[0] : x[3], fp = lo ? f[0] : f[3], ep = lo ? e[0] : e[3];
+  const T u = lo ? e[1] : e[2], fu = lo ? f[1] : f[2], v = lo ? e[2] : e[1], fv = lo ? f[2] : f[1];
+  const T ru = rcp_nr(u - ep), rv = rcp_nr(v - ep);
+  const T fa = fp - p * ru * (fu - fp), fb = fp - p * rv * (fv - fp);
+  return p * ru * p * rv * r30 * (f03 + fa + fb);
 }
 
 // Tetrahedron density of states at eF for one band: M(0; a_0..a_3), quadratic B-spline

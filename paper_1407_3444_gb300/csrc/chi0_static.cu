@@ -48,6 +48,7 @@ namespace {
 
 using grid::kFull;
 using grid::pair_add;
+using grid::quick_div;
 using grid::tet_corners;
 using grid::warp_sum;
 
@@ -177,20 +178,6 @@ __device__ __noinline__ double table_round(const PieceQueue<typename std::condit
     for (int i = 0; i < 8; ++i) lm &= lm - 1u;
   }
   return acc;
-}
-
-// x / d for x < 2^24, d < 2^12 (and the remainder), without a division sequence
-__device__ __forceinline__ int quick_div(int x, int d, int &rem) {
-  int k = (int)__fdividef((float)x + 0.5f, (float)d);
-  rem = x - k * d;
-  if (rem < 0) {
-    --k;
-    rem += d;
-  } else if (rem >= d) {
-    ++k;
-    rem -= d;
-  }
-  return k;
 }
 
 template <bool FP64, int NT, int MINB>
