@@ -10,10 +10,11 @@
 //   int hat_j(u) / (u - w) du = [G(u_{j+1} - w) - 2 G(u_j - w) + G(u_{j-1} - w)] / du,
 // finite also where w is a node.  Summing by parts over the nodes,
 //   Re(w) = (1 / (pi du)) sum_{k=0..m} [G(u_k - w) + G(u_k + w)] (Im_{k-1} - 2 Im_k + Im_{k+1}),
-// with Im_j = 0 for j <= 0 and j >= m.  One thread per output node, FP64, O(m) per node.
+// with Im_j = 0 for j <= 0 and j >= m.  FP64, O(m) per output node.
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "chi0_grid.cuh"
 #include "chi0_internal.h"
 
 namespace chi0int {
@@ -21,14 +22,16 @@ namespace {
 
 __device__ __forceinline__ double gxl(double x) { return x == 0.0 ? 0.0 : x * log(fabs(x)); }
 
-__global__ void __launch_bounds__(256) k_kk(const double *__restrict__ im, int m, double du, double scale,
-                                            const double *__restrict__ dos, int ndos, double *__restrict__ re) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
+// One block per output node, its threads over the nodes k (pairwise sums in a fixed order): one thread
+// per output node left a 400-node transform on two blocks, 1.9 ms of serial logarithms.
+constexpr int kKKThreads = 128;
+__global__ void __launch_bounds__(kKKThreads) k_kk(const double *__restrict__ im, int m, double du, double scale,
+                                                   const double *__restrict__ dos, int ndos, double *__restrict__ re) {
+  const int i = blockIdx.x;
   const double w = i * du;
   double s = 0.0, c = 0.0;  // compensated sum
   auto I = [&](int j) { return j >= 1 && j < m ? im[j] : 0.0; };  // Im(0) = 0; 0 past the grid
-  for (int k = 0; k <= m; ++k) {
+  for (int k = threadIdx.x; k <= m; k += kKKThreads) {
     const double d2 = I(k - 1) - 2.0 * I(k) + I(k + 1);
     if (d2 == 0.0) continue;
     const double uk = k * du;
@@ -37,13 +40,20 @@ __global__ void __launch_bounds__(256) k_kk(const double *__restrict__ im, int m
     c += fabs(s) >= fabs(t) ? (s - y) + t : (t - y) + s;
     s = y;
   }
-  double v = (s + c) / (3.141592653589793 * du);
-  if (dos && i == 0) {  // the q -> 0 intraband limit at w = 0 (Sec. III), as the direct route adds it
-    double sd = 0.0;
-    for (int k = 0; k < ndos; ++k) sd += dos[k];
-    v += scale * sd;
+  double sd = 0.0;  // the q -> 0 intraband limit at w = 0 (Sec. III), as the direct route adds it
+  if (dos && i == 0)
+    for (int k = threadIdx.x; k < ndos; k += kKKThreads) sd += dos[k];
+  __shared__ double red[2][kKKThreads / 32];
+  const double v = grid::warp_sum(s + c);
+  sd = grid::warp_sum(sd);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = v;
+    red[1][threadIdx.x >> 5] = sd;
   }
-  re[i] = v;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    re[i] = ((red[0][0] + red[0][1]) + (red[0][2] + red[0][3])) / (3.141592653589793 * du) +
+            scale * ((red[1][0] + red[1][1]) + (red[1][2] + red[1][3]));
 }
 
 }  // namespace
@@ -51,7 +61,7 @@ __global__ void __launch_bounds__(256) k_kk(const double *__restrict__ im, int m
 cudaError_t launch_kk(const double *im, int m, double du, double scale, const double *dos, int ndos, double *re,
                       cudaStream_t s) {
   if (m <= 1 || !(du > 0.0)) return cudaErrorInvalidValue;
-  k_kk<<<(m + 255) / 256, 256, 0, s>>>(im, m, du, scale, dos, ndos, re);
+  k_kk<<<m, kKKThreads, 0, s>>>(im, m, du, scale, dos, ndos, re);
   return cudaGetLastError();
 }
 
