@@ -63,7 +63,8 @@ struct chi0_plan {
   void *box_tab_d = nullptr;                  // dynamic weights: boxes and sorted frequencies of the pass,
   double *box_part_d = nullptr;               // box moments per warp or CTA, and their totals
   double *box_tot_d = nullptr;
-  void *fb_d = nullptr;                       // dynamic weights: per-warp fallback entries,
+  int *fbn_d = nullptr;                       // dynamic weights: per-warp fallback entries,
+  void *fb_d = nullptr;                       // their counts,
   unsigned long long *fx_d = nullptr;         // per-CTA fixed-point sums (FP32) and the
   unsigned long long *ctr_d = nullptr;        // batch counter
   unsigned long long *pairs_fx_d = nullptr;   // band-pair output: fixed-point totals of one q,
@@ -177,6 +178,7 @@ static void release(chi0_plan_t *p) {
   cudaFree(p->box_part_d);
   cudaFree(p->box_tot_d);
   cudaFree(p->fb_d);
+  cudaFree(p->fbn_d);
   cudaFree(p->fx_d);
   cudaFree(p->ctr_d);
   cudaFree(p->pairs_fx_d);
@@ -349,6 +351,7 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
     CK(p, cudaMalloc(&p->box_part_d, sizeof(double) * warps * dynamic_box_slots(fp64)));
     CK(p, cudaMalloc(&p->box_tot_d, sizeof(double) * dynamic_box_slots(fp64)));
     CK(p, cudaMalloc(&p->fb_d, warps * dynamic_fb_bytes(fp64)));
+    CK(p, cudaMalloc(&p->fbn_d, warps * sizeof(int)));
     CK(p, cudaMalloc(&p->fx_d, dynamic_fx_bytes(dynamic_max_ctas_per_sm(fp64) * device_sms())));
     CK(p, cudaMalloc(&p->ctr_d, sizeof(unsigned long long)));
   }
@@ -664,7 +667,7 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
     a.empf = qb.empf;
     a.cma = op.cma;
     a.tau = (float)op.tau;
-    a.db = DynBufs{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->fb_d, p->fx_d, p->ctr_d};
+    a.db = DynBufs{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->fb_d, p->fbn_d, p->fx_d, p->ctr_d};
     a.counters = op.profile ? p->counters_d : nullptr;
     const bool kk = kk_du > 0.0;
     const double *dos = q.gamma ? p->dos_d : nullptr;
@@ -674,7 +677,7 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
       const size_t at = (size_t)iq * nw + w0;
       tm.start(CHI0_K_DYNAMIC);
       CK(p, launch_dynamic(a, fp64, kk, om_d + w0, nwc, p->dynamic_grid, scale, dos, ndos, outR + at, outI + at, s));
-      p->stats.kernels += kk ? 3 : 4;  // setup, weights, box sums, output
+      p->stats.kernels += kk ? 3 : (fp64 ? 4 : 5);  // setup, weights, (fallback entries,) box sums, output
       tm.stop();
     }
     if (kk) {  // Kramers-Kronig route: Re from Im over the whole grid

@@ -43,7 +43,7 @@
 // ranges and own moments, then all (piece, frequency, term) pairs of the drain are evaluated packed,
 // one per lane, first the own-moment pairs, then the near ones.  Near pairs that the shared
 // divided-difference table leaves go to a per-warp fallback buffer in global memory, evaluated in
-// full rounds when it fills.
+// full rounds when it fills (FP32: the rest by a kernel of its own, k_dyn_fallback).
 // Sums.  FP32 kernel: per-CTA sums in 64-bit fixed point (units of 2^-44) in shared memory, added
 // with integer atomics and written once per CTA: integer sums are exact in any order, so the warps
 // take units from a launch-wide counter and the results are bitwise reproducible for any launch
@@ -337,9 +337,6 @@ __device__ __forceinline__ void fx_add(unsigned *lo, unsigned *hi, int i, float 
   atomicAdd(&hi[i], (unsigned)((unsigned long long)t >> 32) + (old + l < old ? 1u : 0u));
 }
 
-// Out-of-line copy of the fallback's delta term (rare: kept out of the hot code's instruction cache)
-template <typename T> __device__ __noinline__ T delta_sum_ol(const T d[4], const T f[4]) { return delta_sum(d, f, T(0)); }
-
 // the delta term of a near pair: FP64 by the plane section; FP32 by the cubic recursion, whose
 // rounding (a relative 2.9e-8 common to every piece, from its 4/3) its results have always carried
 __device__ __forceinline__ double delta_term(const double x[4], const double e[4], const double f[4]) {
@@ -371,7 +368,9 @@ __device__ __noinline__ typename std::conditional<FP64, double, float>::type nea
   // (the entries that reach this function are the ones the shared table left: the per-vertex
   // table directly, after the series branches)
   if constexpr (FP64) {
+    double v;
     if (series_ok(xx, T(Num<T>::kappa))) return series_sum(xx, f);
+    if (inv_sum_triple(xx, f, v)) return v;
     return inv_sum_table(xx, f);
   } else {
     if (series_ok(xx, Num<float>::kappa)) return series_sum(xx, f);
@@ -381,7 +380,8 @@ __device__ __noinline__ typename std::conditional<FP64, double, float>::type nea
       return inv_sum_table(y, f);
     }
     ++nfp64;
-    double yd[4] = {y[0], y[1], y[2], y[3]}, fd[4] = {f[0], f[1], f[2], f[3]};
+    double yd[4] = {y[0], y[1], y[2], y[3]}, fd[4] = {f[0], f[1], f[2], f[3]}, v;
+    if (inv_sum_triple(yd, fd, v)) return (float)v;
     return (float)inv_sum_table(yd, fd);
   }
 }
@@ -407,9 +407,10 @@ template <bool STRICT, typename T> __device__ __forceinline__ int first_above(co
 }
 
 // a queued piece's frequency ranges (indices of the sorted frequencies): the - term from f0 to f1,
-// its near part n0 to n1; the + term up to p1, its near part up to np
+// its near part n0 to n1; the + term up to p1, its near part up to np; the delta term m0 to m1 (the
+// frequencies inside the knots, one more on each side: the pair's own test decides)
 struct Range {
-  short f0, n0, n1, f1, np, p1;
+  short f0, n0, n1, f1, np, p1, m0, m1;
 };
 
 // IMO: Im only (the delta term of Eq. 2; no principal value, no boxes) for the Kramers-Kronig route
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   __shared__ T s_qv[W][kQC][3];
   __shared__ short s_qb[W][kQC];
   __shared__ Range s_rg[W][DC];
-  __shared__ int s_po[W][DC + 1], s_pn[W][DC + 1];  // prefix sums: own pairs, near pairs
+  __shared__ int s_po[W][DC + 1], s_pn[W][DC + 1], s_pd[W][DC + 1];  // prefix sums: own, near, delta pairs
   // FP64 kernel: per-warp compensated sums; FP32 kernel: per-CTA fixed-point sums (two words)
   constexpr int WA = FX ? 1 : W, NA = FX ? 1 : kNWPass;
   __shared__ T sR[WA][IMO ? 1 : NA], sI[WA][NA];
@@ -525,7 +526,8 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
 #pragma unroll 1
       for (int r = 0; r <= nr; ++r) {
         if (iw >= 0 && rank == r) {
-          if constexpr (!IMO) kadd_t(sR[wib][iw], cR[wib][iw], re);
+          if constexpr (!IMO)
+            if (re != T(0)) kadd_t(sR[wib][iw], cR[wib][iw], re);
           if (im != T(0)) kadd_t(sI[wib][iw], cI[wib][iw], im);
         }
         __syncwarp();
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
 #pragma unroll 1
     for (int base = 0; base < nfb; base += 32) {
       const int k = base + lane;
-      T re = T(0), im = T(0);
+      T re = T(0);
       int iw = -1;
       if (k < nfb) {
         const FbEnt<T> &o = gfb[k];
@@ -552,9 +554,8 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
         const T vr = o.v;
         iw = o.code >> 1;
         re = vr * near_term<FP64>(x, ff, A.tau, nfp64);
-        if ((o.code & 1) == 0 && x[0] < T(0) && x[3] > T(0)) im = vr * delta_sum_ol(x, ff) * T(3.141592653589793);
       }
-      round_add(iw, re, im);
+      round_add(iw, re, T(0));
     }
     nfb = 0;
     __syncwarp();
@@ -562,24 +563,31 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   // evaluates n <= DC queued pieces: ranges and own moments one piece per lane, then their
   // (piece, frequency, term) pairs packed over the lanes
   auto drain = [&](int n) {
-    int no = 0, nn = 0;
+    int no = 0, nn = 0, nd = 0;
     if (lane < n) {
       const int sl = (qh + lane) % kQC;
       const T D0h = s_qv[wib][sl][1];
       const T e0 = s_qe[wib][sl][0], e3 = s_qe[wib][sl][3];
-      Range r;
-      if constexpr (IMO) {  // the frequencies inside the knots, one more on each side (the pair's own test decides)
+      Range r{};
+      {
         const int a = first_above<true>(s_w, nw, D0h + e0), z = first_above<false>(s_w, nw, D0h + e3);
-        r = Range{0, (short)(a > 0 ? a - 1 : 0), (short)(z < nw ? z + 1 : nw), 0, 0, 0};
-        nn = r.n1 - r.n0;
-      } else {
+        r.m0 = (short)(a > 0 ? a - 1 : 0);
+        r.m1 = (short)(z < nw ? z + 1 : nw);
+        nd = r.m1 - r.m0;
+      }
+      if constexpr (!IMO) {
         const int b = s_qb[wib][sl];
         const T half = (e3 - e0) * T(0.5), c = D0h + (e0 + e3) * T(0.5), near = half * T(S::far);
         const int f0 = b >= 0 ? s_rng[b][0] : 0, f1 = b >= 0 ? s_rng[b][1] : nw, p1 = b >= 0 ? s_rng[b][2] : nw;
         const int a = min(max(first_above<true>(s_w, nw, c - near), f0), f1);
         const int z = max(min(first_above<false>(s_w, nw, c + near), f1), a);
         const int p = p1 > 0 ? min(first_above<false>(s_w, nw, near - c), p1) : 0;
-        r = Range{(short)f0, (short)a, (short)z, (short)f1, (short)p, (short)p1};
+        r.f0 = (short)f0;
+        r.n0 = (short)a;
+        r.n1 = (short)z;
+        r.f1 = (short)f1;
+        r.np = (short)p;
+        r.p1 = (short)p1;
         nn = (z - a) + p;
         no = (f1 - f0) - (z - a) + (p1 - p);
         if (no > 0) {
@@ -607,21 +615,23 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
       }
       s_rg[wib][lane] = r;
     }
-    int po = no, pn = nn;  // inclusive prefix sums over the lanes
+    int po = no, pn = nn, pd = nd;  // inclusive prefix sums over the lanes
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(kFull, po, o), y = __shfl_up_sync(kFull, pn, o);
+      const int x = __shfl_up_sync(kFull, po, o), y = __shfl_up_sync(kFull, pn, o), z = __shfl_up_sync(kFull, pd, o);
       if (lane >= o) {
         po += x;
         pn += y;
+        pd += z;
       }
     }
     if (lane < n) {
       s_po[wib][lane + 1] = po;
       s_pn[wib][lane + 1] = pn;
+      s_pd[wib][lane + 1] = pd;
     }
-    if (lane == 0) s_po[wib][0] = s_pn[wib][0] = 0;
-    const int own = __shfl_sync(kFull, po, 31), near = __shfl_sync(kFull, pn, 31);
+    if (lane == 0) s_po[wib][0] = s_pn[wib][0] = s_pd[wib][0] = 0;
+    const int own = __shfl_sync(kFull, po, 31), near = __shfl_sync(kFull, pn, 31), inside = __shfl_sync(kFull, pd, 31);
     __syncwarp();
     if constexpr (!IMO) {
       int p = 0;
@@ -660,68 +670,62 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
         round_add(iw, v, T(0));
       }
     }
-    // near pairs: the shared divided-difference table and the delta term.  Pairs the table leaves
-    // (three clustered knots, three zero knots) go, knots and all, to the fallback buffer.
-    int p = 0;
+    // knots (D0 - |w|) + e of the - term at frequency jw
+    auto load_piece = [&](int sl, T ee[4], T ff[4]) {
+      if constexpr (FP64) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          ee[i] = s_qe[wib][sl][i];
+          ff[i] = s_qf[wib][sl][i];
+        }
+      } else {  // one 16-byte load each
+        const float4 e4 = *reinterpret_cast<const float4 *>(&s_qe[wib][sl][0]);
+        const float4 f4 = *reinterpret_cast<const float4 *>(&s_qf[wib][sl][0]);
+        ee[0] = e4.x, ee[1] = e4.y, ee[2] = e4.z, ee[3] = e4.w;
+        ff[0] = f4.x, ff[1] = f4.y, ff[2] = f4.z, ff[3] = f4.w;
+      }
+    };
+    auto shifted = [&](int sl, int jw, const T ee[4], T x[4]) {
+      const T sh = near_shift(s_qv[wib][sl][1], s_qv[wib][sl][2], s_w[jw], FP64 ? T(0) : s_wl[FP64 ? 0 : jw]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = sh + ee[i];
+    };
+    // near pairs: the shared divided-difference table.  Pairs it leaves (three clustered knots, three
+    // zero knots) go, knots and all, to the fallback buffer.
+    if constexpr (!IMO) {
+      int p = 0;
 #pragma unroll 1
-    for (int base = 0; base < near; base += 32) {  // warp-uniform
-      if (!IMO && nfb > kFbCap - 32) fallback_flush();
-      const int it = base + lane;
-      T re = T(0), im = T(0), x[4], ff[4], vr = T(0);
-      int iw = -1, code = 0;
-      bool left = false;
-      if (it < near) {
-        while (s_pn[wib][p + 1] <= it) ++p;
-        const int sl = (qh + p) % kQC;
-        const Range r = s_rg[wib][p];
-        const int k = it - s_pn[wib][p], k1 = r.n1 - r.n0;
-        const bool plus = k >= k1;
-        const int jw = plus ? k - k1 : r.n0 + k;
-        const T D0h = s_qv[wib][sl][1], D0l = s_qv[wib][sl][2];
-        vr = s_qv[wib][sl][0];
-        T ee[4];
-        if constexpr (FP64) {
+      for (int base = 0; base < near; base += 32) {  // warp-uniform
+        if (nfb > kFbCap - 32) fallback_flush();
+        const int it = base + lane;
+        T re = T(0), x[4], ff[4], vr = T(0);
+        int iw = -1, code = 0;
+        bool left = false;
+        if (it < near) {
+          while (s_pn[wib][p + 1] <= it) ++p;
+          const int sl = (qh + p) % kQC;
+          const Range r = s_rg[wib][p];
+          const int k = it - s_pn[wib][p], k1 = r.n1 - r.n0;
+          const bool plus = k >= k1;
+          const int jw = plus ? k - k1 : r.n0 + k;
+          vr = s_qv[wib][sl][0];
+          T ee[4], v;
+          load_piece(sl, ee, ff);
+          if (plus) {  // knots d + |w|
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            ee[i] = s_qe[wib][sl][i];
-            ff[i] = s_qf[wib][sl][i];
+            for (int i = 0; i < 4; ++i) x[i] = (s_qv[wib][sl][1] + ee[i]) + s_w[jw];
+          } else {
+            shifted(sl, jw, ee, x);
           }
-        } else {  // one 16-byte load each
-          const float4 e4 = *reinterpret_cast<const float4 *>(&s_qe[wib][sl][0]);
-          const float4 f4 = *reinterpret_cast<const float4 *>(&s_qf[wib][sl][0]);
-          ee[0] = e4.x, ee[1] = e4.y, ee[2] = e4.z, ee[3] = e4.w;
-          ff[0] = f4.x, ff[1] = f4.y, ff[2] = f4.z, ff[3] = f4.w;
-        }
-        // - term: knots (D0 - |w|) + e; + term: knots d + |w|
-        const T om = s_w[jw];
-        if (plus) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) x[i] = (D0h + ee[i]) + om;
-        } else {
-          const T sh = near_shift(D0h, D0l, om, FP64 ? T(0) : s_wl[FP64 ? 0 : jw]);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) x[i] = sh + ee[i];
-        }
-        const bool in = !plus && x[0] < T(0) && x[3] > T(0);
-        code = (jw << 1) | (plus ? 1 : 0);
-        if constexpr (IMO) {
-          if (in) {
-            iw = jw;
-            im = vr * delta_term(x, ee, ff) * T(3.141592653589793);
-          }
-        } else {
-          T v;
+          code = (jw << 1) | (plus ? 1 : 0);
           if (inv_sum_shared(x, ff, v)) {
             iw = jw;
             re = vr * v;
-            if (in) im = vr * delta_term(x, ee, ff) * T(3.141592653589793);
           } else {
             left = true;
           }
         }
-      }
-      round_add(iw, re, im);
-      if constexpr (!IMO) {
+        round_add(iw, re, T(0));
         const unsigned bal = __ballot_sync(kFull, left);
         if (bal) {  // warp-uniform
           if (left) {
@@ -737,6 +741,26 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
           nfb += __popc(bal);
         }
       }
+    }
+    // the delta term of the frequencies inside the knots
+    int p = 0;
+#pragma unroll 1
+    for (int base = 0; base < inside; base += 32) {  // warp-uniform
+      const int it = base + lane;
+      T im = T(0);
+      int iw = -1;
+      if (it < inside) {
+        while (s_pd[wib][p + 1] <= it) ++p;
+        const int sl = (qh + p) % kQC, jw = s_rg[wib][p].m0 + (it - s_pd[wib][p]);
+        T ee[4], ff[4], x[4];
+        load_piece(sl, ee, ff);
+        shifted(sl, jw, ee, x);
+        if (x[0] < T(0) && x[3] > T(0)) {
+          iw = jw;
+          im = s_qv[wib][sl][0] * delta_term(x, ee, ff) * T(3.141592653589793);
+        }
+      }
+      round_add(iw, T(0), im);
     }
     qh += n;
     __syncwarp();
@@ -1091,7 +1115,11 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
     }
     if (end) break;
   }
-  if (nfb > 0) fallback_flush();  // warp-uniform
+  if constexpr (FX && !IMO) {
+    if (lane == 0) db.fbn[gwarp] = nfb;  // the rest of the buffer: k_dyn_fallback
+  } else {
+    if (nfb > 0) fallback_flush();  // warp-uniform
+  }
   if constexpr (FX) {
     // the CTA's fixed-point sums into its rows
     __syncthreads();
@@ -1127,6 +1155,32 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
       atomicAdd(&A.counters[3], x);
     }
   }
+}
+
+// FP32 kernel: what is left in the warps' fallback buffers, one entry per thread, into the
+// fixed-point rows.  At the end of k_dynamic each warp would walk its last few hundred entries
+// through the per-vertex table (up to 50 us a round, most of its lanes in the FP64 branch of
+// near-degenerate knots) while finished SMs idle: 30% of the time of a 64 x 64 x 16 pass.
+__global__ void __launch_bounds__(128) k_dyn_fallback(DynBufs db, int nbuf, int nrows, float tau,
+                                                      unsigned long long *__restrict__ counters) {
+  unsigned long long *row = db.fx + (size_t)(blockIdx.x % nrows) * 2 * kNWPass;
+  int nfp64 = 0;
+  for (int buf = blockIdx.x; buf < nbuf; buf += gridDim.x) {
+    const int n = db.fbn[buf];
+    const FbEnt<float> *ent = (const FbEnt<float> *)db.fb + (size_t)buf * kFbCap;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const FbEnt<float> &o = ent[k];
+      float x[4], f[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        x[i] = o.x[i];
+        f[i] = o.f[i];
+      }
+      const float v = o.v * near_term<false>(x, f, tau, nfp64);
+      atomicAdd(&row[o.code >> 1], (unsigned long long)fx_of(v));
+    }
+  }
+  if (counters && nfp64) atomicAdd(&counters[1], (unsigned long long)nfp64);
 }
 
 // box totals: slot i summed over the rows of the weight launch (FP64 kernel: per-warp FP64
@@ -1275,6 +1329,7 @@ cudaError_t launch_weights(const DynArgs &a, const double *omega, int nw, int nb
   k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, (BoxTab<T> *)db.box_tab);
   k_dynamic<FP64, IMO><<<nblocks, DynShape<FP64>::threads, IMO ? 0 : dyn_smem<FP64>(), s>>>(
       a, nw, dyn_unit_log2(a.g.ntet, a.q.hi - a.q.lo, FP64));
+  if (!FP64 && !IMO) k_dyn_fallback<<<rows * DynShape<FP64>::warps, 128, 0, s>>>(db, rows * DynShape<FP64>::warps, rows, a.tau, a.counters);
   if (!IMO) k_box_sum<FP64><<<(NS + 31) / 32, 256, 0, s>>>(db.box_part, rows, db.box_tot);
   k_dyn_out<FP64><<<nw, 128, 0, s>>>(omega, nw, db.box_tab, db.box_tot, db, rows, scale, dos, ndos, IMO ? nullptr : re, im);
   return cudaGetLastError();
@@ -1304,7 +1359,7 @@ cudaError_t launch_dynamic(const DynArgs &a, int fp64, int im_only, const double
   const DynBufs &db = a.db;
   if (nw > kNWPass || nw <= 0 || nblocks <= 0) return cudaErrorInvalidValue;
   if (!fp64 && (!a.Eklo || !a.Ekqlo)) return cudaErrorInvalidValue;
-  if (!db.box_tab || !db.box_part || !db.box_tot || !db.fb || !db.fx || !db.ctr || !db.partR || !db.partI)
+  if (!db.box_tab || !db.box_part || !db.box_tot || !db.fb || !db.fbn || !db.fx || !db.ctr || !db.partR || !db.partI)
     return cudaErrorInvalidValue;
   if (fp64)
     return im_only ? launch_weights<true, true>(a, omega, nw, nblocks, scale, dos, ndos, re, im, s)

@@ -131,6 +131,7 @@ struct DynBufs {
   double *box_tot;          // [dynamic_box_slots(fp64)]
   void *fb;                 // [warps of the launch][dynamic_fb_bytes(fp64)]: near-field entries
                             // left to the per-vertex table (scratch)
+  int *fbn;                 // FP32 kernel: [warps of the launch] entries left at its end
   unsigned long long *fx;   // FP32 kernel: [CTAs of the launch][2][dynamic_max_nw()] fixed-point sums
   unsigned long long *ctr;  // FP32 kernel: unit counter (reset by the launch)
 };

@@ -674,6 +674,72 @@ template <typename T> __device__ __forceinline__ bool inv_sum_shared(const T x[4
   return true;
 }
 
+// The case inv_sum_shared leaves most often, in FP64: three knots B of one sign together (adjacent
+// ones within kRhoShared) and the fourth, A, apart.  With L = ln|c|, c = mean(B), e = (B - c)/c,
+//   g[n + 1 knots of B] = c^(3-n) (sum_{k=n..3} G_k h_{k-n}(e) + sum_{k>=4} K_k h_{k-n}(e)),
+//   G_1 = 3 L + 1, G_2 = 3 L + 5/2, G_3 = L + 11/6, K_k = 6 (-1)^k / (k (k-1) (k-2) (k-3)),
+// so one loop over the degree gives g[B1,B2], g[B1,B2,B3] and g[B1,B2,B3,Bj] for every j, and the
+// entries with A follow by the difference recursion, whose gaps to A are wide.  Three logarithms and
+// some 20 terms, where the per-vertex tables sum up to six Taylor series for each of four vertices
+// (2400 FP64 operations against 500).
+__device__ __forceinline__ bool inv_sum_triple(const double x[4], const double f[4], double &out) {
+  const double s = tabs(x[0]) > tabs(x[3]) ? tabs(x[0]) : tabs(x[3]);
+  if (!(s > 0.0)) return false;
+  const double si = rcp_nr(s);
+  double u[4];
+  bool cl[3];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) u[i] = x[i] * si;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double a = u[i], b = u[i + 1];
+    cl[i] = (a > 0.0 && b - a <= kRhoShared * a) || (b < 0.0 && b - a <= kRhoShared * (-b));
+  }
+  if (!cl[1] || cl[0] == cl[2]) return false;
+  const bool low = cl[0];  // the lower three are together
+  const double A = low ? u[3] : u[0], fA = low ? f[3] : f[0];
+  const double B[3] = {low ? u[0] : u[1], low ? u[1] : u[2], low ? u[2] : u[3]};
+  const double fB[3] = {low ? f[0] : f[1], low ? f[1] : f[2], low ? f[2] : f[3]};
+  const double c = (B[0] + B[1] + B[2]) * (1.0 / 3.0), ci = rcp_nr(c);
+  double e[3];
+  float em = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    e[i] = fma(B[i], ci, -1.0);
+    em = fmaxf(em, fabsf((float)e[i]));
+  }
+  const double L = log(tabs(c));
+  // terms: e^n at 2^-58 (the kernel's unit roundoff with the growth of h_m on top)
+  int n = 2;
+  if (em > 1e-17f) n += (int)(-58.0f / __log2f(em < 0.5f ? em : 0.5f));
+  double h1 = 1.0, h2 = 1.0, h3 = 1.0, p0 = 1.0, p1 = 1.0, p2 = 1.0;  // h_m of e1; e1,e2; e1..e3; and of e1..e3, ej
+  double s1 = 3.0 * L + 1.0, s2 = 3.0 * L + 2.5, s30 = L + 11.0 / 6.0, s31 = s30, s32 = s30;
+  for (int m = 1; m <= n; ++m) {
+    h1 = e[0] * h1;
+    h2 = h1 + e[1] * h2;
+    h3 = h2 + e[2] * h3;
+    p0 = h3 + e[0] * p0;
+    p1 = h3 + e[1] * p1;
+    p2 = h3 + e[2] * p2;
+    // K_k = taylor_coef(k - 4)
+    const double k3 = taylor_coef<double>(m - 1);
+    const double k2 = m == 1 ? L + 11.0 / 6.0 : taylor_coef<double>(m - 2 < 0 ? 0 : m - 2);
+    const double k1 = m == 1 ? 3.0 * L + 2.5 : (m == 2 ? L + 11.0 / 6.0 : taylor_coef<double>(m - 3 < 0 ? 0 : m - 3));
+    s1 += k1 * h2;
+    s2 += k2 * h3;
+    s30 += k3 * p0;
+    s31 += k3 * p1;
+    s32 += k3 * p2;
+  }
+  const double g1 = c * c * s1, g2 = c * s2;
+  const double r1 = rcp_nr(B[0] - A), r2 = rcp_nr(B[1] - A), r3 = rcp_nr(B[2] - A);
+  const double LA = A == 0.0 ? 0.0 : log(tabs(A)), A2 = A * A;
+  const double a1 = (g0(B[0]) - A2 * A * LA) * r1, a2 = (g1 - a1) * r2, a3 = (g2 - a2) * r3;
+  const double d1 = (a1 - (3.0 * A2 * LA + A2)) * r1, d2 = (a2 - d1) * r2, d3 = (a3 - d2) * r3;
+  out = (fA * d3 + fB[0] * ((s30 - a3) * r1) + fB[1] * ((s31 - a3) * r2) + fB[2] * ((s32 - a3) * r3)) * si;
+  return true;
+}
+
 // the shared table where it applies, else the per-vertex table
 template <typename T> __device__ __forceinline__ T inv_sum_fast(const T x[4], const T f[4]) {
   T r;

@@ -23,9 +23,9 @@
 // warp 16 cycles of the FP64 pipe whatever its lanes need: all pieces wait in queues by their
 // spread, so that a round of 32 runs mean_series to the length its queue needs (K = 12 for most
 // whole tetrahedra of a 24^3 mesh, 28 for the longest of any 32 neighbours).
-// table_round: the long tiers of mean_series, then the shared divided-difference table, and for
-// what that leaves (three clustered knots; near-degenerate knots of the mixed form, in FP64) the
-// per-vertex table with four lanes per piece.
+// table_round: the long tiers of mean_series, then the shared divided-difference table, then (FP64
+// form, and near-degenerate knots of the mixed form) its triple-cluster case, and for what is left
+// the per-vertex table with four lanes per piece.
 // Bound: instruction issue (mixed: 2.2 warp instructions per SM cycle), the FP64 pipe (FP64
 // form: busy 75-80%).  Measured per q, weights and reduction, before (classification by loading
 // every item's energies, one lane per cut item, a global queue and three more kernels for it,
@@ -134,6 +134,15 @@ __device__ __noinline__ double table_round(const PieceQueue<typename std::condit
     T v;
     if (inv_sum_shared(d, f, v)) {
       acc = (double)(wv * v);
+      left = false;
+    }
+  }
+  if (FP64 ? left : (left && fp)) {
+    const double xd[4] = {(double)d[0], (double)d[1], (double)d[2], (double)d[3]};
+    const double fd[4] = {(double)f[0], (double)f[1], (double)f[2], (double)f[3]};
+    double v;
+    if (inv_sum_triple(xd, fd, v)) {
+      acc = (double)wv * v;
       left = false;
     }
   }

@@ -100,3 +100,9 @@ extern "C" int host_short_series(const float *d, const float *f, float *v, float
   *w = series_sum(d, f);
   return 1;
 }
+
+// three clustered knots: the shared evaluation (0: not its case) and the per-vertex table
+extern "C" int host_triple(const double *x, const double *f, double *v, double *w) {
+  *w = inv_sum_table(x, f);
+  return inv_sum_triple(x, f, *v) ? 1 : 0;
+}

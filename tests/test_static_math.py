@@ -7,7 +7,9 @@ Mean series: a dozen roundings at the end and offsets exact to one each, amplifi
 (1 + R)/(1 - R) = 8.1 at the widest tier: 12 x 8.1 x 2^-53 = 1.1e-14; below R = 0.3 the factor is
 1.9: 2.6e-15.  Short recurrence: both forms carry some ten roundings of 2^-24, amplified by
 (1 + r)/(1 - r) = 5.7 at r = 0.7: 10 x 5.7 x 2^-24 = 3.4e-6; their mean difference, which the
-common truncation rule keeps from being a bias, over N samples below that over sqrt(N)."""
+common truncation rule keeps from being a bias, over N samples below that over sqrt(N).
+Triple clusters: sums of terms of size f/s (s the largest knot) divided by gaps of at least s/9
+to the fourth knot three times over: 9^3 x 20 roundings x 2^-53 = 1.6e-12 of f/s."""
 import ctypes as ct
 import os
 import subprocess
@@ -102,3 +104,22 @@ def test_short_recurrence_is_series_sum(H, spread):
     diff = np.array(diff)
     assert len(diff) > 1000 and np.max(np.abs(diff)) < 3.4e-6
     assert abs(diff.mean()) < 3.4e-6 / np.sqrt(len(diff))
+
+
+@pytest.mark.parametrize("width", [0.0, 1e-14, 1e-9, 1e-4, 0.02, 0.06])
+@pytest.mark.parametrize("where", ["apart", "zero", "near"])
+def test_triple_cluster_matches_the_table(H, width, where):
+    rng = np.random.default_rng(24)
+    v, w = ct.c_double(), ct.c_double()
+    done = 0
+    for _ in range(400):
+        c = rng.choice([-1.0, 1.0]) * rng.uniform(0.2, 2.0)
+        a = {"apart": rng.uniform(-3.0, 3.0), "zero": 0.0, "near": c * rng.choice([0.6, 1.6])}[where]
+        x = np.sort(np.concatenate([c * (1.0 + width * rng.uniform(-1.0, 1.0, 3)), [a]]))
+        f = rng.uniform(0.0, 1.0, 4)
+        if not H.host_triple(_p(x), _p(f), ct.byref(v), ct.byref(w)):
+            assert abs(a - c) < 0.3 * abs(c)  # all four together: not this case
+            continue
+        done += 1
+        assert abs(v.value - w.value) < 1.6e-12 * f.sum() / np.max(np.abs(x)), (x, f, v.value, w.value)
+    assert done > 250
