@@ -623,32 +623,39 @@ template <typename T> __device__ __forceinline__ bool inv_sum_shared(const T x[4
 #pragma unroll
   for (int p = 0; p < 3; ++p) {
     const T d = u[p + 1] - u[p];
-    if (!cl[p] && !(d > T(0))) {  // two knots at 0 (a tie elsewhere is clustered): the limits
-      G1[p] = T(0);               // g'(0) = 0 and g''(0)/2 = 0
-      HL[p] = T(0);
-      HR[p] = T(0);
-    } else if (!cl[p]) {
-      const T r = rcp(d);
-      G1[p] = (g[p + 1] - g[p]) * r;
-      HL[p] = (G1[p] - gp[p]) * r;
-      HR[p] = (gp[p + 1] - G1[p]) * r;
-    } else {
-      const T a = u[p], y = d * rcp(a), Lp = L[p];
-      const T g2 = T(6) * a * Lp + T(5) * a, g3 = T(6) * Lp + T(11);
-      // T_4 = a y^2 / 4; successive terms: T_{k+1} = -T_k (k-3) y / (k+1)
-      T t = T(0.25) * a * y * y;
-      T s0 = T(0), s1 = T(0);
+    const bool zero = !(d > T(0));  // two knots at 0 (a tie elsewhere is clustered): the limits
+    const T r = rcp(zero ? T(1) : d);  // g'(0) = 0 and g''(0)/2 = 0
+    G1[p] = zero ? T(0) : (g[p + 1] - g[p]) * r;
+    HL[p] = zero ? T(0) : (G1[p] - gp[p]) * r;
+    HR[p] = zero ? T(0) : (gp[p + 1] - G1[p]) * r;
+  }
+  // the clustered pairs, one after the other whichever they are (at most two: the lanes of a warp
+  // share the loop, where a series at each of the three places ran in nearly every warp)
+  unsigned cm = (cl[0] ? 1u : 0u) | (cl[1] ? 2u : 0u) | (cl[2] ? 4u : 0u);
 #pragma unroll 1
-      for (int k = 4; k < 4 + Num<T>::kmax; ++k) {
-        s0 += t;
-        s1 += T(k - 1) * t;
-        if (tabs(t) <= Num<T>::tol * (tabs(s0) + tabs(g2) + tabs(g3))) break;
-        t *= -T(k - 3) * y / T(k + 1);
-      }
-      HL[p] = T(0.5) * g2 + d * g3 * T(1.0 / 6.0) + s0;
-      HR[p] = T(0.5) * g2 + d * g3 * T(1.0 / 3.0) + s1;
-      G1[p] = gp[p] + d * (T(0.5) * g2 + d * g3 * T(1.0 / 6.0) + s0);
+  while (cm) {
+    const bool c0 = cm & 1u, c1 = (cm & 3u) == 2u;
+    const T a = c0 ? u[0] : (c1 ? u[1] : u[2]), b = c0 ? u[1] : (c1 ? u[2] : u[3]);
+    const T Lp = c0 ? L[0] : (c1 ? L[1] : L[2]), gpp = c0 ? gp[0] : (c1 ? gp[1] : gp[2]);
+    const T d = b - a, y = d * rcp(a);
+    const T g2 = T(6) * a * Lp + T(5) * a, g3 = T(6) * Lp + T(11);
+    // T_4 = a y^2 / 4; successive terms: T_{k+1} = -T_k (k-3) y / (k+1)
+    T t = T(0.25) * a * y * y;
+    T s0 = T(0), s1 = T(0);
+#pragma unroll 1
+    for (int k = 4; k < 4 + Num<T>::kmax; ++k) {
+      s0 += t;
+      s1 += T(k - 1) * t;
+      if (tabs(t) <= Num<T>::tol * (tabs(s0) + tabs(g2) + tabs(g3))) break;
+      t *= -T(k - 3) * y / T(k + 1);
     }
+    const T hl = T(0.5) * g2 + d * g3 * T(1.0 / 6.0) + s0, hr = T(0.5) * g2 + d * g3 * T(1.0 / 3.0) + s1;
+    const T g1 = gpp + d * (T(0.5) * g2 + d * g3 * T(1.0 / 6.0) + s0);
+    const bool c2 = !c0 && !c1;
+    G1[0] = c0 ? g1 : G1[0], HL[0] = c0 ? hl : HL[0], HR[0] = c0 ? hr : HR[0];
+    G1[1] = c1 ? g1 : G1[1], HL[1] = c1 ? hl : HL[1], HR[1] = c1 ? hr : HR[1];
+    G1[2] = c2 ? g1 : G1[2], HL[2] = c2 ? hl : HL[2], HR[2] = c2 ? hr : HR[2];
+    cm &= cm - 1u;
   }
   const T r02 = rcp(u[2] - u[0]), r13 = rcp(u[3] - u[1]), r03 = rcp(u[3] - u[0]);
   const T G012 = (G1[1] - G1[0]) * r02, G123 = (G1[2] - G1[1]) * r13;
