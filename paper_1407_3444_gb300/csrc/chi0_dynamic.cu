@@ -52,12 +52,14 @@
 // reduction per moment, in the warp's order; 26 KB of shared memory per warp for them had kept an
 // SM at four warps): bitwise reproducible for a given launch shape.
 //
-// Bound: instruction issue and dependent latency (FP32: 12 warps per SM, 1.6 instructions per
-// cycle), the FP64 pipe (FP64: 74% busy while an SM has work).  Measured per 256-frequency pass,
-// before (one (piece, frequency range) at a time, 64-bit float conversions and atomics, batches of
-// 32 tetrahedra) and now: 64 x 64 x 16 mesh, 10 bands FP32 10.5 -> 7.0 ms, 32^3, 80 bands FP32 836
-// -> 590 ms; 16 x 16 x 8, 10 bands, 128 frequencies FP64 58-100 -> 13 ms; Im alone, 32^3, 12 bands
-// FP32 3.3 -> 0.8 ms.
+// Bound: instruction issue, dependent latency and instruction fetch (FP32: 12 warps per SM), the FP64
+// pipe (FP64).  Share of the FP32 kernel's time (32^3, 80 bands; time that goes when a part is left
+// out): near pairs 25% and the entries they leave 17%, own pairs 12%, delta terms 5%, own moments 4%,
+// carving, boxes and box moments 10%.  Measured per 256-frequency pass, before (one (piece, frequency
+// range) at a time, 64-bit float conversions and atomics, batches of 32 tetrahedra, the per-vertex
+// table for every left entry) and now: 64 x 64 x 16 mesh, 10 bands FP32 10.5 -> 3.8 ms (k_dyn_fallback
+// 0.35 of it), 32^3, 80 bands FP32 836 -> 395 ms; 16 x 16 x 8, 10 bands, 128 frequencies FP64
+// 58-100 -> 6.2 ms; Im alone, 32^3, 12 bands FP32 3.3 -> 0.77 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -151,15 +153,17 @@ template <bool FP64> __host__ __device__ constexpr int slot_base(int b) {
                                               : kBoxFine * S::KF + kBoxG * S::KG + (b - kBoxFine - kBoxG) * S::KW);
 }
 
-// the pass's boxes and its frequencies in ascending |w|, in the kernels' precision (written by
-// k_box_setup)
-template <typename T> struct BoxTab {
+// the pass's boxes, and with them its frequencies in ascending |w|, in the kernels' precision
+// (written by k_box_setup)
+template <typename T> struct BoxGeo {
   T C[kBoxes], R[kBoxes];  // centre and radius
   T lowG[kBoxG + 1];       // lower edges x_b of the geometric boxes (x = c - u_max)
   T W0, x0, umax;
   int on;
-  T om[kNWPass];      // |w| ascending
-  T oml[kNWPass];     // |w| - (T)|w|
+};
+template <typename T> struct BoxTab : BoxGeo<T> {
+  T om[kNWPass];        // |w| ascending
+  T oml[kNWPass];       // |w| - (T)|w|
   short rank[kNWPass];  // place of frequency i in that order
 };
 
@@ -226,7 +230,7 @@ __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict_
 }
 
 // box of a final tetrahedron with midpoint c and half-width s (-1: none, evaluate directly)
-template <typename T> __device__ __forceinline__ int box_of(T c, T s, const BoxTab<T> &tb) {
+template <typename T> __device__ __forceinline__ int box_of(T c, T s, const BoxGeo<T> &tb) {
   if (!tb.on) return -1;
   const T x = c - tb.umax;
   int wide = -1;
@@ -376,7 +380,9 @@ __device__ __noinline__ typename std::conditional<FP64, double, float>::type nea
     if (series_ok(xx, Num<float>::kappa)) return series_sum(xx, f);
     float y[4];
     if (!mixed_knots(y, xx, tau)) {
+      float v;
       if (series_ok(y, Num<float>::kappa_long)) return series_sum(y, f);
+      if (inv_sum_triple_table(y, f, v)) return v;
       return inv_sum_table(y, f);
     }
     ++nfp64;
@@ -448,7 +454,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   __shared__ T s_w[kNWPass];                 // |w| ascending
   __shared__ T s_wl[FP64 ? 1 : kNWPass];     // FP32 path: |w| - (float)|w|
   __shared__ short s_rng[kBoxFine][3];  // frequencies a fine box leaves to its pieces: - term [lo, hi), + term [0, p)
-  __shared__ BoxTab<T> s_tab;
+  __shared__ BoxGeo<T> s_tab;
   extern __shared__ __align__(16) unsigned char s_dyn[];  // FP32: box sums, low and high words [NS]
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
@@ -464,7 +470,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   FbEnt<T> *gfb = (FbEnt<T> *)db.fb + gwarp * kFbCap;
   {
     const BoxTab<T> *src = (const BoxTab<T> *)db.box_tab;
-    constexpr int nwords = (int)(offsetof(BoxTab<T>, om) / 4);
+    constexpr int nwords = (int)(sizeof(BoxGeo<T>) / 4);
 #pragma unroll 1
     for (int i = threadIdx.x; i < nwords; i += blockDim.x) ((int *)&s_tab)[i] = ((const int *)src)[i];
 #pragma unroll 1
@@ -1159,8 +1165,9 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
 
 // FP32 kernel: what is left in the warps' fallback buffers, one entry per thread, into the
 // fixed-point rows.  At the end of k_dynamic each warp would walk its last few hundred entries
-// through the per-vertex table (up to 50 us a round, most of its lanes in the FP64 branch of
+// (the per-vertex table took up to 50 us a round, most of its lanes in the FP64 branch of
 // near-degenerate knots) while finished SMs idle: 30% of the time of a 64 x 64 x 16 pass.
+// 64 x 64 x 16, 10 bands: 0.35 ms a pass, 1.05 with the per-vertex table for every entry.
 __global__ void __launch_bounds__(128) k_dyn_fallback(DynBufs db, int nbuf, int nrows, float tau,
                                                       unsigned long long *__restrict__ counters) {
   unsigned long long *row = db.fx + (size_t)(blockIdx.x % nrows) * 2 * kNWPass;
