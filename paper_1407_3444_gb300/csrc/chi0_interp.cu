@@ -35,7 +35,14 @@ __device__ __forceinline__ void st(void *C, int dtype, long long i, Cd v) {
   else ((double2 *)C)[i] = make_double2(v.x, v.y);
 }
 
-// one thread per (corner, band)
+// One thread per (corner, band).  Bound: the FP64 pipe (some 30 operations per corner, band and
+// orbital).  NO: orbitals at most (0: any number), whose sums then stay in registers between the norm
+// and the store; the weights are folded into the phases, and the norms go through one reciprocal
+// square root.  33 x 32 x 31 corners, 9 orbitals, complex128: 0.25 ms (0.40 with unfolded weights, the
+// sums formed twice, square roots and divisions).  The line at 16: 24^3 corners, complex128, registers
+// against the general form: 10 orbitals 135 against 184 us, 16 orbitals 305 against 423 us (64 of the
+// registers are sums there; more would leave too few warps).
+template <int NO>
 __global__ void __launch_bounds__(256) k_interp_kq(Grid g, const double *__restrict__ E, const void *__restrict__ C,
                                                    int dtype, double q0, double q1, double q2,
                                                    double *__restrict__ Eq, void *__restrict__ Cq) {
@@ -75,37 +82,63 @@ __global__ void __launch_bounds__(256) k_interp_kq(Grid g, const double *__restr
   for (int v = 0; v < 4; ++v) e += w[v] * E[cc[v] * g.nb + b];
   Eq[c * g.nb + b] = e;
   if (!C) return;
-  // phases of corners 1..3 relative to corner 0: <v_0|v_i>
-  Cd ph[4] = {{1.0, 0.0}, {1.0, 0.0}, {1.0, 0.0}, {1.0, 0.0}};
-  for (int v = 1; v < 4; ++v) {
-    double re = 0.0, im = 0.0;
+  // phases of corners 1..3 relative to corner 0, conj(<v_0|v_i>) / |.|, times the weights
+  const long long at = b, st_o = g.nb;
+  Cd ph[4] = {{w[0], 0.0}, {w[1], 0.0}, {w[2], 0.0}, {w[3], 0.0}};
+  {
+    double re[3] = {0.0, 0.0, 0.0}, im[3] = {0.0, 0.0, 0.0};
     for (int o = 0; o < g.norb; ++o) {
-      const Cd a = ld(C, dtype, (cc[0] * g.norb + o) * g.nb + b), z = ld(C, dtype, (cc[v] * g.norb + o) * g.nb + b);
-      re += a.x * z.x + a.y * z.y;
-      im += a.x * z.y - a.y * z.x;
+      const Cd a = ld(C, dtype, cc[0] * g.norb * st_o + o * st_o + at);
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        const Cd z = ld(C, dtype, (cc[v + 1] * g.norb + o) * st_o + at);
+        re[v] += a.x * z.x + a.y * z.y;
+        im[v] += a.x * z.y - a.y * z.x;
+      }
     }
-    const double m = sqrt(re * re + im * im);
-    if (m > 0.0) ph[v] = Cd{re / m, -im / m};  // conj(<v_0|v_i>) / |.|
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      const double m2 = re[v] * re[v] + im[v] * im[v];
+      if (m2 > 0.0) {
+        const double r = w[v + 1] * rsqrt(m2);
+        ph[v + 1] = Cd{re[v] * r, -im[v] * r};
+      }
+    }
   }
+  // the weighted sum, orbital by orbital
+  auto mix = [&](int o) {
+    const Cd z0 = ld(C, dtype, (cc[0] * g.norb + o) * st_o + at);
+    double sx = ph[0].x * z0.x, sy = ph[0].x * z0.y;
+#pragma unroll
+    for (int v = 1; v < 4; ++v) {
+      const Cd z = ld(C, dtype, (cc[v] * g.norb + o) * st_o + at);
+      sx += z.x * ph[v].x - z.y * ph[v].y;
+      sy += z.x * ph[v].y + z.y * ph[v].x;
+    }
+    return Cd{sx, sy};
+  };
   double nrm = 0.0;
-  for (int o = 0; o < g.norb; ++o) {
-    double sx = 0.0, sy = 0.0;
-    for (int v = 0; v < 4; ++v) {
-      const Cd z = ld(C, dtype, (cc[v] * g.norb + o) * g.nb + b);
-      sx += w[v] * (z.x * ph[v].x - z.y * ph[v].y);
-      sy += w[v] * (z.x * ph[v].y + z.y * ph[v].x);
+  if (NO > 0) {  // at most NO orbitals: kept in registers until the norm is known
+    Cd s[NO > 0 ? NO : 1];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) {
+      s[o] = o < g.norb ? mix(o) : Cd{0.0, 0.0};
+      nrm += s[o].x * s[o].x + s[o].y * s[o].y;
     }
-    nrm += sx * sx + sy * sy;
-  }
-  const double sc = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
-  for (int o = 0; o < g.norb; ++o) {
-    double sx = 0.0, sy = 0.0;
-    for (int v = 0; v < 4; ++v) {
-      const Cd z = ld(C, dtype, (cc[v] * g.norb + o) * g.nb + b);
-      sx += w[v] * (z.x * ph[v].x - z.y * ph[v].y);
-      sy += w[v] * (z.x * ph[v].y + z.y * ph[v].x);
+    const double sc = nrm > 0.0 ? rsqrt(nrm) : 0.0;
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+      if (o < g.norb) st(Cq, dtype, (c * g.norb + o) * st_o + at, Cd{s[o].x * sc, s[o].y * sc});
+  } else {
+    for (int o = 0; o < g.norb; ++o) {
+      const Cd s = mix(o);
+      nrm += s.x * s.x + s.y * s.y;
     }
-    st(Cq, dtype, (c * g.norb + o) * g.nb + b, Cd{sx * sc, sy * sc});
+    const double sc = nrm > 0.0 ? rsqrt(nrm) : 0.0;
+    for (int o = 0; o < g.norb; ++o) {
+      const Cd s = mix(o);
+      st(Cq, dtype, (c * g.norb + o) * st_o + at, Cd{s.x * sc, s.y * sc});
+    }
   }
 }
 
@@ -114,7 +147,11 @@ __global__ void __launch_bounds__(256) k_interp_kq(Grid g, const double *__restr
 cudaError_t launch_interp_kq(const Grid &g, const double *E, const void *C, int c64, const double q[3], double *Eq,
                              void *Cq, cudaStream_t s) {
   const long long n = g.nc * g.nb;
-  k_interp_kq<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(g, E, C, c64 ? 0 : 1, q[0], q[1], q[2], Eq, Cq);
+  const unsigned blocks = (unsigned)((n + 255) / 256);
+  const int dt = c64 ? 0 : 1;
+  if (g.norb <= 10) k_interp_kq<10><<<blocks, 256, 0, s>>>(g, E, C, dt, q[0], q[1], q[2], Eq, Cq);
+  else if (g.norb <= 16) k_interp_kq<16><<<blocks, 256, 0, s>>>(g, E, C, dt, q[0], q[1], q[2], Eq, Cq);
+  else k_interp_kq<0><<<blocks, 256, 0, s>>>(g, E, C, dt, q[0], q[1], q[2], Eq, Cq);
   return cudaGetLastError();
 }
 
