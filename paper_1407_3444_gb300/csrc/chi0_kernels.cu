@@ -33,7 +33,7 @@ using grid::tet_corners;
 using grid::warp_sum;
 
 using grid::d2f_int;
-template <typename T> __device__ __forceinline__ T cvt(double x);
+template <typename T> __device__ __forceinline__ T cvt(double x) { return (T)x; }
 template <> __device__ __forceinline__ float cvt<float>(double x) { return d2f_int(x); }
 template <typename T> __device__ __forceinline__ T cvt(float x) { return (T)x; }
 
@@ -79,44 +79,125 @@ __global__ void __launch_bounds__(kThreads) k_overlap(const __grid_constant__ Ov
   }
 }
 
-// Warp per corner for small blocks (norb * w <= kOvlSmall): both eigenvector blocks
-// C_k[:, lo:hi] and C_{k+q}[:, lo:hi] are read once, coalesced, into shared memory in
-// the arithmetic precision, then the lanes form the w x w |overlap|^2 block.
+// Small blocks (norb * w <= kOvlSmall): a warp takes a run of corners, as many as its lanes hold
+// 3 x 3 tiles of (m, n) for (three corners at w = 9, two at w = 10, 12; past 25 tiles one, whose
+// tiles the lanes share out).  The eigenvector blocks C_k[:, lo:hi] and C_{k+q}[:, lo:hi] are read
+// once, coalesced, into shared memory in the arithmetic precision; a lane then reads six complex
+// numbers per orbital for its nine products, where one output per lane and step reads eighteen; and
+// the blocks leave through shared memory, coalesced.
+// Bound: FP32 memory and the shared-memory traffic of the tiles; FP64 the FP64 pipe (four FMAs per
+// product; written as re += xr * yr + xi * yi they were six operations).  One output per lane, one
+// corner at a time: 48^3 corners x 9 bands FP32 113 us, now 87; FP64, by the general form (one
+// output per thread, operands from the caches): 24^3 x 9 bands 114 us, now 85.
 constexpr int kOvlSmall = 256;
+constexpr int kOvlBuf = 320;  // complex numbers staged a side: two corners of 12 x 12
+template <typename T> constexpr int kOvlThreads = sizeof(T) == 8 ? 128 : 256;
+__device__ __forceinline__ void conj_mul_add(float &re, float &im, float2 x, float2 y) {
+  re += x.x * y.x + x.y * y.y;
+  im += x.x * y.y - x.y * y.x;
+}
+__device__ __forceinline__ void conj_mul_add(double &re, double &im, double2 x, double2 y) {
+  re = fma(x.x, y.x, re);
+  im = fma(x.x, y.y, im);
+  re = fma(x.y, y.y, re);
+  im = fma(-x.y, y.x, im);
+}
 template <typename CT, typename CTq, typename T>
-__global__ void __launch_bounds__(kThreads) k_overlap_small(const __grid_constant__ OverlapArgs A,
-                                                             const CT *__restrict__ C, int explicit_q) {
+__global__ void __launch_bounds__(kOvlThreads<T>, 4) k_overlap_small(const __grid_constant__ OverlapArgs A,
+                                                                  const CT *__restrict__ C, int explicit_q) {
+  using V = typename std::conditional<sizeof(T) == 8, double2, float2>::type;
+  constexpr int kW = kOvlThreads<T> / 32;
   const Grid &g = A.g;
   const Q &q = A.q[blockIdx.y];
   const CTq *Cb = explicit_q ? (const CTq *)q.Cq : (const CTq *)C;
   T *W2 = (T *)A.W2[blockIdx.y];
-  __shared__ T sA[kWarps][2][kOvlSmall], sB[kWarps][2][kOvlSmall];
+  __shared__ V sm[kW][2][kOvlBuf];  // both sides; then the outputs
+  __shared__ long long s_ck[kW][32];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int w = q.hi - q.lo, no = g.norb, nel = no * w;
-  for (long long c = (long long)blockIdx.x * kWarps + wib; c < g.nc; c += (long long)gridDim.x * kWarps) {
-    const long long ck = explicit_q ? c : shift_corner(g, c, q.shift);
-    for (int i = lane; i < nel; i += 32) {
-      const int o = i / w, mm = i - o * w;
-      const CT x = C[(c * no + o) * g.nb + q.lo + mm];
-      const CTq y = Cb[(ck * no + o) * g.nb + q.lo + mm];
-      sA[wib][0][i] = cvt<T>(x.x);
-      sA[wib][1][i] = cvt<T>(x.y);
-      sB[wib][0][i] = cvt<T>(y.x);
-      sB[wib][1][i] = cvt<T>(y.y);
-    }
+  V *sA = sm[wib][0], *sB = sm[wib][1];
+  const int w = q.hi - q.lo, no = g.norb, nel = no * w, ww = w * w;
+  const int tr = (w + 2) / 3, nt = tr * tr;  // tiles a side, tiles a corner
+  int cpw = nt >= 32 ? 1 : 32 / nt;          // corners a step
+  cpw = min(cpw, kOvlBuf / nel);
+  const bool through = nt <= 32 && cpw * ww <= 2 * kOvlBuf;  // one round of tiles, and the outputs fit the buffers
+  const int st_o = 32 / w, st_m = 32 - st_o * w, o0 = lane / w, m0 = lane - o0 * w;  // staging steps
+  const int myj = nt >= 32 ? 0 : lane / nt, mytile = nt >= 32 ? lane : lane - myj * nt;
+  for (long long c0 = ((long long)blockIdx.x * kW + wib) * cpw; c0 < g.nc; c0 += (long long)gridDim.x * kW * cpw) {
+    const int nj = (int)(g.nc - c0 < cpw ? g.nc - c0 : cpw);
+    if (lane < nj) s_ck[wib][lane] = explicit_q ? c0 + lane : shift_corner(g, c0 + lane, q.shift);
     __syncwarp();
-    for (int out = lane; out < w * w; out += 32) {
-      const int mm = out / w, nn = out - mm * w;
-      T re = T(0), im = T(0);
-      for (int o = 0; o < no; ++o) {
-        const T xr = sA[wib][0][o * w + mm], xi = sA[wib][1][o * w + mm];
-        const T yr = sB[wib][0][o * w + nn], yi = sB[wib][1][o * w + nn];
-        re += xr * yr + xi * yi;  // conj(x) * y
-        im += xr * yi - xi * yr;
+    {
+      // element i = (corner j, orbital o, band mm), i = lane, lane + 32, ...
+      int j = 0, o = o0, mm = m0;
+      while (o >= no) {
+        o -= no;
+        ++j;
       }
-      W2[c * w * w + out] = re * re + im * im;
+      const CT *Ck = C + c0 * no * g.nb + q.lo;
+      for (int i = lane; i < nj * nel; i += 32) {
+        const CT x = Ck[(j * no + o) * g.nb + mm];
+        const CTq y = Cb[(s_ck[wib][j] * no + o) * g.nb + q.lo + mm];
+        V a, b;
+        a.x = cvt<T>(x.x);
+        a.y = cvt<T>(x.y);
+        b.x = cvt<T>(y.x);
+        b.y = cvt<T>(y.y);
+        sA[i] = a;
+        sB[i] = b;
+        mm += st_m;
+        o += st_o;
+        if (mm >= w) {
+          mm -= w;
+          ++o;
+        }
+        while (o >= no) {
+          o -= no;
+          ++j;
+        }
+      }
     }
     __syncwarp();
+    for (int base = 0; base < (nt >= 32 ? nt : 1); base += 32) {  // warp-uniform
+      const int t = base + mytile;
+      const bool on = myj < nj && t < nt;
+      const int ti = on ? t / tr : 0, tj = on ? t - ti * tr : 0;
+      int mi[3], ni[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        mi[k] = min(ti * 3 + k, w - 1);
+        ni[k] = min(tj * 3 + k, w - 1);
+      }
+      const V *a = sA + (on ? myj : 0) * nel, *b = sB + (on ? myj : 0) * nel;
+      T re[3][3] = {}, im[3][3] = {};
+      for (int o = 0; o < no; ++o, a += w, b += w) {
+        V x[3], y[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          x[k] = a[mi[k]];
+          y[k] = b[ni[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+          for (int l = 0; l < 3; ++l) conj_mul_add(re[k][l], im[k][l], x[k], y[l]);
+      }
+      if (through) __syncwarp();  // every lane has read its operands
+      T *out = through ? reinterpret_cast<T *>(sA) + myj * ww : W2 + (c0 + myj) * ww;
+      if (on) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+          for (int l = 0; l < 3; ++l)
+            if (ti * 3 + k < w && tj * 3 + l < w)
+              out[(ti * 3 + k) * w + tj * 3 + l] = re[k][l] * re[k][l] + im[k][l] * im[k][l];
+      }
+    }
+    __syncwarp();
+    if (through) {
+      const T *o = reinterpret_cast<const T *>(sA);
+      for (int i = lane; i < nj * ww; i += 32) W2[c0 * ww + i] = o[i];
+      __syncwarp();
+    }
   }
 }
 
@@ -233,14 +314,18 @@ cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int f
   const int blocks = (int)(nb < device_sms() * 16 ? nb : device_sms() * 16);
   if (blocks <= 0) return cudaSuccess;
   const bool ex = a.q[0].Cq != nullptr;  // (a group's q points are all explicit or all shifts)
-  const bool small = (long long)g.norb * w <= kOvlSmall && !fp64;
-  if (small) {
+  if ((long long)g.norb * w <= kOvlSmall) {
+    const long long warps = fp64 ? 4 : 8, nbw = (g.nc + warps - 1) / warps, cap = device_sms() * 4;  // resident blocks
+    const dim3 bw((unsigned)(nbw < cap ? nbw : cap), (unsigned)a.nq);
+    if (fp64) {
+      if (dtype == DT_C128) k_overlap_small<double2, double2, double><<<bw, 128, 0, s>>>(a, (const double2 *)C, ex ? 1 : 0);
+      else k_overlap_small<float2, float2, double><<<bw, 128, 0, s>>>(a, (const float2 *)C, ex ? 1 : 0);
+      return cudaGetLastError();
+    }
     // k side in complex64 (the plan's copy when the inputs are complex128)
     const float2 *Ck = (const float2 *)(C32 ? C32 : C);
-    long long nbw = (g.nc + kWarps - 1) / kWarps;
-    const dim3 bw((unsigned)(nbw < device_sms() * 8 ? nbw : device_sms() * 8), (unsigned)a.nq);
-    if (ex && dtype == DT_C128) k_overlap_small<float2, double2, float><<<bw, kThreads, 0, s>>>(a, Ck, 1);
-    else k_overlap_small<float2, float2, float><<<bw, kThreads, 0, s>>>(a, Ck, ex ? 1 : 0);
+    if (ex && dtype == DT_C128) k_overlap_small<float2, double2, float><<<bw, 256, 0, s>>>(a, Ck, 1);
+    else k_overlap_small<float2, float2, float><<<bw, 256, 0, s>>>(a, Ck, ex ? 1 : 0);
     return cudaGetLastError();
   }
   const dim3 bg((unsigned)blocks, (unsigned)a.nq);
