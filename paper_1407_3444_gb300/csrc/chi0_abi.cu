@@ -525,8 +525,9 @@ static int enqueue_overlap(chi0_plan_t *p, const Q *q, int n, Timer &tm, bool tc
   return CHI0_OK;
 }
 
-// bounds and FP32 energies of n q points with explicit k+q energies into slots 0 .. n - 1
-static int enqueue_bands(chi0_plan_t *p, const Q *q, int n, Timer &tm) {
+// bounds and FP32 energies (lo: with their remainders, for the dynamic weights) of n q points with
+// explicit k+q energies into slots 0 .. n - 1
+static int enqueue_bands(chi0_plan_t *p, const Q *q, int n, bool lo, Timer &tm) {
   const Grid &g = p->g;
   const size_t ncb = (size_t)g.nc * g.nb;
   const bool mixed = p->opts.precision == CHI0_PREC_MIXED;
@@ -535,7 +536,7 @@ static int enqueue_bands(chi0_plan_t *p, const Q *q, int n, Timer &tm) {
   a.out = bounds_at(p->boundsq_d, g.nc);
   a.stride_c = 4 * (size_t)g.nc;
   a.E32 = mixed ? p->Eq32_d : nullptr;
-  a.E32lo = mixed ? p->Eq32_d + ncb : nullptr;
+  a.E32lo = mixed && lo ? p->Eq32_d + ncb : nullptr;
   a.stride_e = 2 * ncb;
   tm.start(CHI0_K_BANDS);
   CK(p, launch_bands(a, n, g.nc, g.nb, g.ef, p->stream));
@@ -576,7 +577,7 @@ static int enqueue_static(chi0_plan_t *p, const chi0_q_t *qs, int nq, double *ou
     }
     if (outP) CK(p, cudaMemsetAsync(p->pairs_fx_d, 0, sizeof(unsigned long long) * n * wp * wp, s));
     int rc = enqueue_overlap(p, q, n, tm, tc);
-    if (!rc && ex) rc = enqueue_bands(p, q, n, tm);
+    if (!rc && ex) rc = enqueue_bands(p, q, n, false, tm);
     if (rc) return rc;
     StaticArgs a{};
     a.g = g;
@@ -649,7 +650,7 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
     if ((rc = enqueue_overlap(p, &q, 1, tm, tc))) return rc;
     const int ndos = static_blocks();
     if (q.gamma && (rc = enqueue_dos(p, q, 0, nullptr, tm))) return rc;
-    if (q.Eq && (rc = enqueue_bands(p, &q, 1, tm))) return rc;
+    if (q.Eq && (rc = enqueue_bands(p, &q, 1, true, tm))) return rc;
     const size_t ncb = (size_t)p->g.nc * p->g.nb;
     const BandBounds kb = bounds_at(p->bounds_d, p->g.nc), qb = q.Eq ? bounds_at(p->boundsq_d, p->g.nc) : kb;
     DynArgs a{};

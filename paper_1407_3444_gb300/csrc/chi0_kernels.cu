@@ -208,6 +208,9 @@ __global__ void __launch_bounds__(kOvlThreads<T>, 4) k_overlap_small(const __gri
 // band with not e > eF (every band from it on is empty).  For ascending energies occf = occ and
 // empf = emp but for levels at eF; neither order nor absence of NaN is relied on.
 // E32 (optional) receives the energies relative to eF in FP32 for the mixed-precision path.
+// Sides and FP32 values by integer operations where the value is a normal FP32 number: on the FP64
+// pipe two comparisons and a conversion took 16 cycles each per warp (48^3 corners x 9 bands: 16 us,
+// now 11 us).
 // A block reads a run of corners' energies coalesced, one energy per thread and step, notes
 // each one's side of eF in shared memory, and one thread per corner walks the notes; one
 // thread per corner walking the energies themselves took 16 us on a 48^3 mesh of 9 bands.
@@ -228,9 +231,12 @@ __global__ void __launch_bounds__(kThreads) k_bands(const __grid_constant__ Band
     const int ncb = (int)(nc - c0 < per ? nc - c0 : per);
     for (int i = threadIdx.x; i < ncb * nb; i += kThreads) {
       const double x = E[c0 * nb + i] - ef;
-      s_side[i] = (x < 0.0 ? 1 : 0) | (x > 0.0 ? 2 : 0);
+      const int hi = __double2hiint(x), mag = hi & 0x7fffffff;
+      const bool nan = mag > 0x7ff00000 || (mag == 0x7ff00000 && __double2loint(x) != 0);
+      const bool zero = (mag | __double2loint(x)) == 0;
+      s_side[i] = nan || zero ? 0 : (hi < 0 ? 1 : 2);
       if (E32) {
-        const float h = (float)x;
+        const float h = mag - 0x38100000 < 0x0fd00000 && mag >= 0x38100000 ? d2f_int(x) : (float)x;
         E32[c0 * nb + i] = h;
         if (E32lo) E32lo[c0 * nb + i] = (float)(x - (double)h);
       }
