@@ -279,20 +279,19 @@ def arithmetic_peaks(chi0):
 
 
 # Executed FP32 operations (FFMA counted twice, FADD, FMUL) per final tetrahedron of the mixed
-# static weight kernels on the Cr-like 48^3 workload (ncu instruction counters of k_static +
-# k_static_tab, before the long-series queue was compacted over the call: the same arithmetic
-# per piece now runs in k_tab_eval).  Their DRAM bytes per final tetrahedron (3.58 then) are
-# not reported: the kernels have changed since the counters were taken.
-FLOPS_PER_PIECE_MIXED = 202.6
+# static weight kernel on the Cr-like 48^3 workload (ncu instruction counters of k_static, three q
+# points).  DRAM bytes per final tetrahedron are not reported: 3.2 B, the |M|^2 table once.
+FLOPS_PER_PIECE_MIXED = 153.0
 TRAFFIC_PER_PIECE_MIXED = None
-# The same for the dynamic weight kernel per final tetrahedron over one pass of 256 frequencies
-# (ncu instruction counters of k_dynamic on a seeded sample of 16384 tetrahedra of the 80-band
-# 72^3 mesh, one q: the full mesh's mix of pieces; the FP64 kernel's FP64 operations likewise).
+# The same for the dynamic weight kernels per final tetrahedron over one pass of 256 frequencies
+# (ncu instruction counters of k_dynamic and k_dyn_fallback on a seeded sample of 16384 tetrahedra
+# of the 80-band 72^3 mesh, one q: the full mesh's mix of pieces; the FP64 kernel's FP64 operations
+# likewise).
 # DRAM bytes: not taken from the sample (its scattered tetrahedra defeat the caches that the
-# whole mesh uses); on whole meshes they fall per final tetrahedron as the mesh grows (29.3 B at
-# 24^3, 16.4 B at 48^3), so no per-unit figure scales to the 72^3 launch: None until counted there.
-FLOPS_PER_PIECE_DYN32 = 2987.4
-FLOPS_PER_PIECE_DYN64 = 6346.5
+# whole mesh uses), and on whole meshes they fall per final tetrahedron as the mesh grows, so no
+# per-unit figure scales to the 72^3 launch: None until counted there.
+FLOPS_PER_PIECE_DYN32 = 2780.7
+FLOPS_PER_PIECE_DYN64 = None
 TRAFFIC_PER_PIECE_DYN32 = None
 
 
@@ -564,7 +563,7 @@ def run_ours(args):
         launches_w = s1.launches[chi0.CHI0_K_STATIC] - s0.launches[chi0.CHI0_K_STATIC]
         fpu, tpu, kname = (FLOPS_PER_PIECE_MIXED if args.workload == "cr" else None,
                            TRAFFIC_PER_PIECE_MIXED if args.workload == "cr" else None,
-                           "static weights (k_static + k_static_tab, mixed)")
+                           "static weights (k_static, mixed)")
         uname = "final tetrahedron"
     else:
         k_ms = stage_ms(s0, s1, chi0.CHI0_K_DYNAMIC)

@@ -30,8 +30,8 @@
 // form: busy 75-80%).  Measured per q, weights and reduction, before (classification by loading
 // every item's energies, one lane per cut item, a global queue and three more kernels for it,
 // FP64 series with a convergence test and a table past knot ratio 5/3) and now: 48^3 x 9 bands
-// mixed 708 -> 330 us, 32^3 x 40 bands (windows of 4 to 40) mixed 3.0 -> 1.05 ms, 24^3 x 9 bands
-// FP64 8.5 -> 0.75 ms, 16^3 free electron FP64 1.9 ms -> 40 us (32 q in one launch).
+// mixed 708 -> 333 us, 32^3 x 40 bands (windows of 4 to 40) mixed 3.0 -> 1.03 ms, 24^3 x 9 bands
+// FP64 8.5 -> 0.62 ms, 16^3 free electron FP64 1.9 ms -> 23 us (32 q in one launch).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
