@@ -585,9 +585,11 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
         const int b = s_qb[wib][sl];
         const T half = (e3 - e0) * T(0.5), c = D0h + (e0 + e3) * T(0.5), near = half * T(S::far);
         const int f0 = b >= 0 ? s_rng[b][0] : 0, f1 = b >= 0 ? s_rng[b][1] : nw, p1 = b >= 0 ? s_rng[b][2] : nw;
-        const int a = min(max(first_above<true>(s_w, nw, c - near), f0), f1);
-        const int z = max(min(first_above<false>(s_w, nw, c + near), f1), a);
-        const int p = p1 > 0 ? min(first_above<false>(s_w, nw, near - c), p1) : 0;
+        // (closed ends: a frequency at the midpoint of a flat piece, half = 0 or lost in c, is near:
+        // the table takes a zero knot, the own moments' 1/(c - w) does not)
+        const int a = min(max(first_above<false>(s_w, nw, c - near), f0), f1);
+        const int z = max(min(first_above<true>(s_w, nw, c + near), f1), a);
+        const int p = p1 > 0 ? min(first_above<true>(s_w, nw, near - c), p1) : 0;
         r.f0 = (short)f0;
         r.n0 = (short)a;
         r.n1 = (short)z;
