@@ -414,7 +414,7 @@ template <bool STRICT, typename T> __device__ __forceinline__ int first_above(co
 
 // a queued piece's frequency ranges (indices of the sorted frequencies): the - term from f0 to f1,
 // its near part n0 to n1; the + term up to p1, its near part up to np; the delta term m0 to m1 (the
-// frequencies inside the knots, one more on each side: the pair's own test decides)
+// frequencies inside the knots, ends included: the pair's own test decides)
 struct Range {
   short f0, n0, n1, f1, np, p1, m0, m1;
 };
@@ -576,9 +576,13 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
       const T e0 = s_qe[wib][sl][0], e3 = s_qe[wib][sl][3];
       Range r{};
       {
-        const int a = first_above<true>(s_w, nw, D0h + e0), z = first_above<false>(s_w, nw, D0h + e3);
-        r.m0 = (short)(a > 0 ? a - 1 : 0);
-        r.m1 = (short)(z < nw ? z + 1 : nw);
+        // frequencies inside the knots, up to the roundings of D0 and |w| to T (ties with either end
+        // included, however many); the pair's own test decides
+        const T dlo = D0h + e0, dhi = D0h + e3;
+        const T eps = FP64 ? T(0) : T(2.384185791015625e-07);  // 2^-22
+        const int a = first_above<false>(s_w, nw, dlo - eps * (tabs(D0h) + tabs(dlo)));
+        r.m0 = (short)a;
+        r.m1 = (short)max(first_above<true>(s_w, nw, dhi + eps * (tabs(D0h) + tabs(dhi))), a);
         nd = r.m1 - r.m0;
       }
       if constexpr (!IMO) {

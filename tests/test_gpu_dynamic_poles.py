@@ -101,3 +101,35 @@ def test_bands_split_rigidly_at_gamma(C, O, prec):
     off = np.arange(len(omega)) != at
     assert np.max(np.abs(gr - r)[off]) < TOL[prec] * np.max(np.abs(r[off]))
     assert np.max(np.abs(gi - i)[off]) < TOL[prec] * np.max(np.abs(i))
+
+
+def mixed_spectrum():
+    """Flat bands D = 1.5 and 3 beside a dispersive one that covers the same range."""
+    W = flat()
+    c = wl.corner_frac(W.n, True)
+    E = np.array(W.E)
+    E[:, 2] = 1.5 + np.round(1.25 * np.cos(2 * np.pi * c).mean(axis=1) * 2.0**16) / 2.0**16
+    return wl.Workload("beside", W.n, True, 3, 3, E, W.C, 0.0, (0, 3), False, W.qs)
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("extra", ["signs", "three", "eight", "close"])
+def test_repeats_at_a_flat_band_leave_the_others_alone(C, O, prec, extra):
+    """The same frequency several times (and with the other sign, and as neighbours that one FP32 number
+    stands for) where a flat D equals it: every other frequency keeps its values, bitwise in the mixed
+    form (integer sums), and all of Im agrees with the oracle."""
+    W = mixed_spectrum()
+    omega = np.arange(1, 33) / 8.0
+    more = {"signs": [-1.5], "three": [1.5, 1.5], "eight": [1.5] * 4 + [-1.5] * 3,
+            "close": 1.5 + 1e-9 * np.arange(1, 8)}[extra]
+    all_w = np.concatenate([omega, more])
+    r0, i0 = run(C, W, prec, omega)
+    r1, i1 = run(C, W, prec, all_w)
+    _, i = O.chi0_q(W, W.qs[0], omega=all_w)
+    assert np.max(np.abs(i1 - i)) < TOL[prec] * np.max(np.abs(i)), (i1, i)
+    n = len(omega)
+    if prec == "mixed":
+        assert np.array_equal(r1[:n], r0) and np.array_equal(i1[:n], i0)
+    else:
+        assert np.max(np.abs(r1[:n] - r0)) < TOL[prec] * np.max(np.abs(r0))
+        assert np.max(np.abs(i1[:n] - i0)) < TOL[prec] * np.max(np.abs(i0))
