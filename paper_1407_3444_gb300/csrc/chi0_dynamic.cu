@@ -160,6 +160,7 @@ template <typename T> struct BoxGeo {
   T lowG[kBoxG + 1];       // lower edges x_b of the geometric boxes (x = c - u_max)
   T W0, x0, umax;
   int on;
+  int nv;  // frequencies that are finite in T: the first nv of the sorted ones
 };
 template <typename T> struct BoxTab : BoxGeo<T> {
   T om[kNWPass];        // |w| ascending
@@ -175,19 +176,27 @@ template <typename T> __device__ __forceinline__ void kadd_t(T &sum, T &comp, T 
   sum = t;
 }
 
-// one block: the sorted frequencies, u_max of the pass and the box table (boxes = 0: none)
+// one block: the sorted frequencies, u_max of the pass and the box table (boxes = 0: none).
+// Frequencies that are not finite (NaN, infinite, past T's range) come last and take no part in the
+// searches, the boxes or u_max; k_dyn_out gives them their values.
 template <typename T>
 __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict__ omega, int nw, int boxes,
                                                        BoxTab<T> *tab) {
   __shared__ double red[8];
+  __shared__ int cnt[8];
   __shared__ unsigned long long key[kNWPass];
   const int i = threadIdx.x;
   const double a = i < nw ? fabs(omega[i]) : 0.0;
+  const bool ok = i < nw && (double)(T)a < (double)INFINITY;
   key[i] = (unsigned long long)__double_as_longlong(a);  // ascends with a; a NaN comes last
-  double u = a;
+  double u = ok ? a : 0.0;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) u = fmax(u, __shfl_xor_sync(kFull, u, o));
-  if ((i & 31) == 0) red[i >> 5] = u;
+  const unsigned oks = __ballot_sync(kFull, ok);
+  if ((i & 31) == 0) {
+    red[i >> 5] = u;
+    cnt[i >> 5] = __popc(oks);
+  }
   __syncthreads();
   if (i < nw) {
     int r = 0;
@@ -197,14 +206,19 @@ __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict_
     tab->oml[r] = (T)(a - (double)(T)a);
   }
   double umax = 0.0;
-  for (int k = 0; k < kNWPass / 32; ++k) umax = fmax(umax, red[k]);
+  int nv = 0;
+  for (int k = 0; k < kNWPass / 32; ++k) {
+    umax = fmax(umax, red[k]);
+    nv += cnt[k];
+  }
   const T W0 = (T)(umax / kBoxJ0), um = (T)umax, x0 = W0 * T(5);
-  const int on = (boxes && nw >= kMinBoxNw && umax > 1e-30 && umax < 1e30 && W0 > T(0)) ? 1 : 0;
+  const int on = (boxes && nv >= kMinBoxNw && umax > 1e-30 && umax < 1e30 && W0 > T(0)) ? 1 : 0;
   if (i == 0) {
     tab->W0 = W0;
     tab->x0 = x0;
     tab->umax = um;
     tab->on = on;
+    tab->nv = nv;
     double lo = (double)x0;
     for (int b = 0; b <= kBoxG; ++b) {
       tab->lowG[b] = (T)lo;
@@ -498,9 +512,9 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   if constexpr (!IMO) {
 #pragma unroll 1
     for (int b = threadIdx.x; b < kBoxFine; b += blockDim.x) {
-      int a = nw, z = 0, p = 0;  // (intervals: |w| ascends)
+      int a = kNWPass, z = 0, p = 0;  // (intervals: |w| ascends)
 #pragma unroll 1
-      for (int i = 0; i < nw; ++i) {
+      for (int i = 0; i < s_tab.nv; ++i) {
         if (!box_far(s_tab.C[b], s_tab.R[b], b, s_w[i], 0)) {
           a = a < i ? a : i;
           z = i + 1;
@@ -571,7 +585,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   auto drain = [&](int n) {
     int no = 0, nn = 0, nd = 0;
     if (lane < n) {
-      const int sl = (qh + lane) % kQC;
+      const int sl = (qh + lane) % kQC, nv = s_tab.nv;
       const T D0h = s_qv[wib][sl][1];
       const T e0 = s_qe[wib][sl][0], e3 = s_qe[wib][sl][3];
       Range r{};
@@ -580,20 +594,20 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
         // included, however many); the pair's own test decides
         const T dlo = D0h + e0, dhi = D0h + e3;
         const T eps = FP64 ? T(0) : T(2.384185791015625e-07);  // 2^-22
-        const int a = first_above<false>(s_w, nw, dlo - eps * (tabs(D0h) + tabs(dlo)));
+        const int a = first_above<false>(s_w, nv, dlo - eps * (tabs(D0h) + tabs(dlo)));
         r.m0 = (short)a;
-        r.m1 = (short)max(first_above<true>(s_w, nw, dhi + eps * (tabs(D0h) + tabs(dhi))), a);
+        r.m1 = (short)max(first_above<true>(s_w, nv, dhi + eps * (tabs(D0h) + tabs(dhi))), a);
         nd = r.m1 - r.m0;
       }
       if constexpr (!IMO) {
         const int b = s_qb[wib][sl];
         const T half = (e3 - e0) * T(0.5), c = D0h + (e0 + e3) * T(0.5), near = half * T(S::far);
-        const int f0 = b >= 0 ? s_rng[b][0] : 0, f1 = b >= 0 ? s_rng[b][1] : nw, p1 = b >= 0 ? s_rng[b][2] : nw;
+        const int f0 = b >= 0 ? s_rng[b][0] : 0, f1 = b >= 0 ? s_rng[b][1] : nv, p1 = b >= 0 ? s_rng[b][2] : nv;
         // (closed ends: a frequency at the midpoint of a flat piece, half = 0 or lost in c, is near:
         // the table takes a zero knot, the own moments' 1/(c - w) does not)
-        const int a = min(max(first_above<false>(s_w, nw, c - near), f0), f1);
-        const int z = max(min(first_above<true>(s_w, nw, c + near), f1), a);
-        const int p = p1 > 0 ? min(first_above<true>(s_w, nw, near - c), p1) : 0;
+        const int a = min(max(first_above<false>(s_w, nv, c - near), f0), f1);
+        const int z = max(min(first_above<true>(s_w, nv, c + near), f1), a);
+        const int p = p1 > 0 ? min(first_above<true>(s_w, nv, near - c), p1) : 0;
         r.f0 = (short)f0;
         r.n0 = (short)a;
         r.n1 = (short)z;
@@ -830,7 +844,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
       }
     }
     // (Im only: pieces whose knot range meets the pass's frequencies)
-    const bool queue = has && (IMO ? (D0h + ee[3] > s_w[0] && D0h + ee[0] < s_w[nw - 1]) : b < kBoxFine);
+    const bool queue = has && (IMO ? s_tab.nv > 0 && D0h + ee[3] > s_w[0] && D0h + ee[0] < s_w[s_tab.nv - 1] : b < kBoxFine);
     const unsigned qm = __ballot_sync(kFull, queue);
     if (queue) {
       const int sl = (qt + __popc(qm & lt)) % kQC;
@@ -1255,6 +1269,13 @@ __global__ void __launch_bounds__(128) k_dyn_out(const double *__restrict__ omeg
   const int iw = blockIdx.x;
   const double wv = omega[iw], u = fabs(wv);
   const int rk = tb.rank[iw];
+  if (rk >= tb.nv) {  // not finite: Re of a NaN is NaN, at infinity everything is 0
+    if (threadIdx.x == 0) {
+      if (re) re[iw] = wv != wv ? wv : 0.0;
+      im[iw] = 0.0;
+    }
+    return;
+  }
   const T om = tb.om[rk];
   double v = 0.0, vi = 0.0;
   unsigned long long ar = 0ull, ai = 0ull;

@@ -133,3 +133,34 @@ def test_repeats_at_a_flat_band_leave_the_others_alone(C, O, prec, extra):
     else:
         assert np.max(np.abs(r1[:n] - r0)) < TOL[prec] * np.max(np.abs(r0))
         assert np.max(np.abs(i1[:n] - i0)) < TOL[prec] * np.max(np.abs(i0))
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("odd", [[np.nan], [np.nan, np.inf, -np.inf, np.nan, 1e300], [np.nan] * 40, [np.inf] * 3],
+                         ids=["nan", "mixture", "many_nan", "inf"])
+def test_frequencies_that_are_not_finite_stay_by_themselves(C, prec, odd):
+    """The finite frequencies keep their values (bitwise in the mixed form); a NaN has Re = NaN and
+    Im = 0, an infinite one (in the mixed form one past FP32's range) the limit 0."""
+    W = mixed_spectrum()
+    omega = np.arange(1, 33) / 8.0 + 0.03
+    rng = np.random.default_rng(7)
+    all_w = np.concatenate([omega, odd])
+    order = rng.permutation(len(all_w))
+    r0, i0 = run(C, W, prec, omega)
+    r1, i1 = np.empty(len(all_w)), np.empty(len(all_w))
+    r1[order], i1[order] = run(C, W, prec, all_w[order])
+    n = len(omega)
+    if prec == "mixed":
+        assert np.array_equal(r1[:n], r0) and np.array_equal(i1[:n], i0)
+    else:
+        assert np.max(np.abs(r1[:n] - r0)) < TOL[prec] * np.max(np.abs(r0))
+        assert np.max(np.abs(i1[:n] - i0)) < TOL[prec] * np.max(np.abs(i0))
+    nan = np.isnan(all_w[n:])
+    assert np.all(np.isnan(r1[n:][nan]))
+    assert np.all(np.abs(r1[n:][~nan]) <= 1e-290) and np.all(i1[n:] == 0.0)
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_no_finite_frequency_at_all(C, prec):
+    r, i = run(C, flat(), prec, np.array([np.nan, np.inf]))
+    assert np.isnan(r[0]) and r[1] == 0.0 and np.all(i == 0.0)
