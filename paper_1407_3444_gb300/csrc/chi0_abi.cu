@@ -518,8 +518,9 @@ static int enqueue_overlap(chi0_plan_t *p, const Q *q, int n, Timer &tm, bool tc
       a.q[i] = q[i];
       a.W2[i] = (char *)p->W2_d + i * slot;
     }
-    CK(p, launch_overlap(a, p->C_d, p->dtype, fp64, p->stream, p->C32_d));
-    p->stats.kernels += 1;
+    int launches = 0;
+    CK(p, launch_overlap(a, p->C_d, p->dtype, fp64, p->stream, p->C32_d, &launches));
+    p->stats.kernels += launches;
   }
   tm.stop();
   return CHI0_OK;

@@ -68,7 +68,8 @@ struct OverlapArgs {
   Q q[kMaxGroup];
   void *W2[kMaxGroup];
 };
-cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int fp64, cudaStream_t s, const void *C32);
+cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int fp64, cudaStream_t s, const void *C32,
+                           int *launches = nullptr);
 // complex128 -> complex64 copy (the k-side eigenvectors of a mixed-precision plan)
 cudaError_t launch_c128_to_c64(const void *in, void *out, long long n, cudaStream_t s);
 

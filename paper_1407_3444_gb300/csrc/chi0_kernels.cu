@@ -311,37 +311,56 @@ cudaError_t launch_c128_to_c64(const void *in, void *out, long long n, cudaStrea
   return cudaGetLastError();
 }
 
-cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int fp64, cudaStream_t s, const void *C32) {
-  int w = 0;
-  for (int i = 0; i < a.nq; ++i) w = a.q[i].hi - a.q[i].lo > w ? a.q[i].hi - a.q[i].lo : w;
+// the q points of a group with norb w <= kOvlSmall, or the others (windows differ): so that a q's values
+// do not depend on what it is grouped with
+static void pick_overlap(const OverlapArgs &a, bool small, OverlapArgs &out) {
+  out.g = a.g;
+  out.nq = 0;
+  for (int i = 0; i < a.nq; ++i) {
+    if (((long long)a.g.norb * (a.q[i].hi - a.q[i].lo) <= kOvlSmall) != small) continue;
+    out.q[out.nq] = a.q[i];
+    out.W2[out.nq++] = a.W2[i];
+  }
+}
+
+cudaError_t launch_overlap(const OverlapArgs &a, const void *C, int dtype, int fp64, cudaStream_t s, const void *C32,
+                           int *launches) {
   const Grid &g = a.g;
-  const long long total = g.nc * (long long)w * w;
-  long long nb = (total + kThreads - 1) / kThreads;
-  const int blocks = (int)(nb < device_sms() * 16 ? nb : device_sms() * 16);
-  if (blocks <= 0) return cudaSuccess;
+  if (launches) *launches = 0;
+  if (a.nq < 1 || g.nc < 1) return cudaSuccess;
   const bool ex = a.q[0].Cq != nullptr;  // (a group's q points are all explicit or all shifts)
-  if ((long long)g.norb * w <= kOvlSmall) {
+  OverlapArgs p;
+  pick_overlap(a, true, p);
+  if (p.nq > 0) {
     const long long warps = fp64 ? 4 : 8, nbw = (g.nc + warps - 1) / warps, cap = device_sms() * 4;  // resident blocks
-    const dim3 bw((unsigned)(nbw < cap ? nbw : cap), (unsigned)a.nq);
+    const dim3 bw((unsigned)(nbw < cap ? nbw : cap), (unsigned)p.nq);
     if (fp64) {
-      if (dtype == DT_C128) k_overlap_small<double2, double2, double><<<bw, 128, 0, s>>>(a, (const double2 *)C, ex ? 1 : 0);
-      else k_overlap_small<float2, float2, double><<<bw, 128, 0, s>>>(a, (const float2 *)C, ex ? 1 : 0);
-      return cudaGetLastError();
+      if (dtype == DT_C128) k_overlap_small<double2, double2, double><<<bw, 128, 0, s>>>(p, (const double2 *)C, ex ? 1 : 0);
+      else k_overlap_small<float2, float2, double><<<bw, 128, 0, s>>>(p, (const float2 *)C, ex ? 1 : 0);
+    } else {
+      // k side in complex64 (the plan's copy when the inputs are complex128)
+      const float2 *Ck = (const float2 *)(C32 ? C32 : C);
+      if (ex && dtype == DT_C128) k_overlap_small<float2, double2, float><<<bw, 256, 0, s>>>(p, Ck, 1);
+      else k_overlap_small<float2, float2, float><<<bw, 256, 0, s>>>(p, Ck, ex ? 1 : 0);
     }
-    // k side in complex64 (the plan's copy when the inputs are complex128)
-    const float2 *Ck = (const float2 *)(C32 ? C32 : C);
-    if (ex && dtype == DT_C128) k_overlap_small<float2, double2, float><<<bw, 256, 0, s>>>(a, Ck, 1);
-    else k_overlap_small<float2, float2, float><<<bw, 256, 0, s>>>(a, Ck, ex ? 1 : 0);
-    return cudaGetLastError();
-  }
-  const dim3 bg((unsigned)blocks, (unsigned)a.nq);
-  if (dtype == DT_C128) {
-    if (fp64) k_overlap<double2, double><<<bg, kThreads, 0, s>>>(a, (const double2 *)C);
-    else k_overlap<double2, float><<<bg, kThreads, 0, s>>>(a, (const double2 *)C);
+    if (launches) ++*launches;
+    if (p.nq == a.nq) return cudaGetLastError();
+    pick_overlap(a, false, p);
   } else {
-    if (fp64) k_overlap<float2, double><<<bg, kThreads, 0, s>>>(a, (const float2 *)C);
-    else k_overlap<float2, float><<<bg, kThreads, 0, s>>>(a, (const float2 *)C);
+    p = a;
   }
+  int w = 0;
+  for (int i = 0; i < p.nq; ++i) w = p.q[i].hi - p.q[i].lo > w ? p.q[i].hi - p.q[i].lo : w;
+  const long long nb = (g.nc * (long long)w * w + kThreads - 1) / kThreads, cap = device_sms() * 16;
+  const dim3 bg((unsigned)(nb < cap ? nb : cap), (unsigned)p.nq);
+  if (dtype == DT_C128) {
+    if (fp64) k_overlap<double2, double><<<bg, kThreads, 0, s>>>(p, (const double2 *)C);
+    else k_overlap<double2, float><<<bg, kThreads, 0, s>>>(p, (const double2 *)C);
+  } else {
+    if (fp64) k_overlap<float2, double><<<bg, kThreads, 0, s>>>(p, (const float2 *)C);
+    else k_overlap<float2, float><<<bg, kThreads, 0, s>>>(p, (const float2 *)C);
+  }
+  if (launches) ++*launches;
   return cudaGetLastError();
 }
 
