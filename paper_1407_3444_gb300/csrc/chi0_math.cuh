@@ -496,7 +496,7 @@ __device__ __forceinline__ float series_sum_short(const float x[4], const float 
   if (tabs(t) + tabs(tp) > thr) {
     xb = fmaf(r2, xb, n3);
 #pragma unroll 1
-    for (int k = 3; k < Num<float>::kmax; k += 2) {
+    for (int k = 3; k + 1 < Num<float>::kmax; k += 2) {  // (two coefficients a step)
       yb = fmaf(r2, yb, xb);
       tp = series_coef<float>(k) * step(yb);
       sum += tp;
