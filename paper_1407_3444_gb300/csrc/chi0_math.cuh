@@ -1295,10 +1295,19 @@ template <typename T> __device__ __forceinline__ T sel4(const T v[4], unsigned i
 }
 __device__ __forceinline__ float cut_quot(float a, float b) { return quot(a, b); }
 __device__ __forceinline__ double cut_quot(double a, double b) { return a * rcp_nr(b); }
-// cut fraction of slot k (0 for an unused slot) and the values at its vertex
-template <typename T> __device__ __forceinline__ T cut_frac(unsigned rec, int k, const T key[4]) {
+// cut fraction of slot k (0 for an unused slot) and the values at its vertex.  FP64 key differences below
+// 2^-1022 have no finite reciprocal.  They are scaled here, exactly; or the caller's keys come scaled
+// (SCALED), which costs the FP64 static weights nothing where this test took 1.4% of them.
+template <typename T> constexpr T kKeyScale = sizeof(T) == 8 ? T(18446744073709551616.0) : T(1);  // 2^64
+template <bool SCALED = false, typename T> __device__ __forceinline__ T cut_frac(unsigned rec, int k, const T key[4]) {
   const unsigned sl = rec >> (5 * k);
-  const T ki = sel4(key, sl & 3u), den = ki - sel4(key, (sl >> 2) & 3u);
+  T ki = sel4(key, sl & 3u), den = ki - sel4(key, (sl >> 2) & 3u);
+  if constexpr (sizeof(T) == 8 && !SCALED) {
+    if (Mean<T>::bits(den) < 0x00100000) {
+      ki *= kKeyScale<T>;
+      den *= kKeyScale<T>;
+    }
+  }
   return den != T(0) ? cut_quot(ki, den) : T(0);
 }
 template <typename T> __device__ __forceinline__ T cut_mix(unsigned rec, int k, const T v[4], T t) {

@@ -368,14 +368,19 @@ __global__ void __launch_bounds__(NT, MINB) k_static(const __grid_constant__ Sta
         b[i] = en[(long long)cq[i] * nb];
       }
     };
-    // a relative to eF and D = b - a
+    // D = b - a, and the first cut's keys a - eF; FP64 keys carry the factor S = 2^64 (exact, and free
+    // in the multiply-add; |E| < 2^959), so that levels as close to eF as the smallest numbers have
+    // quotients
+    constexpr T S = kKeyScale<T>;
     auto relative = [&](T a[4], const T b[4], T D[4]) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         D[i] = b[i] - a[i];
-        if constexpr (FP64) a[i] -= g.ef;
+        if constexpr (FP64) a[i] = fma(a[i], S, -S * g.ef);
       }
     };
+    // the second cut's key, -b, at a vertex of key a (0 on the first cut's plane)
+    auto key_b = [&](T a, T D) { return FP64 ? -fma(D, S, a) : -(a + D); };
     // FP32: the vertices in ascending order of the key, as cut_piece takes them
     auto sort_key = [&](T key[4], T x[4], T y[4]) {
       if constexpr (!FP64) {
@@ -471,7 +476,7 @@ __global__ void __launch_bounds__(NT, MINB) k_static(const __grid_constant__ Sta
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         m1 |= (is_neg(a[i]) ? 1u : 0u) << i;
-        eb |= (is_neg(-(a[i] + D[i])) ? 1u : 0u) << i;
+        eb |= (is_neg(key_b(a[i], D[i])) ? 1u : 0u) << i;
         dpos = dpos && is_neg(-D[i]);
       }
       const int n1 = has ? cut_count(m1) : 0;
@@ -487,7 +492,7 @@ __global__ void __launch_bounds__(NT, MINB) k_static(const __grid_constant__ Sta
           } else {
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-              const T x = cut_mix(rec, k, D, cut_frac(rec, k, a));
+              const T x = cut_mix(rec, k, D, cut_frac<true>(rec, k, a));
               m2 |= (cut_used(rec, k) ? (is_neg(-x) ? 1u : 0u) : (eb >> ((rec >> (5 * k)) & 3u)) & 1u) << k;
             }
           }
@@ -536,21 +541,22 @@ __global__ void __launch_bounds__(NT, MINB) k_static(const __grid_constant__ Sta
             unsigned rec = s_rec[m * 4 + (sub >> 6)];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-              const T t = cut_frac(rec, k, u);
+              const T t = cut_frac<true>(rec, k, u);
               D1[k] = cut_mix(rec, k, x, t);
               f1[k] = cut_mix(rec, k, y, t);
-              key[k] = -(cut_used(rec, k) ? D1[k] : sel4(u, (rec >> (5 * k)) & 3u) + D1[k]);
+              if constexpr (FP64) key[k] = key_b(cut_used(rec, k) ? T(0) : sel4(u, (rec >> (5 * k)) & 3u), D1[k]);
+              else key[k] = -(cut_used(rec, k) ? D1[k] : sel4(u, (rec >> (5 * k)) & 3u) + D1[k]);
               r *= cut_factor(rec, k, t);
             }
             D1[3] = sel4(x, (rec >> 15) & 3u);
             f1[3] = sel4(y, (rec >> 15) & 3u);
-            key[3] = -(sel4(u, (rec >> 15) & 3u) + D1[3]);
+            key[3] = key_b(sel4(u, (rec >> 15) & 3u), D1[3]);
             // second cut, by the side mask the piece was listed with
             sort_key(key, D1, f1);
             rec = s_rec[(sub & 15u) * 4 + ((sub >> 4) & 3u)];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-              const T t = cut_frac(rec, k, key);
+              const T t = cut_frac<true>(rec, k, key);
               d[k] = cut_mix(rec, k, D1, t);
               f[k] = cut_mix(rec, k, f1, t);
               r *= cut_factor(rec, k, t);
