@@ -317,7 +317,7 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
   // unit partials of the static weights; per-warp sums of the FP64 dynamic weights
   const size_t np = op.precision == CHI0_PREC_FP64 ? (size_t)dynamic_max_ctas_per_sm(1) * device_sms() *
                                                          dynamic_warps_per_cta(1) * dynamic_max_nw() : 1;
-  const size_t ns = G * (size_t)static_max_units(g.ntet);
+  const size_t ns = G * (size_t)static_units(g.ntet, w);
   CK(p, cudaMalloc(&p->partR, sizeof(double) * (np > ns ? np : ns)));
   CK(p, cudaMalloc(&p->partI, sizeof(double) * np));
   CK(p, cudaMalloc(&p->dos_d, sizeof(double) * G * static_blocks()));

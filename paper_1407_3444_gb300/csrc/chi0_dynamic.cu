@@ -84,7 +84,6 @@ constexpr int kNWPass = 256;   // frequencies per dynamic pass
 // per-CTA total stays far below 2^19, and one rounding of 2^-45 per term is far below the
 // FP32 terms' own error)
 constexpr double kFxUnit = 1.0 / 17592186044416.0;
-constexpr int kFbCap = 4096;   // near-field entries left to the per-vertex table, per warp
 constexpr int kQC = 64;        // queue of final tetrahedra that evaluate frequencies themselves
 constexpr int kCodes = 128;    // listed pieces of cut items per warp: < 32 left over + 3 x 32
 
@@ -105,6 +104,9 @@ template <bool FP64> struct DynShape {
   static constexpr int KO = FP64 ? 40 : 32;  // own moments of a queued piece, at most
   static constexpr int KG = FP64 ? 18 : 12;  // moments of a geometric box (z <= 2/9)
   static constexpr int KW = FP64 ? 32 : 20;  // moments of a wide box (z <= 5/9)
+  // near-field entries left to the per-vertex table that a warp collects: FP64 flushes them in full
+  // rounds when they fill (100 MB for all warps), FP32 leaves the last ones to k_dyn_fallback
+  static constexpr int fb = FP64 ? 1024 : 4096;
 };
 template <bool FP64> constexpr bool poly_ok(double tol) {
   using S = DynShape<FP64>;
@@ -481,7 +483,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
   const long long units = (g.ntet + (1LL << tlog) - 1) >> tlog;
   const long long gwarp = (long long)blockIdx.x * W + wib, nwarps = (long long)gridDim.x * W;
   double *gbox = db.box_part + gwarp * NS;  // FP64: the warp's box moments
-  FbEnt<T> *gfb = (FbEnt<T> *)db.fb + gwarp * kFbCap;
+  FbEnt<T> *gfb = (FbEnt<T> *)db.fb + gwarp * S::fb;
   {
     const BoxTab<T> *src = (const BoxTab<T> *)db.box_tab;
     constexpr int nwords = (int)(sizeof(BoxGeo<T>) / 4);
@@ -722,7 +724,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
       int p = 0;
 #pragma unroll 1
       for (int base = 0; base < near; base += 32) {  // warp-uniform
-        if (nfb > kFbCap - 32) fallback_flush();
+        if (nfb > S::fb - 32) fallback_flush();
         const int it = base + lane;
         T re = T(0), x[4], ff[4], vr = T(0);
         int iw = -1, code = 0;
@@ -1194,7 +1196,7 @@ __global__ void __launch_bounds__(128) k_dyn_fallback(DynBufs db, int nbuf, int 
   int nfp64 = 0;
   for (int buf = blockIdx.x; buf < nbuf; buf += gridDim.x) {
     const int n = db.fbn[buf];
-    const FbEnt<float> *ent = (const FbEnt<float> *)db.fb + (size_t)buf * kFbCap;
+    const FbEnt<float> *ent = (const FbEnt<float> *)db.fb + (size_t)buf * DynShape<false>::fb;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
       const FbEnt<float> &o = ent[k];
       float x[4], f[4];
@@ -1376,7 +1378,7 @@ int dynamic_warps_per_cta(int fp64) { return fp64 ? DynShape<true>::warps : DynS
 size_t dynamic_box_slots(int fp64) { return fp64 ? box_slots<true>() : box_slots<false>(); }
 size_t dynamic_fx_bytes(int nblocks) { return (size_t)nblocks * 2 * kNWPass * sizeof(unsigned long long); }
 size_t dynamic_fb_bytes(int fp64) {
-  return (size_t)kFbCap * (fp64 ? sizeof(FbEnt<double>) : sizeof(FbEnt<float>));
+  return fp64 ? DynShape<true>::fb * sizeof(FbEnt<double>) : DynShape<false>::fb * sizeof(FbEnt<float>);
 }
 size_t dynamic_box_tab_bytes() {
   return sizeof(BoxTab<double>) > sizeof(BoxTab<float>) ? sizeof(BoxTab<double>) : sizeof(BoxTab<float>);

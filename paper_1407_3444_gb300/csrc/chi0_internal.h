@@ -118,8 +118,8 @@ cudaError_t launch_static(StaticArgs &a, int fp64, int nblocks, cudaStream_t s, 
 cudaError_t launch_static_reduce(const StaticArgs &a, double scale, int ndos, double *out, cudaStream_t s);
 int static_persistent_blocks(int fp64);
 long long static_batches(long long ntet);  // runs of 32 tetrahedra (the dynamic weights' batches)
-long long static_units(long long ntet, int w);   // partials of one q with a window of w bands
-long long static_max_units(long long ntet);      // ... of any window
+// partials of one q with a window of w bands (never more with a narrower one)
+long long static_units(long long ntet, int w);
 
 // message of the last failed call made without a plan (chi0_last_error(NULL))
 void set_global_error(const char *msg);

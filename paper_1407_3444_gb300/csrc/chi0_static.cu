@@ -661,8 +661,6 @@ long long static_units(long long ntet, int w) {
   return (ntet + (1LL << t) - 1) >> t;
 }
 
-long long static_max_units(long long ntet) { return (ntet + 3) >> 2; }
-
 int static_max_ctas_per_sm(int fp64, int variant) {
   int nb = 0;
   cudaError_t e;
