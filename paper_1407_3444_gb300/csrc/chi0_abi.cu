@@ -554,6 +554,12 @@ static int enqueue_dos(chi0_plan_t *p, const Q &q, int slot, unsigned long long 
   return CHI0_OK;
 }
 
+// q points whose band-pair totals (w x w 64-bit sums each) a static call keeps at a time: 64 MB
+static int pairs_group(const chi0_plan_t *p) {
+  const size_t w = (size_t)(p->win.hi - p->win.lo), fit = ((size_t)64 << 20) / (sizeof(unsigned long long) * w * w);
+  return fit < 1 ? 1 : (fit < (size_t)p->group ? (int)fit : p->group);
+}
+
 // Launches of a static call, a group of q points at a time: overlaps, DOS at Gamma, band bounds
 // of explicit k+q energies, weights, reduction.  A group is a run of q points that are all
 // shifts or all explicit; explicit data from the host go one q at a time (two staging buffers,
@@ -569,7 +575,7 @@ static int enqueue_static(chi0_plan_t *p, const chi0_q_t *qs, int nq, double *ou
   size_t poff = 0;  // band-pair output: offset of this q's w x w block
   for (int i0 = 0; i0 < nq;) {
     const bool ex = qs[i0].e_kq != nullptr;
-    const int most = ex && !op.inputs_on_device ? 1 : p->group;
+    const int most = ex && !op.inputs_on_device ? 1 : (outP ? pairs_group(p) : p->group);
     Q q[kMaxGroup];
     int n = 0, slot = -1;
     for (; n < most && i0 + n < nq && (qs[i0 + n].e_kq != nullptr) == ex; ++n) {
@@ -801,7 +807,7 @@ static int run(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double *omega, 
   size_t npairs = 0;
   if (pairs) {
     const int wp = p->win.hi - p->win.lo;
-    int rc = ensure(p, (void **)&p->pairs_fx_d, &p->pairs_fx_cap, sizeof(unsigned long long) * p->group * wp * wp);
+    int rc = ensure(p, (void **)&p->pairs_fx_d, &p->pairs_fx_cap, sizeof(unsigned long long) * pairs_group(p) * wp * wp);
     if (rc) return rc;
     for (int iq = 0; iq < nq; ++iq) {
       const int lo = qs[iq].win.lo < 0 ? p->win.lo : qs[iq].win.lo, hi = qs[iq].win.lo < 0 ? p->win.hi : qs[iq].win.hi;

@@ -38,3 +38,33 @@ def test_small_fp64_plan(C):
     held = f0 - free_bytes()
     P.close()
     assert held < 180 * MB, held / MB
+
+
+def test_band_pair_totals_of_a_wide_window(C):
+    """1024 bands without matrix elements, 8 q: the fixed-point totals of the q in flight stay within
+    64 MB (8 MB a q), and each q's block is bitwise that of the q alone."""
+    nb = 1024
+    E = np.linspace(-1.0, 1.0, nb)[None, :] * np.array([1.0, 1.1])[:, None]
+    W = wl.Workload("wide", (1, 1, 2), True, nb, nb, E, None, 0.0, (0, nb), True,
+                    [wl.QPoint(shift=(0, 0, 1)) for _ in range(8)])
+    q = [wl.QPoint(shift=(0, 0, 1), window=(0, nb) if j % 2 else (8 * j, nb)) for j in range(12)]
+    W.qs = q
+    S = C.DeviceInputs(W)
+    P = C.Plan(W, precision="fp64", staged=S)
+    f0 = free_bytes()
+    import torch
+    npairs = sum((nb - (0 if j % 2 else 8 * j)) ** 2 for j in range(12))
+    chi = torch.empty(12, dtype=torch.float64, device="cuda")
+    pairs = torch.empty(npairs, dtype=torch.float64, device="cuda")
+    f0 = free_bytes()
+    C.chi0_static_pairs(P.h, P.qarr, 12, chi.data_ptr(), pairs.data_ptr())
+    held = f0 - free_bytes()
+    assert held <= 96 * MB, held / MB
+    off = 0
+    for j in range(12):
+        w = nb - (0 if j % 2 else 8 * j)
+        one, p1 = torch.empty(1, dtype=torch.float64, device="cuda"), torch.empty(w * w, dtype=torch.float64, device="cuda")
+        C.chi0_static_pairs(P.h, (C.chi0_q_t * 1)(P.qarr[j]), 1, one.data_ptr(), p1.data_ptr())
+        assert torch.equal(p1, pairs[off:off + w * w]) and torch.equal(one, chi[j:j + 1])
+        off += w * w
+    P.close()
