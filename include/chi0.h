@@ -257,8 +257,8 @@ int chi0_static(chi0_plan_t *plan, const chi0_q_t *q, int nq, double *chi);
  * at k, empty band n at k+q (Eq. 1), the normalisation and sign of chi; at a q flagged
  * Gamma the intraband pairs (m, m) carry the q -> 0 limit N(eF) of band m (Sec. III).  The
  * pairs of a q add up to chi[iq].  Each pair is summed in 64-bit fixed point (units of
- * 2^-50 before the normalisation: exact in any order, reproducible, one rounding of 2^-51
- * per term).  pairs is a host or device pointer like chi (opts.outputs_on_device) with room
+ * 2^-50 before the normalisation, in the caller's unit of energy: exact in any order,
+ * reproducible, one rounding of 2^-51 per term, totals up to 2^13).  pairs is a host or device pointer like chi (opts.outputs_on_device) with room
  * for sum_q w_q^2 doubles; the call does not use graph capture.  Errors as chi0_static, plus
  * CHI0_EINVAL for pairs NULL or a plan window wider than 1024 bands.  The paper's figure is
  * a plot of these numbers; this entry point has no other counterpart in it. */
@@ -266,7 +266,10 @@ int chi0_static_pairs(chi0_plan_t *plan, const chi0_q_t *q, int nq, double *chi,
 
 /* Dynamic chi0(q, w) (Eqs. 1-3) on nw frequencies: re[iq*nw + iw], im[iq*nw + iw].
  * Re is the principal value of Eq. 1; Im is Eq. 2 for w > 0, 0 at w = 0, and odd
- * (Eq. 3) for w < 0.  Errors as chi0_static, plus CHI0_EINVAL for nw <= 0. */
+ * (Eq. 3) for w < 0.  Frequencies in any order; one that is not finite leaves the others alone
+ * (a NaN gives Re = NaN, Im = 0; an infinite one 0).  Energies in any unit: the mixed form's
+ * fixed-point sums are scaled by W, the largest |E - eF| of the plan's window, and hold
+ * W |chi0| up to 2^15.  Errors as chi0_static, plus CHI0_EINVAL for nw <= 0. */
 int chi0_dynamic(chi0_plan_t *plan, const chi0_q_t *q, int nq, const double *omega, int nw,
                  double *re, double *im);
 

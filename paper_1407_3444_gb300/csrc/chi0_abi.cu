@@ -66,7 +66,8 @@ struct chi0_plan {
   int *fbn_d = nullptr;                       // dynamic weights: per-warp fallback entries,
   void *fb_d = nullptr;                       // their counts,
   unsigned long long *fx_d = nullptr;         // per-CTA fixed-point sums (FP32) and the
-  unsigned long long *ctr_d = nullptr;        // batch counter
+  unsigned long long *ctr_d = nullptr;        // unit counter
+  unsigned long long *erange_d = nullptr;     // largest |E - eF| of the window (mixed precision)
   unsigned long long *pairs_fx_d = nullptr;   // band-pair output: fixed-point totals of one q,
   size_t pairs_fx_cap = 0;                    // and the FP64 results of the call (host outputs)
   double *pairs_out_d = nullptr;
@@ -181,6 +182,7 @@ static void release(chi0_plan_t *p) {
   cudaFree(p->fbn_d);
   cudaFree(p->fx_d);
   cudaFree(p->ctr_d);
+  cudaFree(p->erange_d);
   cudaFree(p->pairs_fx_d);
   cudaFree(p->pairs_out_d);
   cudaFree(p->ikq_E_d);
@@ -198,7 +200,7 @@ extern "C" void chi0_destroy(chi0_plan_t *p) {
 // band bounds per corner: four arrays of nc from base on
 static BandBounds bounds_at(short *base, long long nc) { return BandBounds{base, base + nc, base + 2 * nc, base + 3 * nc}; }
 
-// bounds and FP32 energies of the plan's own eigen-data
+// bounds, FP32 energies and energy range of the plan's own eigen-data
 static cudaError_t plan_bands(chi0_plan_t *p) {
   const Grid &g = p->g;
   BandArgs a{};
@@ -206,7 +208,9 @@ static cudaError_t plan_bands(chi0_plan_t *p) {
   a.out = bounds_at(p->bounds_d, g.nc);
   a.E32 = p->E32_d;
   a.E32lo = p->E32_d ? p->E32_d + (size_t)g.nc * g.nb : nullptr;
-  return launch_bands(a, 1, g.nc, g.nb, g.ef, p->stream);
+  const cudaError_t e = launch_bands(a, 1, g.nc, g.nb, g.ef, p->stream);
+  if (e != cudaSuccess || !p->erange_d) return e;
+  return launch_energy_range(p->E_d, g.nc, g.nb, p->win.lo, p->win.hi, g.ef, p->erange_d, p->stream);
 }
 
 static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t *tt, chi0_band_window_t win,
@@ -328,6 +332,7 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
   if (op.precision == CHI0_PREC_MIXED) {
     CK(p, cudaMalloc(&p->E32_d, 2 * sizeof(float) * ncb));
     CK(p, cudaMalloc(&p->Eq32_d, G * 2 * sizeof(float) * ncb));
+    CK(p, cudaMalloc(&p->erange_d, sizeof(unsigned long long)));
   }
   CK(p, plan_bands(p));
   if (op.precision == CHI0_PREC_MIXED && !op.cma && p->dtype == CHI0_C128) {
@@ -675,7 +680,8 @@ static int enqueue_call(chi0_plan_t *p, const chi0_q_t *qs, int nq, const double
     a.empf = qb.empf;
     a.cma = op.cma;
     a.tau = (float)op.tau;
-    a.db = DynBufs{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->fb_d, p->fbn_d, p->fx_d, p->ctr_d};
+    a.db = DynBufs{p->partR, p->partI, p->box_tab_d, p->box_part_d, p->box_tot_d, p->fb_d, p->fbn_d, p->fx_d, p->ctr_d,
+                   p->erange_d};
     a.counters = op.profile ? p->counters_d : nullptr;
     const bool kk = kk_du > 0.0;
     const double *dos = q.gamma ? p->dos_d : nullptr;
@@ -731,7 +737,7 @@ static void drop_graph(chi0_plan_t *p) {
 static int derive_inputs(chi0_plan_t *p) {
   const Grid &g = p->g;
   CK(p, plan_bands(p));
-  p->stats.kernels += 1;
+  p->stats.kernels += p->erange_d ? 2 : 1;
   if (p->C32_d) {
     CK(p, launch_c128_to_c64(p->C_d, p->C32_d, g.nc * (long long)g.norb * g.nb, p->stream));
     p->stats.kernels += 1;

@@ -80,10 +80,19 @@ using grid::quick_div;
 using grid::tet_corners;
 
 constexpr int kNWPass = 256;   // frequencies per dynamic pass
-// FP32 kernel: sums in 64-bit fixed point, units of 2^-44 (exact and order-independent; every
-// per-CTA total stays far below 2^19, and one rounding of 2^-45 per term is far below the
-// FP32 terms' own error)
+// FP32 kernel: sums in 64-bit fixed point, units of 2^-44 (exact and order-independent; one rounding of
+// 2^-45 per term).  Re and Im are sums of v f / energy, so the range (2^19) and the rounding are held
+// against the energies: W being the largest |E - eF| of the plan's window, the terms carry a power of
+// two S that is 1 for 2^-4 <= W < 2^8 and keeps S / W in [2^3, 2^4] below, in [2^-8, 2^-7] above.  So
+// W |sum| may reach 2^15 at least (80 bands: some 10 with |M|^2, a few 1000 without), and a sum of 10^9
+// terms rounds by 5e-10 / S, at most 1.3e-7 / W.
 constexpr double kFxUnit = 1.0 / 17592186044416.0;
+__device__ __forceinline__ float fx_scale(unsigned long long bits) {
+  const double W = __longlong_as_double((long long)bits);
+  if (!(W > 0.0)) return 1.0f;
+  const int e = ilogb(W);  // 2^e <= W < 2^(e + 1)
+  return (float)exp2((double)max(min(e < -4 ? e + 4 : (e > 7 ? e - 7 : 0), 100), -100));
+}
 constexpr int kQC = 64;        // queue of final tetrahedra that evaluate frequencies themselves
 constexpr int kCodes = 128;    // listed pieces of cut items per warp: < 32 left over + 3 x 32
 
@@ -161,6 +170,7 @@ template <typename T> struct BoxGeo {
   T C[kBoxes], R[kBoxes];  // centre and radius
   T lowG[kBoxG + 1];       // lower edges x_b of the geometric boxes (x = c - u_max)
   T W0, x0, umax;
+  T S;     // FP32 kernel: factor of the fixed-point sums (1 in FP64)
   int on;
   int nv;  // frequencies that are finite in T: the first nv of the sorted ones
 };
@@ -183,7 +193,7 @@ template <typename T> __device__ __forceinline__ void kadd_t(T &sum, T &comp, T 
 // searches, the boxes or u_max; k_dyn_out gives them their values.
 template <typename T>
 __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict__ omega, int nw, int boxes,
-                                                       BoxTab<T> *tab) {
+                                                       const unsigned long long *__restrict__ erange, BoxTab<T> *tab) {
   __shared__ double red[8];
   __shared__ int cnt[8];
   __shared__ unsigned long long key[kNWPass];
@@ -221,6 +231,7 @@ __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict_
     tab->umax = um;
     tab->on = on;
     tab->nv = nv;
+    tab->S = sizeof(T) == 4 ? (T)fx_scale(*erange) : T(1);
     double lo = (double)x0;
     for (int b = 0; b <= kBoxG; ++b) {
       tab->lowG[b] = (T)lo;
@@ -855,7 +866,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
         s_qe[wib][sl][i] = ee[i];
         s_qf[wib][sl][i] = ff[i];
       }
-      s_qv[wib][sl][0] = vr;
+      s_qv[wib][sl][0] = FX ? vr * s_tab.S : vr;
       s_qv[wib][sl][1] = D0h;
       s_qv[wib][sl][2] = D0l;
       s_qb[wib][sl] = (short)b;
@@ -1331,8 +1342,9 @@ __global__ void __launch_bounds__(128) k_dyn_out(const double *__restrict__ omeg
     v = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
     vi = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
     if constexpr (!FP64) {
-      v += (double)(long long)(rad[0][0] + rad[0][1] + rad[0][2] + rad[0][3]) * kFxUnit;
-      vi = (double)(long long)(rad[1][0] + rad[1][1] + rad[1][2] + rad[1][3]) * kFxUnit;
+      const double unit = kFxUnit / (double)tb.S;
+      v += (double)(long long)(rad[0][0] + rad[0][1] + rad[0][2] + rad[0][3]) * unit;
+      vi = (double)(long long)(rad[1][0] + rad[1][1] + rad[1][2] + rad[1][3]) * unit;
     }
     if (re) re[iw] = scale * v;
     im[iw] = wv < 0.0 ? -scale * vi : scale * vi;
@@ -1362,7 +1374,7 @@ cudaError_t launch_weights(const DynArgs &a, const double *omega, int nw, int nb
   if (!FP64) e = cudaMemsetAsync(db.ctr, 0, sizeof(unsigned long long), s);
   else if (!IMO) e = cudaMemsetAsync(db.box_part, 0, sizeof(double) * (size_t)rows * NS, s);
   if (e != cudaSuccess) return e;
-  k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, (BoxTab<T> *)db.box_tab);
+  k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, db.erange, (BoxTab<T> *)db.box_tab);
   k_dynamic<FP64, IMO><<<nblocks, DynShape<FP64>::threads, IMO ? 0 : dyn_smem<FP64>(), s>>>(
       a, nw, dyn_unit_log2(a.g.ntet, a.q.hi - a.q.lo, FP64));
   if (!FP64 && !IMO) k_dyn_fallback<<<rows * DynShape<FP64>::warps, 128, 0, s>>>(db, rows * DynShape<FP64>::warps, rows, a.tau, a.counters);
@@ -1394,7 +1406,7 @@ cudaError_t launch_dynamic(const DynArgs &a, int fp64, int im_only, const double
                            double scale, const double *dos, int ndos, double *re, double *im, cudaStream_t s) {
   const DynBufs &db = a.db;
   if (nw > kNWPass || nw <= 0 || nblocks <= 0) return cudaErrorInvalidValue;
-  if (!fp64 && (!a.Eklo || !a.Ekqlo)) return cudaErrorInvalidValue;
+  if (!fp64 && (!a.Eklo || !a.Ekqlo || !db.erange)) return cudaErrorInvalidValue;
   if (!db.box_tab || !db.box_part || !db.box_tot || !db.fb || !db.fbn || !db.fx || !db.ctr || !db.partR || !db.partI)
     return cudaErrorInvalidValue;
   if (fp64)

@@ -261,6 +261,21 @@ __global__ void __launch_bounds__(kThreads) k_bands(const __grid_constant__ Band
   }
 }
 
+// ---------------------------------------------------------------- energy range
+// largest finite |E - eF| of bands [lo, hi), as the bits of a double (out: 0 on entry)
+__global__ void __launch_bounds__(kThreads) k_energy_range(const double *__restrict__ E, long long nc, int nb, int lo,
+                                                           int w, double ef, unsigned long long *__restrict__ out) {
+  double m = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * w; i += (long long)gridDim.x * blockDim.x) {
+    const long long c = i / w;
+    const double x = fabs(E[c * nb + lo + (int)(i - c * w)] - ef);
+    if (x < (double)INFINITY) m = fmax(m, x);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(grid::kFull, m, o));
+  if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+}
+
 // ---------------------------------------------------------------- Gamma DOS term
 __global__ void __launch_bounds__(kThreads) k_dos(Grid g, Tet tet, const double *__restrict__ E, int lo,
                                                    int hi, double *__restrict__ partial,
@@ -369,6 +384,15 @@ cudaError_t launch_bands(const BandArgs &a, int nq, long long nc, int nb, double
   const long long nblk = (nc + per - 1) / per;
   const int cap = device_sms() * 8;
   k_bands<<<dim3((unsigned)(nblk < cap ? nblk : cap), (unsigned)nq), kThreads, 0, s>>>(a, nc, nb, ef);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_energy_range(const double *E, long long nc, int nb, int lo, int hi, double ef, unsigned long long *out,
+                                cudaStream_t s) {
+  const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  const long long nblk = (nc * (hi - lo) + kThreads - 1) / kThreads, cap = device_sms() * 8;
+  k_energy_range<<<(unsigned)(nblk < cap ? nblk : cap), kThreads, 0, s>>>(E, nc, nb, lo, hi - lo, ef, out);
   return cudaGetLastError();
 }
 
