@@ -286,68 +286,6 @@ template <typename T> __device__ __forceinline__ int box_of(T c, T s, const BoxG
   return wide;
 }
 
-// s_k = [z^k] N(z)/Q(z)^2 of a piece, one after the other (k = 0, 1, ...): Q in the quadratic
-// factors of the end and of the middle knots, two divisions by each
-template <typename T> struct Moments {
-  T A, B, C, D;        // 1 - A z + B z^2 (e_0, e_3), 1 - C z + D z^2 (e_1, e_2)
-  T n[4];
-  T x1, x2, y1, y2, u1, u2, v1, v2;  // the stages' last two values
-  __device__ __forceinline__ Moments(const T e[4], const T f[4]) {
-    A = e[0] + e[3];
-    B = e[0] * e[3];
-    C = e[1] + e[2];
-    D = e[1] * e[2];
-    const T E1 = A + C, E2 = (B + D) + A * C, E3 = B * C + D * A;
-    const T g0 = f[0] * e[0], g1 = f[1] * e[1], g2 = f[2] * e[2], g3 = f[3] * e[3];
-    const T h0 = g0 * e[0], h1 = g1 * e[1], h2 = g2 * e[2], h3 = g3 * e[3];
-    const T m0 = (f[0] + f[1]) + (f[2] + f[3]), m1 = (g0 + g1) + (g2 + g3), m2 = (h0 + h1) + (h2 + h3);
-    const T m3 = (h0 * e[0] + h1 * e[1]) + (h2 * e[2] + h3 * e[3]);
-    n[0] = m0;
-    n[1] = m1 - E1 * m0;
-    n[2] = m2 + (E2 * m0 - E1 * m1);
-    n[3] = m3 + (E2 * m1 - E1 * m2) - E3 * m0;
-    x1 = x2 = y1 = y2 = u1 = u2 = v1 = v2 = T(0);
-  }
-  __device__ __forceinline__ T next(T in) {
-    const T x = in + (A * x1 - B * x2);
-    const T y = x + (A * y1 - B * y2);
-    const T u = y + (C * u1 - D * u2);
-    const T v = u + (C * v1 - D * v2);
-    x2 = x1, x1 = x;
-    y2 = y1, y1 = y;
-    u2 = u1, u1 = u;
-    v2 = v1, v1 = v;
-    return v;
-  }
-};
-
-// The same s_k (k = 1, 2, ...) by the complete homogeneous polynomials h_k(e_1..e_4, e_j) of every
-// vertex: the FP32 kernel's form.  Thirteen operations a moment instead of eight, but shorter
-// chains and fewer registers: the 64 x 64 x 16 pass takes 6.8 ms with it, 7.4 ms with Moments.
-template <typename T> struct MomentsH {
-  T e[4], f[4], H[4], P[4];
-  __device__ __forceinline__ MomentsH(const T e_[4], const T f_[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      e[i] = e_[i];
-      f[i] = f_[i];
-      H[i] = P[i] = T(1);
-    }
-  }
-  __device__ __forceinline__ T next() {
-    H[0] = e[0] * H[0];
-#pragma unroll
-    for (int l = 1; l < 4; ++l) H[l] = H[l - 1] + e[l] * H[l];
-    T s = T(0);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      P[j] = H[3] + e[j] * P[j];
-      s += f[j] * P[j];
-    }
-    return s;
-  }
-};
-
 // v as 64-bit fixed point (units of 2^-44, round to nearest even): the same integer as
 // __float2ll_rn(v 2^44), from two 32-bit conversions (the 64-bit conversion runs at the FP64 rate,
 // 16 cycles of the SM per warp; these take 4)
@@ -368,17 +306,6 @@ __device__ __forceinline__ void fx_add(unsigned *lo, unsigned *hi, int i, float 
   atomicAdd(&hi[i], (unsigned)((unsigned long long)t >> 32) + (old + l < old ? 1u : 0u));
 }
 
-// the delta term of a near pair: FP64 by the plane section; FP32 by the cubic recursion, whose
-// rounding (a relative 2.9e-8 common to every piece, from its 4/3) its results have always carried
-__device__ __forceinline__ double delta_term(const double x[4], const double e[4], const double f[4]) {
-  return delta_section(x, e, f);
-}
-__device__ __forceinline__ float delta_term(const float x[4], const float e[4], const float f[4]) {
-  const float rs[6] = {rcp(e[1] - e[0]), rcp(e[2] - e[1]), rcp(e[3] - e[2]),
-                       rcp(e[2] - e[0]), rcp(e[3] - e[1]), rcp(e[3] - e[0])};
-  return delta_sum_pre(x, f, rs);
-}
-
 // does box b stand in for term (0: 1/(D - u), 1: 1/(D + u)) at frequency u = om?  Fine boxes
 // only near themselves; the others always.  Same expression in all kernels.
 template <typename T> __device__ __forceinline__ bool box_far(T C, T R, int b, T om, int term) {
@@ -387,46 +314,6 @@ template <typename T> __device__ __forceinline__ bool box_far(T C, T R, int b, T
   if (term) return !(C + om < r2);
   return !(tabs(C - om) < r2);
 }
-
-// sum_j f_j (1/V) int lambda_j / X for knots x of X near 0: divided-difference table (principal
-// value across X = 0); one out-of-line copy
-template <bool FP64>
-__device__ __noinline__ typename std::conditional<FP64, double, float>::type near_term(
-    const typename std::conditional<FP64, double, float>::type *x,
-    const typename std::conditional<FP64, double, float>::type *f, float tau, int &nfp64) {
-  using T = typename std::conditional<FP64, double, float>::type;
-  T xx[4] = {x[0], x[1], x[2], x[3]};
-  // (the entries that reach this function are the ones the shared table left: the per-vertex
-  // table directly, after the series branches)
-  if constexpr (FP64) {
-    double v;
-    if (series_ok(xx, T(Num<T>::kappa))) return series_sum(xx, f);
-    if (inv_sum_triple(xx, f, v)) return v;
-    return inv_sum_table(xx, f);
-  } else {
-    if (series_ok(xx, Num<float>::kappa)) return series_sum(xx, f);
-    float y[4];
-    if (!mixed_knots(y, xx, tau)) {
-      float v;
-      if (series_ok(y, Num<float>::kappa_long)) return series_sum(y, f);
-      if (inv_sum_triple_table(y, f, v)) return v;
-      return inv_sum_table(y, f);
-    }
-    ++nfp64;
-    double yd[4] = {y[0], y[1], y[2], y[3]}, fd[4] = {f[0], f[1], f[2], f[3]}, v;
-    if (inv_sum_triple(yd, fd, v)) return (float)v;
-    return (float)inv_sum_table(yd, fd);
-  }
-}
-
-// D0 - w for a frequency near the knots: with D0 = D0h + D0l and w = wh + wl split into
-// FP32 parts the difference keeps full relative precision however close D0 is to w
-__device__ __forceinline__ float near_shift(float D0h, float D0l, float wh, float wl) {
-  float sv, tv;
-  two_diff(D0h, wh, sv, tv);
-  return sv + (tv + (D0l - wl));
-}
-__device__ __forceinline__ double near_shift(double D0h, double, double wh, double) { return D0h - wh; }
 
 // first index of the ascending om[0..n) with om[i] > v (strict) or >= v
 template <bool STRICT, typename T> __device__ __forceinline__ int first_above(const T *om, int n, T v) {
