@@ -809,7 +809,7 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
 #pragma unroll
     for (int i = 0; i < 4; ++i) f[i] = A.cma ? T(1) : pw[(long long)ck[i] * w * w];
   };
-  // FP32: the vertices in ascending order of the key, as cut_piece takes them
+  // FP32: the vertices in ascending order of the key (chi0_math.cuh, recipes)
   auto sort_key = [&](T key[4], T x[4], T y[4]) {
     if constexpr (!FP64) {
       auto sw = [&](int i, int j) {

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(NT, MINB) k_static(const __grid_constant__ Sta
     };
     // the second cut's key, -b, at a vertex of key a (0 on the first cut's plane)
     auto key_b = [&](T a, T D) { return FP64 ? -fma(D, S, a) : -(a + D); };
-    // FP32: the vertices in ascending order of the key, as cut_piece takes them
+    // FP32: the vertices in ascending order of the key (chi0_math.cuh, recipes)
     auto sort_key = [&](T key[4], T x[4], T y[4]) {
       if constexpr (!FP64) {
         auto sw = [&](int i, int j) {
