@@ -521,7 +521,8 @@ __global__ void __launch_bounds__(DynShape<FP64>::threads, DynShape<FP64>::minb)
 #pragma unroll
           for (int i = 0; i < 4; ++i) ff[i] = s_qf[wib][sl][i];
           if constexpr (FP64) {  // about the midpoint, offsets in units of the half-width
-            const T ri = half > T(0) ? rcp_nr(half) : T(0), mid = (e0 + e3) * T(0.5), vr = s_qv[wib][sl][0];
+            // (a half-width below 2^-1000 counts as flat: it has no finite reciprocal below 2^-1022)
+            const T ri = half > T(1e-300) ? rcp_nr(half) : T(0), mid = (e0 + e3) * T(0.5), vr = s_qv[wib][sl][0];
             T e[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) e[i] = (s_qe[wib][sl][i] - mid) * ri;
