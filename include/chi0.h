@@ -268,8 +268,9 @@ int chi0_static_pairs(chi0_plan_t *plan, const chi0_q_t *q, int nq, double *chi,
  * Re is the principal value of Eq. 1; Im is Eq. 2 for w > 0, 0 at w = 0, and odd
  * (Eq. 3) for w < 0.  Frequencies in any order; one that is not finite leaves the others alone
  * (a NaN gives Re = NaN, Im = 0; an infinite one 0).  Energies in any unit: the mixed form's
- * fixed-point sums are scaled by W, the largest |E - eF| of the plan's window, and hold
- * W |chi0| up to 2^15.  Errors as chi0_static, plus CHI0_EINVAL for nw <= 0. */
+ * fixed-point sums are scaled by the bands' largest |E - eF|, W_m, and hold W |chi0| up to 2^15,
+ * W being the largest W_m of the q's window where that is below 1/16, the smallest where that is
+ * above 256; in between |chi0| up to 2^19.  Errors as chi0_static, plus CHI0_EINVAL for nw <= 0. */
 int chi0_dynamic(chi0_plan_t *plan, const chi0_q_t *q, int nq, const double *omega, int nw,
                  double *re, double *im);
 

@@ -67,7 +67,7 @@ struct chi0_plan {
   void *fb_d = nullptr;                       // their counts,
   unsigned long long *fx_d = nullptr;         // per-CTA fixed-point sums (FP32) and the
   unsigned long long *ctr_d = nullptr;        // unit counter
-  unsigned long long *erange_d = nullptr;     // largest |E - eF| of the window (mixed precision)
+  unsigned long long *erange_d = nullptr;     // largest |E - eF| of every band (mixed precision)
   unsigned long long *pairs_fx_d = nullptr;   // band-pair output: fixed-point totals of one q,
   size_t pairs_fx_cap = 0;                    // and the FP64 results of the call (host outputs)
   double *pairs_out_d = nullptr;
@@ -200,7 +200,7 @@ extern "C" void chi0_destroy(chi0_plan_t *p) {
 // band bounds per corner: four arrays of nc from base on
 static BandBounds bounds_at(short *base, long long nc) { return BandBounds{base, base + nc, base + 2 * nc, base + 3 * nc}; }
 
-// bounds, FP32 energies and energy range of the plan's own eigen-data
+// bounds, FP32 energies and energy ranges of the plan's own eigen-data
 static cudaError_t plan_bands(chi0_plan_t *p) {
   const Grid &g = p->g;
   BandArgs a{};
@@ -210,7 +210,7 @@ static cudaError_t plan_bands(chi0_plan_t *p) {
   a.E32lo = p->E32_d ? p->E32_d + (size_t)g.nc * g.nb : nullptr;
   const cudaError_t e = launch_bands(a, 1, g.nc, g.nb, g.ef, p->stream);
   if (e != cudaSuccess || !p->erange_d) return e;
-  return launch_energy_range(p->E_d, g.nc, g.nb, p->win.lo, p->win.hi, g.ef, p->erange_d, p->stream);
+  return launch_energy_range(p->E_d, g.nc, g.nb, g.ef, p->erange_d, p->stream);
 }
 
 static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t *tt, chi0_band_window_t win,
@@ -332,7 +332,7 @@ static int build_plan(chi0_plan_t *p, const chi0_kgrid_t *kg, const chi0_tetra_t
   if (op.precision == CHI0_PREC_MIXED) {
     CK(p, cudaMalloc(&p->E32_d, 2 * sizeof(float) * ncb));
     CK(p, cudaMalloc(&p->Eq32_d, G * 2 * sizeof(float) * ncb));
-    CK(p, cudaMalloc(&p->erange_d, sizeof(unsigned long long)));
+    CK(p, cudaMalloc(&p->erange_d, sizeof(unsigned long long) * g.nb));
   }
   CK(p, plan_bands(p));
   if (op.precision == CHI0_PREC_MIXED && !op.cma && p->dtype == CHI0_C128) {

@@ -82,16 +82,18 @@ using grid::tet_corners;
 constexpr int kNWPass = 256;   // frequencies per dynamic pass
 // FP32 kernel: sums in 64-bit fixed point, units of 2^-44 (exact and order-independent; one rounding of
 // 2^-45 per term).  Re and Im are sums of v f / energy, so the range (2^19) and the rounding are held
-// against the energies: W being the largest |E - eF| of the plan's window, the terms carry a power of
-// two S that is 1 for 2^-4 <= W < 2^8 and keeps S / W in [2^3, 2^4] below, in [2^-8, 2^-7] above.  So
-// W |sum| may reach 2^15 at least (80 bands: some 10 with |M|^2, a few 1000 without), and a sum of 10^9
-// terms rounds by 5e-10 / S, at most 1.3e-7 / W.
+// against the energies: the terms carry a power of two S.  With W_m the largest |E - eF| of band m, S is
+// below 1 where every band of the q's window is narrow (the largest W_m < 2^-4: S / W_m in [2^3, 2^4]),
+// above 1 where every band is wide (the smallest W_m >= 2^8: S / W_m in [2^-8, 2^-7]), and else 1: core
+// levels or placeholder bands at 1e10 do not move the scale of the others.  So W |sum| may reach 2^15 at
+// least (80 bands: some 10 with |M|^2, a few 1000 without), W being that largest or smallest W_m, and a
+// sum of 10^9 terms rounds by 5e-10 / S, at most 1.3e-7 / W.
 constexpr double kFxUnit = 1.0 / 17592186044416.0;
-__device__ __forceinline__ float fx_scale(unsigned long long bits) {
-  const double W = __longlong_as_double((long long)bits);
-  if (!(W > 0.0)) return 1.0f;
-  const int e = ilogb(W);  // 2^e <= W < 2^(e + 1)
-  return (float)exp2((double)max(min(e < -4 ? e + 4 : (e > 7 ? e - 7 : 0), 100), -100));
+// (least, most: high words of the W_m as doubles; most = 0: none)
+__device__ __forceinline__ float fx_scale(unsigned least, unsigned most) {
+  if (most == 0u) return 1.0f;
+  const int e0 = (int)(least >> 20) - 1023, e1 = (int)(most >> 20) - 1023;  // 2^e <= W < 2^(e + 1)
+  return ldexpf(1.0f, max(min(e1 < -4 ? e1 + 4 : (e0 > 7 ? e0 - 7 : 0), 100), -100));
 }
 constexpr int kQC = 64;        // queue of final tetrahedra that evaluate frequencies themselves
 constexpr int kCodes = 128;    // listed pieces of cut items per warp: < 32 left over + 3 x 32
@@ -193,8 +195,10 @@ template <typename T> __device__ __forceinline__ void kadd_t(T &sum, T &comp, T 
 // searches, the boxes or u_max; k_dyn_out gives them their values.
 template <typename T>
 __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict__ omega, int nw, int boxes,
-                                                       const unsigned long long *__restrict__ erange, BoxTab<T> *tab) {
+                                                       const unsigned long long *__restrict__ erange, int lo, int hi,
+                                                       BoxTab<T> *tab) {
   __shared__ double red[8];
+  __shared__ unsigned rlo[8], rhi[8];
   __shared__ int cnt[8];
   __shared__ unsigned long long key[kNWPass];
   const int i = threadIdx.x;
@@ -205,8 +209,20 @@ __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict_
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) u = fmax(u, __shfl_xor_sync(kFull, u, o));
   const unsigned oks = __ballot_sync(kFull, ok);
+  unsigned least = ~0u, most = 0u;  // of the bands' W_m (a band at eF throughout, or not finite, has none)
+  if constexpr (sizeof(T) == 4) {
+    for (int m = lo + i; m < hi; m += kNWPass) {
+      const unsigned W = (unsigned)(erange[m] >> 32);
+      if (W) least = min(least, W);
+      most = max(most, W);
+    }
+    least = __reduce_min_sync(kFull, least);
+    most = __reduce_max_sync(kFull, most);
+  }
   if ((i & 31) == 0) {
     red[i >> 5] = u;
+    rlo[i >> 5] = least;
+    rhi[i >> 5] = most;
     cnt[i >> 5] = __popc(oks);
   }
   __syncthreads();
@@ -231,7 +247,11 @@ __global__ void __launch_bounds__(kNWPass) k_box_setup(const double *__restrict_
     tab->umax = um;
     tab->on = on;
     tab->nv = nv;
-    tab->S = sizeof(T) == 4 ? (T)fx_scale(*erange) : T(1);
+    for (int k = 1; k < kNWPass / 32; ++k) {
+      least = min(least, rlo[k]);
+      most = max(most, rhi[k]);
+    }
+    tab->S = sizeof(T) == 4 ? (T)fx_scale(least, most) : T(1);
     double lo = (double)x0;
     for (int b = 0; b <= kBoxG; ++b) {
       tab->lowG[b] = (T)lo;
@@ -1262,7 +1282,7 @@ cudaError_t launch_weights(const DynArgs &a, const double *omega, int nw, int nb
   if (!FP64) e = cudaMemsetAsync(db.ctr, 0, sizeof(unsigned long long), s);
   else if (!IMO) e = cudaMemsetAsync(db.box_part, 0, sizeof(double) * (size_t)rows * NS, s);
   if (e != cudaSuccess) return e;
-  k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, db.erange, (BoxTab<T> *)db.box_tab);
+  k_box_setup<T><<<1, kNWPass, 0, s>>>(omega, nw, IMO ? 0 : 1, db.erange, a.q.lo, a.q.hi, (BoxTab<T> *)db.box_tab);
   k_dynamic<FP64, IMO><<<nblocks, DynShape<FP64>::threads, IMO ? 0 : dyn_smem<FP64>(), s>>>(
       a, nw, dyn_unit_log2(a.g.ntet, a.q.hi - a.q.lo, FP64));
   if (!FP64 && !IMO) k_dyn_fallback<<<rows * DynShape<FP64>::warps, 128, 0, s>>>(db, rows * DynShape<FP64>::warps, rows, a.tau, a.counters);

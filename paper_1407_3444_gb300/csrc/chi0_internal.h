@@ -88,8 +88,8 @@ struct BandArgs {
   size_t stride_c, stride_e;
 };
 cudaError_t launch_bands(const BandArgs &a, int nq, long long nc, int nb, double ef, cudaStream_t s);
-// *out = bits of the largest finite |E - eF| of bands [lo, hi) (the scale of the FP32 dynamic weights' sums)
-cudaError_t launch_energy_range(const double *E, long long nc, int nb, int lo, int hi, double ef, unsigned long long *out,
+// out[band] = bits of the band's largest finite |E - eF| (they give the scale of the FP32 dynamic weights' sums)
+cudaError_t launch_energy_range(const double *E, long long nc, int nb, double ef, unsigned long long *out,
                                 cudaStream_t s);
 
 // one q of a static launch: k+q energies (FP64 absolute, or FP32 relative to eF) and their band
@@ -138,7 +138,7 @@ struct DynBufs {
   int *fbn;                 // FP32 kernel: [warps of the launch] entries left at its end
   unsigned long long *fx;   // FP32 kernel: [CTAs of the launch][2][dynamic_max_nw()] fixed-point sums
   unsigned long long *ctr;  // FP32 kernel: unit counter (reset by the launch)
-  const unsigned long long *erange;  // FP32 kernel: largest |E - eF| of the plan's window (bits of a double)
+  const unsigned long long *erange;  // FP32 kernel: largest |E - eF| of every band (bits of doubles)
 };
 // one q of a dynamic launch: energies FP64 absolute, or FP32 relative to eF (hi and lo parts), their
 // band bounds, |M|^2

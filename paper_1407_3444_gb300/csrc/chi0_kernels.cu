@@ -262,18 +262,28 @@ __global__ void __launch_bounds__(kThreads) k_bands(const __grid_constant__ Band
 }
 
 // ---------------------------------------------------------------- energy range
-// largest finite |E - eF| of bands [lo, hi), as the bits of a double (out: 0 on entry)
-__global__ void __launch_bounds__(kThreads) k_energy_range(const double *__restrict__ E, long long nc, int nb, int lo,
-                                                           int w, double ef, unsigned long long *__restrict__ out) {
-  double m = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc * w; i += (long long)gridDim.x * blockDim.x) {
-    const long long c = i / w;
-    const double x = fabs(E[c * nb + lo + (int)(i - c * w)] - ef);
-    if (x < (double)INFINITY) m = fmax(m, x);
+// largest finite |E - eF| of every band over the corners, as the bits of a double (out: 0 on entry).
+// A thread stays with one band, kThreads / (bands of the tile) corners a block at a time: the loads of
+// a step are consecutive, and a block adds one atomic a band.
+__global__ void __launch_bounds__(kThreads) k_energy_range(const double *__restrict__ E, long long nc, int nb, double ef,
+                                                           unsigned long long *__restrict__ out) {
+  __shared__ unsigned long long s_max[kThreads];
+  for (int b0 = 0; b0 < nb; b0 += kThreads) {
+    const int wt = min(nb - b0, kThreads), rows = kThreads / wt, r = threadIdx.x / wt, b = threadIdx.x - r * wt;
+    double m = 0.0;
+    if (r < rows)
+      for (long long c = (long long)blockIdx.x * rows + r; c < nc; c += (long long)gridDim.x * rows) {
+        const double x = fabs(E[c * nb + b0 + b] - ef);
+        if (x < (double)INFINITY) m = fmax(m, x);
+      }
+    s_max[threadIdx.x] = (unsigned long long)__double_as_longlong(m);
+    __syncthreads();
+    if (r == 0) {
+      for (int k = 1; k < rows; ++k) m = fmax(m, __longlong_as_double((long long)s_max[k * wt + b]));
+      if (m > 0.0) atomicMax(out + b0 + b, (unsigned long long)__double_as_longlong(m));
+    }
+    __syncthreads();
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(grid::kFull, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
 // ---------------------------------------------------------------- Gamma DOS term
@@ -387,12 +397,12 @@ cudaError_t launch_bands(const BandArgs &a, int nq, long long nc, int nb, double
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_range(const double *E, long long nc, int nb, int lo, int hi, double ef, unsigned long long *out,
+cudaError_t launch_energy_range(const double *E, long long nc, int nb, double ef, unsigned long long *out,
                                 cudaStream_t s) {
-  const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
+  const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long) * nb, s);
   if (e != cudaSuccess) return e;
-  const long long nblk = (nc * (hi - lo) + kThreads - 1) / kThreads, cap = device_sms() * 8;
-  k_energy_range<<<(unsigned)(nblk < cap ? nblk : cap), kThreads, 0, s>>>(E, nc, nb, lo, hi - lo, ef, out);
+  const long long nblk = (nc * nb + kThreads - 1) / kThreads, cap = device_sms() * 8;
+  k_energy_range<<<(unsigned)(nblk < cap ? nblk : cap), kThreads, 0, s>>>(E, nc, nb, ef, out);
   return cudaGetLastError();
 }
 
