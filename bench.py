@@ -280,7 +280,8 @@ def arithmetic_peaks(chi0):
 
 # Executed FP32 operations (FFMA counted twice, FADD, FMUL) per final tetrahedron of the mixed
 # static weight kernel on the Cr-like 48^3 workload (ncu instruction counters of k_static, three q
-# points).  DRAM bytes per final tetrahedron are not reported: 3.2 B, the |M|^2 table once.
+# points).  DRAM bytes per final tetrahedron: None in the JSON line; they are the |M|^2 table read once
+# (3.2 B on this mesh), which follows from the mesh and the window, not from the pieces.
 FLOPS_PER_PIECE_MIXED = 153.0
 TRAFFIC_PER_PIECE_MIXED = None
 # The same for the dynamic weight kernels per final tetrahedron over one pass of 256 frequencies
@@ -290,7 +291,7 @@ TRAFFIC_PER_PIECE_MIXED = None
 # DRAM bytes: not taken from the sample (its scattered tetrahedra defeat the caches that the
 # whole mesh uses), and on whole meshes they fall per final tetrahedron as the mesh grows, so no
 # per-unit figure scales to the 72^3 launch: None until counted there.
-FLOPS_PER_PIECE_DYN32 = 2780.7
+FLOPS_PER_PIECE_DYN32 = 2776.5
 FLOPS_PER_PIECE_DYN64 = None
 TRAFFIC_PER_PIECE_DYN32 = None
 

@@ -315,7 +315,7 @@ int chi0_interpolate_kq(chi0_plan_t *plan, const double *qfrac, double *e_kq, vo
  *     CTAs per SM of the dynamic weight kernel;
  *   - corners per MMA round of the tensor-core overlap (CHI0_OVL_BF16X3, BF16X6 or TF32 only;
  *     1, 2, 3, 4, 8, ... up to the most that fit one tile).
- * Every candidate computes the same chi0 up to rounding: the k-batch partials and their
+ * Every candidate computes the same chi0 up to rounding: the unit partials and their
  * summation order do not depend on the grid, and the corner grouping only changes how the
  * tensor-core FP32 accumulators are split.  Each timed call writes its results to chi / re,
  * im like chi0_static / chi0_dynamic.  *result: the chosen shape, the candidates timed, the

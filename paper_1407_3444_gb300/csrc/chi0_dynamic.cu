@@ -59,7 +59,7 @@
 // range) at a time, 64-bit float conversions and atomics, batches of 32 tetrahedra, the per-vertex
 // table for every left entry) and now: 64 x 64 x 16 mesh, 10 bands FP32 10.5 -> 3.8 ms (k_dyn_fallback
 // 0.35 of it), 32^3, 80 bands FP32 836 -> 395 ms; 16 x 16 x 8, 10 bands, 128 frequencies FP64
-// 58-100 -> 6.2 ms; Im alone, 32^3, 12 bands FP32 3.3 -> 0.77 ms.
+// 58-100 -> 6.2 ms; Im alone, 32^3, 12 bands FP32 3.3 -> 0.70 ms.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

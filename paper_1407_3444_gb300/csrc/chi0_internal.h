@@ -120,7 +120,7 @@ struct StaticArgs {
 cudaError_t launch_static(StaticArgs &a, int fp64, int nblocks, cudaStream_t s, int variant = 0);
 cudaError_t launch_static_reduce(const StaticArgs &a, double scale, int ndos, double *out, cudaStream_t s);
 int static_persistent_blocks(int fp64);
-long long static_batches(long long ntet);  // runs of 32 tetrahedra (the dynamic weights' batches)
+long long static_batches(long long ntet);  // runs of 32 tetrahedra (the no-allocation entry point sizes its array by them)
 // partials of one q with a window of w bands (never more with a narrower one)
 long long static_units(long long ntet, int w);
 

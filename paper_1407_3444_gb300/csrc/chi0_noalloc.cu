@@ -33,9 +33,9 @@ static __device__ __align__(256) unsigned char g_chi0_scratch[CHI0_NOALLOC_SCRAT
 namespace {
 
 constexpr int kMaxDevices = 64;
-// the array's work region per batch of 32 tetrahedra: 640 (FP32) or 1280 (FP64) bytes, of which
-// the unit partials (at most 64 per batch) and the band bounds beyond occ and emp (16 per
-// corner, at most 8 corners per cube) take less than half
+// the array's work region per run of 32 tetrahedra: 640 (FP32) or 1280 (FP64) bytes, of which
+// the unit partials (at most eight a run, 64 bytes) and the band bounds beyond occ and emp (8 bytes a
+// corner) take two fifths at most (FP32, an open 1 x 1 x 5 mesh)
 constexpr size_t kNoallocWork32 = 640, kNoallocWork64 = 1280;
 unsigned char *g_scratch_ptr[kMaxDevices] = {nullptr};
 std::mutex g_scratch_mu;
@@ -101,6 +101,7 @@ Layout layout(const Grid &g, int w, int fp64, int cma, int dtype) {
   L.next = take(sizeof(int));
   L.counters = take(4 * sizeof(unsigned long long));
   L.work = take(mul_sat(fp64 ? kNoallocWork64 : kNoallocWork32, nbatch));
+  // not used: with these two the same meshes fit the array as in every version so far
   take(mul_sat(sizeof(int), nbatch));
   take(mul_sat(sizeof(double), mul_sat(2, nbatch)));
   L.dos = take(mul_sat(sizeof(double), (size_t)static_blocks()));
